@@ -2,28 +2,31 @@
 // map_offset, Section 3.5.1 valid multiplications), for all output tiles of
 // all instances of a table at once.
 //
-// Stream order (after one memset that clears the accumulators):
-//   prep      FP64 norm maps -> FP32 mantissa/exponent "screen" forms (B transposed
-//             so a tile's k-run is contiguous) and per-CTA sums of squared norms;
-//             the last CTA of each instance forms ||A||_F, ||B||_F.
-//   count     each CTA owns 32 tiles of one instance (consecutive in a grouped
-//             raster enumeration: bands of 8 block rows, column by column), one
-//             warp per tile at a time: lanes test k = lane, lane+32, ...; the
-//             ballot words are kept as the tile's survivor bitmask; skipped
-//             products are summed for the bounds; split modes bin the surviving
-//             products by binade; per-CTA totals and per-CTA counts of the
-//             longest-first buckets (floor(log2 survivors) + 1).
-//   finalize  one CTA per instance: one vector scan over its CTAs' totals gives
-//             each CTA's first k_idx slot, non-empty rank and bucket slots;
-//             statistics and the split-flag binade; the last of these CTAs lays
-//             out the batch-wide buckets (largest first) and each instance's
-//             place in them.
-//   fill      same partition: first slots from the CTA base plus a warp scan;
-//             the bitmask words are expanded (ballot ranks place the surviving
-//             k, increasing, at tile_beg[t] + rank); each non-empty tile takes
-//             its slot in the longest-first order (bucket base + CTA base +
-//             rank among the CTA's tiles of the bucket, enumeration order), each
-//             empty tile its slot after all non-empty ones.
+// Output tiles are enumerated in bands of 8 block rows, column by column inside
+// a band; a unit is up to 32 consecutive tiles of one band (8 rows x 4 columns
+// in a full band).  Stream order:
+//   prep   (only when some instance needs ||A||_F ||B||_F before its products
+//          are counted, or the table has more than kScanUnits units) per-CTA
+//          sums of squared norms; clears the accumulators.
+//   count  one CTA per unit: the unit's block rows of A and block columns of B
+//          are turned into FP32 mantissa/exponent "screen" forms in shared
+//          memory; a lane owns a tile, the warps share its k in 32-wide words
+//          (the tile's survivor bitmask, built in a register: no ballots, no
+//          cross-lane reductions per tile); skipped products are summed for
+//          the bounds; split modes bin the surviving products by binade;
+//          per-unit totals and longest-first bucket counts
+//          (floor(log2 survivors) + 1).
+//   fill   every CTA derives the first slots of its units itself, from the
+//          totals of all units before them (no separate scan kernel); the
+//          bitmask words are expanded into k lists (increasing, at
+//          tile_beg[t] + rank); each non-empty tile takes its slot in the
+//          longest-first order (bucket start + earlier units + rank, in
+//          enumeration order inside a bucket), each empty tile its slot after
+//          all non-empty ones; the blocks some surviving triple uses are
+//          listed once each, 32 of them per atomic.
+// Per-instance statistics come from a fill CTA of their own; in split modes every
+// fill CTA forms the flag binade of its units' instances.
+#include <algorithm>
 #include <cstddef>
 #include <cstring>
 #include <vector>
@@ -51,50 +54,103 @@ TauScreen make_tau_screen(double tau) {
 
 namespace {
 
-constexpr int kWarpsPerCta = 8;
-constexpr int kTilesPerCta = 32;   // count and fill: 8 warps x 4 tiles
-constexpr int kTileRounds = kTilesPerCta / kWarpsPerCta;
 constexpr int kPrepThreads = 256;
-constexpr int kFinThreads = 512;
-constexpr int kGroupRows = 8;      // block rows per band of the tile enumeration
-static_assert(kOrderKeys <= kMaxBd + 2 && kOrderKeys <= 32, "order buckets");
-static_assert(kTilesPerCta % kGroupRows == 0, "a CTA of a full band covers whole columns");
+constexpr int kCountWarps = 4;
+constexpr int kCountThreads = kCountWarps * 32;
+constexpr int kFillWarps = 8;
+constexpr int kFillThreads = kFillWarps * 32;
+constexpr int kUnitWarps = 4;        // fill: warps sharing one unit's tiles
+constexpr int kStatWarps = 4;        // parts of an instance's sums over its units
+constexpr int kHistWarps = 8;
+constexpr int kHistTiles = 32;       // histogram: tiles per CTA
+constexpr int kBandRows = 8;         // block rows per band of the tile enumeration
+// Tables of at most kScanUnits units: a fill CTA reads every unit's totals (64
+// bytes each).  Larger ones: groups of units, whose totals the count kernel
+// adds up with atomics, so a fill CTA reads the groups and its own group's units.
+constexpr int kScanUnits = 1024;
+static_assert(kOrderKeys <= 12, "order buckets fit a unit's totals");
 
-// Output tile (i, j) at enumeration position `pos` of an instance: bands of
-// kGroupRows block rows, column by column inside a band, so that tiles close
-// in the enumeration (and so in the multiply's order, which keeps it inside
-// a bucket) share block rows of A and block columns of B in L2.
-__device__ __forceinline__ void tile_at(int64_t pos64, int bm, int bn, int& i, int& j) {
-  const int pos = (int)pos64;              // bm * bn <= 2^22
-  const int band_tiles = kGroupRows * bn;
-  const int band = pos / band_tiles;
-  const int r0 = band * kGroupRows;
-  const int rows = min(kGroupRows, bm - r0);
-  const int w = pos - band * band_tiles;
-  j = w / rows;
-  i = r0 + (w - j * rows);
+// Slots of a unit's (or a group's) totals, kPartInts per unit.
+enum : int { kPartS = 0 /* survivors */, kPartNe = 12, kPartMax = 13 };   // 1 .. 11: buckets
+
+// Columns of a unit: 32 tiles, and at most 16 staged rows and columns.
+__host__ __device__ __forceinline__ int unit_cols(int bm) {
+  if (bm >= kBandRows) return 32 / kBandRows;
+  const int c = 32 / bm;
+  return c < 16 - bm ? c : 16 - bm;
+}
+
+struct Unit {
+  int r0, rows, j0, cols;   // block rows r0 .. r0 + rows - 1, columns j0 .. j0 + cols - 1
+};
+
+__device__ __forceinline__ Unit unit_at(const Inst& in, int lu) {
+  const int uc = unit_cols(in.bm);
+  const int per_band = (in.bn + uc - 1) / uc;
+  const int band = lu / per_band;
+  Unit u;
+  u.r0 = band * kBandRows;
+  u.rows = min(kBandRows, in.bm - u.r0);
+  u.j0 = (lu - band * per_band) * uc;
+  u.cols = min(uc, in.bn - u.j0);
+  return u;
+}
+
+__host__ __device__ __forceinline__ int units_of(const Inst& in) {
+  const int uc = unit_cols(in.bm);
+  return ((in.bm + kBandRows - 1) / kBandRows) * ((in.bn + uc - 1) / uc);
 }
 
 // Longest-first bucket of a survivor count c >= 1: floor(log2 c) + 1.  Near-
 // equal counts share a bucket, so the order keeps the enumeration's locality.
 __device__ __forceinline__ int order_key(int c) { return 32 - __clz(c); }
 
-// Exactly !(na * nb < tau) in FP64, decided in FP32 whenever that is safe.
-__device__ __forceinline__ bool survives(Screen a, Screen b, const double* nA_ptr,
-                                         const double* nB_ptr, const TauScreen& T) {
-  if (T.all) return true;
-  if (a.e == kNonFiniteExp || b.e == kNonFiniteExp) return true;  // Inf or NaN product
-  if (T.none) return false;
-  if (a.e == kZeroExp || b.e == kZeroExp) return false;           // 0 < tau
-  const int D = a.e + b.e - T.e;
-  if (D >= 3) return true;    // mA mB / mT >= 0.25 * 8 / 1 = 2
-  if (D <= -2) return false;  // mA mB / mT <= 1 / 0.5 * 2^-2 = 0.5
-  const float scale = D == -1 ? 0.5f : (D == 0 ? 1.0f : (D == 1 ? 2.0f : 4.0f));
-  const float q = __fmul_rn(__fmul_rn(a.m, b.m), scale);
-  if (q >= T.m_hi) return true;
-  if (q < T.m_lo) return false;
-  const double p = __dmul_rn(*nA_ptr, *nB_ptr);  // the exact FP64 decision
-  return !(p < T.tau);
+// Screens of the pair test.  Zero norms take the mantissa 0.5 and an exponent
+// below every sum that can survive, non-finite ones an exponent above every
+// sum that can be skipped (also against a zero: NaN products survive).
+constexpr int kTestZero = -100000, kTestNonFinite = 300000;
+
+// make_screen's mantissa (rounded to nearest even) and exponent from the bit
+// pattern: integer operations only, the FP64 pipe is narrow on this part.
+__device__ __forceinline__ Screen test_screen(double x) {
+  const int hi = __double2hiint(x);
+  const uint32_t lo = (uint32_t)__double2loint(x);
+  Screen s;
+  if (hi >= 0x00100000 && hi < 0x7ff00000) {   // positive and normal
+    const uint32_t m = (uint32_t)(hi & 0xfffff) << 3 | lo >> 29;
+    const uint32_t up = ((lo & 0x1fffffffu) + (m & 1u)) > 0x10000000u ? 1u : 0u;
+    s.m = __uint_as_float((126u << 23) + m + up);   // a carry gives 1.0
+    s.e = (hi >> 20) - 1022;
+    return s;
+  }
+  s = make_screen(x);
+  if (s.e == kZeroExp) {
+    s.m = 0.5f;
+    s.e = kTestZero;
+  } else if (s.e == kNonFiniteExp) {
+    s.e = kTestNonFinite;
+  }
+  return s;
+}
+
+// tau in the form the test uses: mantissa window and exponent.  tau = 0 puts the
+// exponent below every sum, tau = +Inf between the finite and the non-finite ones.
+struct TestTau {
+  float lo, hi;
+  int e;
+};
+
+__device__ __forceinline__ TestTau test_tau(const TauScreen& T) {
+  if (T.all) return TestTau{1.0f, 1.0f, -1000000};
+  if (T.none) return TestTau{1.0f, 1.0f, 150000};
+  return TestTau{T.m_lo, T.m_hi, T.e};
+}
+
+// q 2^D, D clamped to [-3, 4], for q = mA mB in [0.25, 1] and D = eA + eB - eT:
+// !(na * nb < tau) holds if it is >= T.hi and fails if it is < T.lo; between the
+// two (1 +- 2^-20) the FP64 product decides.
+__device__ __forceinline__ float screen_value(float q, int D) {
+  return __int_as_float(__float_as_int(q) + (min(max(D, -3), 4) * (1 << 23)));
 }
 
 // Extended-range FP32 sums (ExtSum, value m * 2^e): sums of relative products
@@ -130,36 +186,34 @@ __device__ __forceinline__ void ext_add(ExtSum& s, float q, int E) {
   }
 }
 
-// Per-lane sum of a tile's skipped products q 2^E (q = mA mB in [0.25, 1],
-// E = eA + eB), held as S 2^Emax with Emax the largest exponent seen so far;
-// terms more than 126 binades below Emax are dropped.  Zero products (m = 0)
-// add nothing.  A few FP32/integer operations per term and no branch in the
-// common case (E <= Emax).
+// Per-lane sum of a tile's skipped products q 2^D (q = mA mB in [0.25, 1]), held
+// as S 2^Emax with Emax the largest exponent seen so far; terms more than 126
+// binades below Emax are dropped.  A product that is not skipped comes with
+// D = kSkipNone, far below every reference.  Eight products share one rescaling
+// of the sum, without branches: along a decay matrix's rows every other
+// product raises the reference.
 struct SkipSum {
   float S;
   int Emax;
 };
 constexpr int kSkipNone = -(1 << 29);
+constexpr int kSkipStart = kSkipNone + 1000;   // the empty sum's reference
 
 // 2^k for -126 <= k <= 0, and 0 for k < -126.
 __device__ __forceinline__ float pow2f_or_zero(int k) {
   return __int_as_float(max(k + 127, 0) << 23);
 }
 
-__device__ __forceinline__ void skip_add(SkipSum& s, Screen a, Screen b) {
-  const int E = a.e + b.e;
-  const float q = __fmul_rn(a.m, b.m);
-  const int d = E - s.Emax;
-  if (d > 0) {   // a new largest exponent: rescale the running sum
-    s.S = __fmul_rn(s.S, pow2f_or_zero(-d));
-    s.Emax = E;
-  }
-  s.S = __fmaf_rn(q, pow2f_or_zero(min(d, 0)), s.S);
-}
-
-// The lane's sum as an ExtSum (value m 2^e).
-__device__ __forceinline__ ExtSum skip_ext(const SkipSum& s) {
-  return s.S > 0.0f ? ExtSum{s.S, s.Emax} : ExtSum{0.0f, 0};
+template <int N>
+__device__ __forceinline__ void skip_add(SkipSum& s, const float (&q)[N], const int (&D)[N]) {
+  int e = s.Emax;
+#pragma unroll
+  for (int z = 0; z < N; ++z) e = max(e, D[z]);
+  float S = __fmul_rn(s.S, pow2f_or_zero(max(s.Emax - e, -127)));
+#pragma unroll
+  for (int z = 0; z < N; ++z) S = __fmaf_rn(q[z], pow2f_or_zero(D[z] - e), S);
+  s.S = S;
+  s.Emax = e;
 }
 
 // Warp total of ExtSums in one pass: every lane rescales its sum to 2^-40 of
@@ -192,7 +246,13 @@ __device__ __forceinline__ ExtSum ext_warp_sum(ExtSum s) {
 }
 
 __device__ __forceinline__ double ext_value(ExtSum s) {
-  return s.m == 0.0f ? 0.0 : ldexp((double)s.m, s.e);
+  if (s.m == 0.0f) return 0.0;
+  const int e = fexp(s.m) + s.e;   // the value's binade: built from the bits when normal
+  if (e > -1022 && e < 1023) {
+    const uint32_t f = __float_as_uint(s.m) & 0x7fffffu;
+    return __hiloint2double((e + 1023) << 20 | (int)(f >> 3), (int)(f << 29));
+  }
+  return ldexp((double)s.m, s.e);
 }
 
 // floor(log2(fl(fl(na nb) * inv))) clamped to the flag bins: the binade of a relative norm
@@ -205,284 +265,494 @@ __device__ __forceinline__ int rel_bin(double p, double inv) {
   return b < kFlagBinMin ? kFlagBinMin : (b > 1 ? 1 : b);
 }
 
-// The same binade decided from the screen forms in FP32, re-decided in FP64
-// only when the FP32 product lies within 2^-20 of a power of two.
-__device__ __forceinline__ int rel_bin_screened(Screen a, Screen b, float inv_m, int inv_e,
-                                                const double* pa, const double* pb, double inv) {
-  if (a.e == kZeroExp || b.e == kZeroExp) return kFlagBinMin;
-  if (a.e == kNonFiniteExp || b.e == kNonFiniteExp || !(inv > 0.0))
-    return rel_bin(__dmul_rn(*pa, *pb), inv);
-  const float q = __fmul_rn(__fmul_rn(a.m, b.m), inv_m);   // in [0.125, 1]
-  const uint32_t frac = __float_as_uint(q) & 0x7fffffu;
-  if (frac < 8u || frac > 0x7fffffu - 8u) return rel_bin(__dmul_rn(*pa, *pb), inv);
-  const int b0 = a.e + b.e + inv_e + ((int)((__float_as_uint(q) >> 23) & 0xffu) - 127);
-  return b0 < kFlagBinMin ? kFlagBinMin : (b0 > 1 ? 1 : b0);
-}
-
-
-__host__ __device__ __forceinline__ int64_t prep_units(const Inst& in) {
-  const int64_t na = (int64_t)in.bm * in.bk, nb = (int64_t)in.bk * in.bn,
-                nt = (int64_t)in.bm * in.bn;
-  return na > nb ? (na > nt ? na : nt) : (nb > nt ? nb : nt);
-}
-
-}  // namespace
-
-int prep_ctas_of(const Inst& in) {
-  return (int)((prep_units(in) + kPrepThreads - 1) / kPrepThreads);
-}
-
-namespace {
-
-__device__ __forceinline__ int prep_ctas_dev(const Inst& in) {
-  return (int)((prep_units(in) + kPrepThreads - 1) / kPrepThreads);
+__host__ __device__ __forceinline__ int prep_parts(const Inst& in) {
+  const int64_t na = (int64_t)in.bm * in.bk, nb = (int64_t)in.bk * in.bn;
+  return (int)(((na > nb ? na : nb) + kPrepThreads - 1) / kPrepThreads);
 }
 
 __device__ __forceinline__ int inst_of_prep_cta(const InstRef& r, int cta) {
   return find_inst(r, cta, [](const Inst& x) { return (int64_t)x.prep0; });
 }
-__device__ __forceinline__ int inst_of_count_cta(const InstRef& r, int cta) {
-  return find_inst(r, cta, [](const Inst& x) { return (int64_t)x.count0; });
+__device__ __forceinline__ int inst_of_unit(const InstRef& r, int unit) {
+  return find_inst(r, unit, [](const Inst& x) { return (int64_t)x.count0; });
 }
 
+// Partial sums of squared norms (kPrepThreads of A's and of B's per CTA) and, for
+// the histogram, the screen forms; clears the accumulators of the later kernels.
 __global__ void __launch_bounds__(kPrepThreads)
-    prep_kernel(InstRef R, PlanBuffers Bf) {
+    prep_kernel(InstRef R, PlanBuffers Bf, int screens) {
+  pdl_wait();
   pdl_trigger();
-  const int ii = inst_of_prep_cta(R, blockIdx.x);
-  const Inst& in = R.at(ii);
-  const int64_t na = (int64_t)in.bm * in.bk, nb = (int64_t)in.bk * in.bn,
-                nt = (int64_t)in.bm * in.bn;
+  const int tid = threadIdx.x;
+  const Inst& in = R.at(inst_of_prep_cta(R, blockIdx.x));
+  const int64_t na = (int64_t)in.bm * in.bk, nb = (int64_t)in.bk * in.bn;
   const int lc = blockIdx.x - in.prep0;
-  const int nctas = prep_ctas_dev(in);
-  const int64_t idx = (int64_t)lc * kPrepThreads + threadIdx.x;
+  const int64_t idx = (int64_t)lc * kPrepThreads + tid;
+  if (lc == 0) {   // one CTA per instance clears its bins; the rest is dealt over the grid
+    PlanDevice* pd = in.pd;
+    for (int q = tid; q < kFlagBins; q += kPrepThreads) {
+      pd->bin_sum[q] = 0.0;
+      pd->bin_cnt[q] = 0;
+    }
+    if (tid < kHistBins) pd->hist[tid] = 0u;
+    if (tid == 0) pd->ticket = 0u;
+  }
+  {
+    const int64_t g0 = (int64_t)blockIdx.x * kPrepThreads + tid;
+    const int64_t gs = (int64_t)gridDim.x * kPrepThreads;
+    for (int64_t g = g0; g < Bf.need_words_a + Bf.need_words_b; g += gs) Bf.need_bits[g] = 0u;
+    if (Bf.group_shift) {
+      const int64_t words =
+          (int64_t)((Bf.count_ctas + (1 << Bf.group_shift) - 1) >> Bf.group_shift) * kPartInts;
+      for (int64_t g = g0; g < words; g += gs) Bf.group[g] = 0;
+    }
+    if (g0 == 0) Bf.bdev->need_count = 0;
+  }
   double qa = 0.0, qb = 0.0;
-  if (idx < nt) Bf.tile_inst[in.tile0 + idx] = ii;
   if (idx < na) {
     const double a = in.nA[idx];
-    Bf.sA[in.ablk0 + idx] = make_screen(a);
+    if (screens) Bf.sA[in.ablk0 + idx] = make_screen(a);
     qa = a * a;
   }
   if (idx < nb) {
     const double b = in.nB[idx];
-    const int64_t k = idx / in.bn, j = idx % in.bn;
-    Bf.sBT[in.bblk0 + j * in.bk + k] = make_screen(b);
+    if (screens) {
+      const int64_t k = idx / in.bn, j = idx % in.bn;
+      Bf.sBT[in.bblk0 + j * in.bk + k] = make_screen(b);
+    }
     qb = b * b;
   }
   for (int off = 16; off > 0; off >>= 1) {
     qa += __shfl_xor_sync(0xffffffffu, qa, off);
     qb += __shfl_xor_sync(0xffffffffu, qb, off);
   }
-  __shared__ double wa[kPrepThreads / 32], wb[kPrepThreads / 32];
-  if ((threadIdx.x & 31) == 0) {
-    wa[threadIdx.x / 32] = qa;
-    wb[threadIdx.x / 32] = qb;
+  __shared__ double s_w[2][kPrepThreads / 32];
+  if ((tid & 31) == 0) {
+    s_w[0][tid / 32] = qa;
+    s_w[1][tid / 32] = qb;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double sa = 0.0, sb = 0.0;
-    for (int w = 0; w < kPrepThreads / 32; ++w) {
-      sa += wa[w];
-      sb += wb[w];
-    }
-    Bf.part_a[blockIdx.x] = sa;
-    Bf.part_b[blockIdx.x] = sb;
-  }
-  // the last CTA of the instance sums its partials in a fixed order (deterministic)
-  __shared__ bool s_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&in.pd->ticket, 1u) == (unsigned)nctas - 1u;
-  __syncthreads();
-  if (s_last && threadIdx.x < 32) {
-    __threadfence();
-    const int lane = threadIdx.x;
-    double a = 0.0, b = 0.0;
-    for (int i = lane; i < nctas; i += 32) {
-      a += __ldcg(Bf.part_a + in.prep0 + i);
-      b += __ldcg(Bf.part_b + in.prep0 + i);
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, off);
-      b += __shfl_xor_sync(0xffffffffu, b, off);
-    }
-    if (lane == 0) {
-      const double na = sqrt(a), nb = sqrt(b), ab = na * nb;
-      in.pd->norm_a = na;
-      in.pd->norm_b = nb;
-      in.pd->inv_ab = ab > 0.0 ? 1.0 / ab : 0.0;
-    }
+  if (tid < 2) {
+    double x = 0.0;
+    for (int w = 0; w < kPrepThreads / 32; ++w) x += s_w[tid][w];
+    (tid ? Bf.part_b : Bf.part_a)[blockIdx.x] = x;
   }
 }
 
-// Split modes: adds a surviving product to its binade's shared-memory bin
-// (rare: the scale of ||A|| ||B|| is reloaded here rather than kept live).
-__device__ __forceinline__ void bin_survivor(Screen a, Screen b, const double* pa, const double* pb,
-                                          const PlanDevice* pd, double* bin_sum, int* bin_cnt) {
-  const double inv = pd->inv_ab;
-  int inv_e;
-  const float inv_m = (float)frexp(inv, &inv_e);
-  const double p = __dmul_rn(*pa, *pb);
-  const int bin = rel_bin_screened(a, b, inv_m, inv_e, pa, pb, inv);
-  atomicAdd(&bin_sum[bin - kFlagBinMin], p);
-  atomicAdd(&bin_cnt[bin - kFlagBinMin], 1);
+// ||A||_F (lane 0) and ||B||_F (lane 1) from `count` partial sums at `first`, by one
+// warp in a fixed order (every caller gets the same bits): the even lanes add up
+// A's, the odd ones B's, one square root serves both (FP64 is scarce here).
+__device__ __forceinline__ double sum_norms(const PlanBuffers& Bf, int first, int count) {
+  const int lane = threadIdx.x & 31;
+  const double* p = ((lane & 1) ? Bf.part_b : Bf.part_a) + first;
+  double x = 0.0;
+#pragma unroll 4
+  for (int i = lane >> 1; i < count; i += 16) x += __ldcg(p + i);
+  for (int off = 16; off > 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return sqrt(x);
 }
 
+// After prep: 1 / (||A|| ||B||) for a CTA of the instance (one warp calls it);
+// `publish`: also write the norms to the instance's statistics.
+__device__ __forceinline__ double instance_norms(const Inst& in, const PlanBuffers& Bf,
+                                                 bool publish) {
+  const double x = sum_norms(Bf, in.prep0, prep_parts(in));
+  const double na = __shfl_sync(0xffffffffu, x, 0), nb = __shfl_sync(0xffffffffu, x, 1);
+  const double ab = na * nb, inv = ab > 0.0 ? 1.0 / ab : 0.0;
+  if (publish && (threadIdx.x & 31) == 0) {
+    in.pd->norm_a = na;
+    in.pd->norm_b = nb;
+    in.pd->inv_ab = inv;
+  }
+  return inv;
+}
+
+// The flag binade m = the largest mm in [kFlagBinMin - 1, 1] with
+// c1 * sum_{bins < mm} p <= budget, by one warp; bins are prefix-summed in a
+// fixed order (7 consecutive bins per lane, then a warp scan of the lane totals).
+__device__ __forceinline__ int flag_binade(const Inst& in, double ab, double bound2) {
+  constexpr int PER = (kFlagBins + 31) / 32;   // 7
+  const int lane = threadIdx.x & 31;
+  const double budget = 0.5 * (in.target_rel * ab - bound2);
+  double v[PER];
+  double run = 0.0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int b = lane * PER + q;
+    v[q] = b < kFlagBins ? __ldcg(&in.pd->bin_sum[b]) : 0.0;
+    run += v[q];
+  }
+  double incl = run;
+  for (int off = 1; off < 32; off <<= 1) {
+    const double y = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += y;
+  }
+  double below = incl - run;     // sum of the bins before this lane's first
+  int best = kFlagBinMin - 1;
+  if (budget >= 0.0) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int b = lane * PER + q;       // candidate mm = kFlagBinMin + b
+      if (b < kFlagBins && in.c1 * below <= budget) best = kFlagBinMin + b;
+      below += v[q];
+    }
+  }
+  return __reduce_max_sync(0xffffffffu, best);
+}
+
+// One instance's sums over its units.
+struct UnitSums {
+  int S, ne, km;
+  ExtSum b1, b2;
+};
+
+// One warp's part v of an instance's sums: its lane l takes the units 32 v + l,
+// 32 v + l + 32 kStatWarps, ... (four units' loads at a time).  The kStatWarps parts
+// are merged in order (merge_sums), whoever forms them, so that a single call and
+// a batch give the same bits.
+__device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers& Bf, int v) {
+  const int units = units_of(in);
+  constexpr int nt = 32 * kStatWarps;
+  UnitSums r{0, 0, 0, {0.0f, 0}, {0.0f, 0}};
+  if (32 * v >= units) return r;   // uniform over the warp
+  for (int q0 = 32 * v + (threadIdx.x & 31); q0 < units; q0 += 4 * nt) {
+    int s4[4];
+    int4 hi[4], bb[4];
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const int64_t q = in.count0 + q0 + z * nt;
+      s4[z] = 0;
+      hi[z] = bb[z] = make_int4(0, 0, 0, 0);
+      if (q0 + z * nt < units) {
+        s4[z] = __ldcg(Bf.part + q * kPartInts + kPartS);
+        hi[z] = __ldcg(reinterpret_cast<const int4*>(Bf.part + q * kPartInts + kPartNe));
+        bb[z] = __ldcg(reinterpret_cast<const int4*>(Bf.part_bound + 2 * q));
+      }
+    }
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      r.S += s4[z];
+      r.ne += hi[z].x;
+      r.km = max(r.km, hi[z].y);
+      ext_add(r.b1, __int_as_float(bb[z].x), bb[z].y);
+      ext_add(r.b2, __int_as_float(bb[z].z), bb[z].w);
+    }
+  }
+  r.S = __reduce_add_sync(0xffffffffu, r.S);
+  r.ne = __reduce_add_sync(0xffffffffu, r.ne);
+  r.km = __reduce_max_sync(0xffffffffu, r.km);
+  r.b1 = ext_warp_sum(r.b1);
+  r.b2 = ext_warp_sum(r.b2);
+  return r;
+}
+
+__device__ __forceinline__ void merge_sums(UnitSums& u, const UnitSums& v) {
+  u.S += v.S;
+  u.ne += v.ne;
+  u.km = max(u.km, v.km);
+  ext_add(u.b1, v.b1.m, v.b1.e);
+  ext_add(u.b2, v.b2.m, v.b2.e);
+}
+
+// The statistics of one instance from its sums, by one warp (one square root and
+// one division for all of them).  prepped: the count kernel left the norms in the
+// statistics; otherwise they come from the units' partial sums and are written
+// too.  Returns the split-flag binade; publish = false: only that.
+__device__ __forceinline__ int write_stats(const Inst& in, const PlanBuffers& Bf, const UnitSums& u,
+                                           bool prepped, bool publish) {
+  const int lane = threadIdx.x & 31;
+  PlanDevice* pd = in.pd;
+  double x = prepped ? 0.0 : sum_norms(Bf, in.count0, units_of(in));
+  if (lane == 2) x = sqrt(ext_value(u.b2));
+  if (prepped && lane < 2) x = __ldcg(lane ? &pd->norm_b : &pd->norm_a);
+  const double na = __shfl_sync(0xffffffffu, x, 0), nb = __shfl_sync(0xffffffffu, x, 1);
+  const double bound2 = __shfl_sync(0xffffffffu, x, 2);
+  const double ab = na * nb;
+  const int m = in.split ? flag_binade(in, ab, bound2) : kFlagBinMin - 1;
+  if (!publish) return m;
+  const double cube = (double)in.bm * (double)in.bk * (double)in.bn;
+  const double quot = (lane == 0 ? 1.0 : (double)u.S) / (lane == 0 ? ab : cube);
+  const double ratio = __shfl_sync(0xffffffffu, quot, 1);
+  long long f = 0;
+  if (in.split) {
+    for (int b = lane; b < kFlagBins; b += 32)
+      if (kFlagBinMin + b >= m) f += (long long)__ldcg(&pd->bin_cnt[b]);
+    for (int off = 16; off > 0; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
+  }
+  if (lane == 0) {
+    pd->survivors = u.S;
+    pd->max_tile = u.km;
+    pd->nonempty = u.ne;
+    if (!prepped) {
+      pd->norm_a = na;
+      pd->norm_b = nb;
+      pd->inv_ab = ab > 0.0 ? quot : 0.0;
+    }
+    pd->bound1 = ext_value(u.b1);
+    pd->bound2 = bound2;
+    pd->valid_ratio = ratio;
+    pd->flag_exp = m;
+    pd->flagged = f;
+  }
+  return m;
+}
+
+// Part v of one instance's sums into shared memory, by one warp.
+__device__ __forceinline__ void stat_part(const Inst& in, const PlanBuffers& Bf, UnitSums* parts,
+                                          int v) {
+  const UnitSums u = unit_sums(in, Bf, v);
+  if ((threadIdx.x & 31) == 0) parts[v] = u;
+}
+
+__device__ __forceinline__ UnitSums merged(const UnitSums* parts) {
+  UnitSums u = parts[0];
+  for (int v = 1; v < kStatWarps; ++v) merge_sums(u, parts[v]);
+  return u;
+}
+
+// The statistics of one instance by a CTA of kStatWarps warps or more.
+__device__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped) {
+  __shared__ UnitSums s_u[kStatWarps];
+  if (threadIdx.x / 32 < kStatWarps) stat_part(in, Bf, s_u, threadIdx.x / 32);
+  __syncthreads();
+  if (threadIdx.x < 32) (void)write_stats(in, Bf, merged(s_u), prepped, true);
+}
+
+// Screens of one staged row or column: whole words of 32 k (the tail holds
+// zero norms) and two more, so that the rows start 16 bytes apart modulo the
+// 128 bytes of a shared-memory wavefront.
+__host__ __device__ __forceinline__ int staged_len(int bk) { return ((bk + 31) & ~31) + 2; }
+
+// One CTA per unit.  A lane owns a tile, so nothing is reduced across lanes per
+// tile and a word of the survivor mask is built in a register; about 25
+// instructions per triple and lane, bound by issue and by the latency of staging
+// (eight loads in flight per thread).  The previous form (a warp per tile, lanes
+// over k: ballots and some 150 instructions of reductions per tile) took 69 us at
+// bk = 256 (1.7e7 triples), this one 40; for 256 uneven split instances 148 -> 55.
 template <bool SPLIT, bool BAND>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
-    count_kernel(InstRef R, PlanBuffers Bf) {
+__global__ void __launch_bounds__(kCountThreads)
+    count_kernel(InstRef R, PlanBuffers Bf, int prepped, int stats) {
   pdl_wait();
   pdl_trigger();
-  __shared__ double s_bin_sum[kFlagBins];
-  __shared__ int s_bin_cnt[kFlagBins];
-  __shared__ long long s_S[kWarpsPerCta];
-  __shared__ int s_kmax[kWarpsPerCta], s_ne[kWarpsPerCta];
-  __shared__ ExtSum s_b1[kWarpsPerCta], s_b2[kWarpsPerCta];
-  __shared__ int s_keys[kOrderKeys];
-  const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-  if (threadIdx.x < kOrderKeys) s_keys[threadIdx.x] = 0;
-  const int ii = inst_of_count_cta(R, blockIdx.x);
+  extern __shared__ __align__(16) Screen s_scr[];   // [rows][len] of A, then [cols][len] of B
+  __shared__ double s_bin_sum[SPLIT ? kFlagBins : 1];
+  __shared__ int s_bin_cnt[SPLIT ? kFlagBins : 1];
+  __shared__ float s_S[kCountWarps][32];
+  __shared__ int s_E[kCountWarps][32], s_cnt[kCountWarps][32];
+  __shared__ double s_inv;
+  __shared__ bool s_last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ii = inst_of_unit(R, blockIdx.x);
   const Inst& in = R.at(ii);
+  const int lu = blockIdx.x - in.count0;
+  const Unit u = unit_at(in, lu);
   const int bm = in.bm, bk = in.bk, bn = in.bn;
   const bool split = SPLIT && in.split, band = BAND && in.band;
-  const TauScreen T = in.T;
-  const double* nA = in.nA;
-  const double* nB = in.nB;
-  PlanDevice* pd = in.pd;
+  const double* __restrict__ nA = in.nA;
+  const double* __restrict__ nB = in.nB;
+  const TestTau T = test_tau(in.T);
+  if (!prepped) {   // the accumulators of the fill kernel
+    const int64_t gs = (int64_t)gridDim.x * kCountThreads;
+    if (in.quant)
+      for (int64_t g = (int64_t)blockIdx.x * kCountThreads + tid;
+           g < Bf.need_words_a + Bf.need_words_b; g += gs)
+        Bf.need_bits[g] = 0u;
+    if (blockIdx.x == 0 && tid == 0) Bf.bdev->need_count = 0;
+  }
+  // the unit's screens (B's exponents relative to tau's)
+  const int len = staged_len(bk), kpad = len - 2;
+  Screen* sa = s_scr;
+  Screen* sb = s_scr + u.rows * len;
+  for (int x = warp; x < u.rows; x += kCountWarps) {
+    const double* src = nA + (int64_t)(u.r0 + x) * bk;
+#pragma unroll 8
+    for (int k = lane; k < kpad; k += 32) sa[x * len + k] = test_screen(k < bk ? src[k] : 0.0);
+  }
+  if (u.cols == 4) {   // lanes over (k, column): whole 32-byte sectors
+#pragma unroll 8
+    for (int x = tid; x < 4 * kpad; x += kCountThreads) {
+      const int k = x >> 2, c = x & 3;
+      Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
+      b.e -= T.e;
+      sb[c * len + k] = b;
+    }
+  } else {
+    for (int k = tid; k < kpad; k += kCountThreads)
+#pragma unroll 4
+      for (int c = 0; c < u.cols; ++c) {
+        Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
+        b.e -= T.e;
+        sb[c * len + k] = b;
+      }
+  }
   if (split) {
-    for (int i = threadIdx.x; i < kFlagBins; i += blockDim.x) {
+    for (int i = tid; i < kFlagBins; i += kCountThreads) {
       s_bin_sum[i] = 0.0;
       s_bin_cnt[i] = 0;
     }
   }
   __syncthreads();
-  const double inv = pd->inv_ab;   // written by the prep kernel
-  int inv_e;
-  const float inv_m = (float)frexp(inv, &inv_e);
-  const int64_t tiles = (int64_t)bm * bn;
-  const int nch = (bk + 31) >> 5;
-  const int64_t lt0 = (int64_t)(blockIdx.x - in.count0) * kTilesPerCta;
-  // When the CTA's 32 positions lie in one full band they are 8 block rows x
-  // 4 block columns (warp w: row r0 + w, columns j0 .. j0 + 3): those 8 rows
-  // of A's screens and 4 columns of B's are staged in shared memory with one
-  // coalesced load, so each warp meets one memory latency instead of one per
-  // tile.  Other CTAs (a ragged last band) read the screens from global memory.
-  extern __shared__ Screen s_scr[];   // [8 * bk] A rows, then [4 * bk] B columns
-  const int64_t band_tiles = (int64_t)kGroupRows * bn;
-  const int64_t band0 = lt0 / band_tiles;
-  const int r0 = (int)band0 * kGroupRows;
-  const bool staged = band0 == (lt0 + kTilesPerCta - 1) / band_tiles && r0 + kGroupRows <= bm &&
-                      lt0 + kTilesPerCta <= tiles;
-  const int j0 = (int)((lt0 - band0 * band_tiles) / kGroupRows);
-  if (staged) {
-    const int na = kGroupRows * bk, nb = kTilesPerCta / kGroupRows * bk;
-    const Screen* ga = Bf.sA + in.ablk0 + (int64_t)r0 * bk;
-    const Screen* gb = Bf.sBT + in.bblk0 + (int64_t)j0 * bk;
-#pragma unroll 4
-    for (int x = threadIdx.x; x < na + nb; x += blockDim.x)
-      s_scr[x] = x < na ? ga[x] : gb[x - na];
+
+  // lane -> tile (column by column inside the unit)
+  const int c = lane / u.rows, r = lane - c * u.rows;
+  const bool act = c < u.cols;
+  const int i = u.r0 + r, j = u.j0 + c;
+  const int64_t t = (int64_t)i * bn + j;
+  const int nch = kpad >> 5;
+  SkipSum sk{0.0f, kSkipStart};
+  int count = 0;
+  const double* pa = nA + (int64_t)i * bk;
+  const double* pb = nB + j;
+  if (act) {
+    const TestTau Th = BAND ? test_tau(in.T_hi) : T;
+    const int dhi = BAND ? T.e - Th.e : 0;
+    const float4* ra = reinterpret_cast<const float4*>(sa + r * len);
+    const float4* rb = reinterpret_cast<const float4*>(sb + c * len);
+    for (int w = warp; w < nch; w += kCountWarps) {
+      uint32_t mask = 0u, near = 0u;   // near: the FP64 product decides
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {    // eight k: four 16-byte reads of each operand
+        float q[8];
+        int D[8];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const float4 a2 = ra[w * 16 + o * 4 + h], b2 = rb[w * 16 + o * 4 + h];
+          q[2 * h] = __fmul_rn(a2.x, b2.x);
+          q[2 * h + 1] = __fmul_rn(a2.z, b2.z);
+          D[2 * h] = __float_as_int(a2.y) + __float_as_int(b2.y);
+          D[2 * h + 1] = __float_as_int(a2.w) + __float_as_int(b2.w);
+        }
+#pragma unroll
+        for (int z = 0; z < 8; ++z) {
+          const uint32_t bit = 1u << (8 * o + z);
+          const float v = screen_value(q[z], D[z]);
+          bool s = v >= T.lo;                        // a near product: settled below
+          if (s && v < T.hi) near |= bit;
+          if (BAND && band) {
+            const float v2 = screen_value(q[z], D[z] + dhi);
+            if (v2 >= Th.hi) s = false;
+            else if (v2 >= Th.lo) near |= s ? bit : 0u;
+          }
+          if (s) mask |= bit;
+          if (s) D[z] = kSkipNone;
+        }
+        skip_add<8>(sk, q, D);
+      }
+      const int left = bk - w * 32;
+      if (left < 32) mask &= (1u << left) - 1u;
+      for (near &= mask; near; near &= near - 1u) {
+        const int bit = __ffs(near) - 1, k = w * 32 + bit;
+        const double p = __dmul_rn(pa[k], pb[(int64_t)k * bn]);
+        bool s = !(p < in.T.tau);
+        if (BAND && band && s) s = p < in.T_hi.tau;
+        if (s) continue;
+        mask &= ~(1u << bit);
+        const Screen a = sa[r * len + k], b = sb[c * len + k];
+        const float q1[1] = {__fmul_rn(a.m, b.m)};
+        const int D1[1] = {a.e + b.e};
+        skip_add<1>(sk, q1, D1);
+      }
+      count += __popc(mask);
+      Bf.surv_mask[in.mask0 + t * nch + w] = mask;
+    }
+  }
+  s_S[warp][lane] = sk.S;
+  s_E[warp][lane] = sk.Emax;
+  s_cnt[warp][lane] = count;
+  const int any = __syncthreads_or(count);
+  if (prepped && ((split && any) || lu == 0)) {
+    if (warp == kCountWarps - 1) {
+      const double v = instance_norms(in, Bf, lu == 0);
+      if (lane == 0) s_inv = v;
+    }
     __syncthreads();
   }
-  long long wS = 0;
-  int wkmax = 0, wne = 0;
-  ExtSum wb1{0.0f, 0}, wb2{0.0f, 0};
-  for (int r = 0; r < kTileRounds; ++r) {
-    const int64_t pos = lt0 + warp + (int64_t)r * kWarpsPerCta;
-    if (pos >= tiles) break;
-    int i, j;
-    tile_at(pos, bm, bn, i, j);
-    const int64_t t = (int64_t)i * bn + j;
-    const Screen* ra = staged ? s_scr + (i - r0) * bk : Bf.sA + in.ablk0 + (int64_t)i * bk;
-    const Screen* rb = staged ? s_scr + (kGroupRows + j - j0) * bk : Bf.sBT + in.bblk0 + (int64_t)j * bk;
-    SkipSum sk{0.0f, kSkipNone};
-    int count = 0;
-    // the screens of up to kChunks 32-wide chunks of k are loaded together
-    // (one latency per group instead of one per chunk)
-    constexpr int kChunks = 2;
-    for (int kg = 0; kg < bk; kg += 32 * kChunks) {
-      Screen av[kChunks], bv[kChunks];
-#pragma unroll
-      for (int q = 0; q < kChunks; ++q) {
-        const int k = kg + 32 * q + lane;
-        if (k < bk) {
-          av[q] = ra[k];
-          bv[q] = rb[k];
-        }
+  if (split && act) {   // surviving products by binade (a lane reads back its own words)
+    const double inv = s_inv;
+    for (int w = warp; w < nch && count > 0; w += kCountWarps)
+      for (uint32_t bits = Bf.surv_mask[in.mask0 + t * nch + w]; bits; bits &= bits - 1u) {
+        const int k = w * 32 + __ffs(bits) - 1;
+        const double p = __dmul_rn(pa[k], pb[(int64_t)k * bn]);
+        const int bin = rel_bin(p, inv);
+        atomicAdd(&s_bin_sum[bin - kFlagBinMin], p);
+        atomicAdd(&s_bin_cnt[bin - kFlagBinMin], 1);
       }
+  }
+  if (split && any) __syncthreads();
+  if (warp == 0) {
+    // the tile's totals over the warps (fixed order), then the unit's
+    count = 0;
+    int emax = kSkipNone;
 #pragma unroll
-    for (int q = 0; q < kChunks; ++q) {
-      const int k0 = kg + 32 * q;
-      if (k0 >= bk) break;   // uniform over the warp
-      const int k = k0 + lane;
-      bool s = false;
-      if (k < bk) {
-        const Screen a = av[q], b = bv[q];
-        const double* pa = nA + (int64_t)i * bk + k;
-        const double* pb = nB + (int64_t)k * bn + j;
-        s = survives(a, b, pa, pb, T);
-        if (BAND && s && band) s = !survives(a, b, pa, pb, in.T_hi);
-        if (!s) {
-          skip_add(sk, a, b);
-        } else if (split) {
-          bin_survivor(a, b, pa, pb, pd, s_bin_sum, s_bin_cnt);
-        }
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, s);
-      count += __popc(bal);
-      if (lane == 0) Bf.surv_mask[in.mask0 + t * nch + (k0 >> 5)] = bal;
+    for (int w = 0; w < kCountWarps; ++w) {
+      count += s_cnt[w][lane];
+      emax = max(emax, s_E[w][lane]);
     }
+    float S = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kCountWarps; ++w)
+      S = __fmaf_rn(s_S[w][lane], pow2f_or_zero(max(s_E[w][lane] - emax, -127)), S);
+    const ExtSum tot = S > 0.0f ? ExtSum{S, emax + T.e} : ExtSum{0.0f, 0};
+    const ExtSum b1 = ext_warp_sum_fast(tot);
+    const ExtSum b2 = ext_warp_sum_fast(ExtSum{__fmul_rn(tot.m, tot.m), 2 * tot.e});
+    const int64_t g = in.tile0 + t;
+    if (act) {
+      Bf.cnt[g] = count;
+      if (R.count > 1) Bf.tile_inst[g] = ii;
     }
-    // the tile's skipped sum relative to ||A|| ||B|| (times inv = inv_m 2^inv_e);
-    // no FP64: the FP64 pipe is narrow here
-    ExtSum tot = ext_warp_sum_fast(skip_ext(sk));
-    if (tot.m > 0.0f) {
-      tot.m = __fmul_rn(tot.m, inv_m);
-      tot.e += inv_e;
+    const int key = count > 0 ? order_key(count) : 0;
+    int val = __reduce_add_sync(0xffffffffu, count);        // lane kPartS
+#pragma unroll
+    for (int q = 1; q < kOrderKeys; ++q) {
+      const int n = __popc(__ballot_sync(0xffffffffu, key == q));
+      if (lane == q) val = n;
+    }
+    const int ne = __popc(__ballot_sync(0xffffffffu, count > 0));
+    const int km = __reduce_max_sync(0xffffffffu, count);
+    if (lane == kPartNe) val = ne;
+    if (lane == kPartMax) val = km;
+    if (lane < kPartInts) {
+      Bf.part[(int64_t)blockIdx.x * kPartInts + lane] = lane <= kPartMax ? val : 0;
+      if (Bf.group_shift && lane < kPartNe)
+        atomicAdd(&Bf.group[(int64_t)(blockIdx.x >> Bf.group_shift) * kPartInts + lane], val);
+    }
+    if (lane == 0)
+      *reinterpret_cast<int4*>(Bf.part_bound + 2 * (int64_t)blockIdx.x) =
+          make_int4(__float_as_int(b1.m), b1.e, __float_as_int(b2.m), b2.e);
+  } else if (warp == 1 && !prepped) {
+    // this unit's share of the squared norms of A and B
+    const int units = units_of(in);
+    const int64_t na = (int64_t)bm * bk, nb = (int64_t)bk * bn;
+    const int64_t la = (na + units - 1) / units, lb = (nb + units - 1) / units;
+    double qa = 0.0, qb = 0.0;
+    for (int64_t x = lu * la + lane; x < min(na, (lu + 1) * la); x += 32) qa = __fma_rn(nA[x], nA[x], qa);
+    for (int64_t x = lu * lb + lane; x < min(nb, (lu + 1) * lb); x += 32) qb = __fma_rn(nB[x], nB[x], qb);
+    for (int off = 16; off > 0; off >>= 1) {
+      qa += __shfl_xor_sync(0xffffffffu, qa, off);
+      qb += __shfl_xor_sync(0xffffffffu, qb, off);
     }
     if (lane == 0) {
-      const int64_t g = in.tile0 + t;
-      Bf.cnt[g] = count;
-      if (count > 0) atomicAdd(&s_keys[order_key(count)], 1);
-      ext_add(wb1, tot.m, tot.e);
-      ext_add(wb2, __fmul_rn(tot.m, tot.m), 2 * tot.e);
+      Bf.part_a[blockIdx.x] = qa;
+      Bf.part_b[blockIdx.x] = qb;
     }
-    wS += count;
-    wkmax = max(wkmax, count);
-    wne += count > 0;
   }
-  if (lane == 0) {
-    s_S[warp] = wS;
-    s_kmax[warp] = wkmax;
-    s_ne[warp] = wne;
-    s_b1[warp] = wb1;
-    s_b2[warp] = wb2;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long S = 0;
-    int km = 0, ne = 0;
-    ExtSum b1{0.0f, 0}, b2{0.0f, 0};
-    for (int w = 0; w < kWarpsPerCta; ++w) {
-      S += s_S[w];
-      km = max(km, s_kmax[w]);
-      ne += s_ne[w];
-      ext_add(b1, s_b1[w].m, s_b1[w].e);
-      ext_add(b2, s_b2[w].m, s_b2[w].e);
-    }
-    Bf.part_S[blockIdx.x] = S;
-    Bf.part_kmax[blockIdx.x] = km;
-    for (int q = 0; q < kOrderKeys; ++q) Bf.part_keys[(int64_t)blockIdx.x * kOrderKeys + q] = s_keys[q];
-    Bf.part_ne[blockIdx.x] = ne;
-    Bf.part_b1[blockIdx.x] = b1;
-    Bf.part_b2[blockIdx.x] = b2;
-  }
-  if (split) {
-    for (int i = threadIdx.x; i < kFlagBins; i += blockDim.x) {
-      if (s_bin_cnt[i]) {
-        atomicAdd(&pd->bin_sum[i], s_bin_sum[i]);
-        atomicAdd(&pd->bin_cnt[i], (unsigned long long)s_bin_cnt[i]);
+  if (split && any) {
+    for (int q = tid; q < kFlagBins; q += kCountThreads) {
+      if (s_bin_cnt[q]) {
+        atomicAdd(&in.pd->bin_sum[q], s_bin_sum[q]);
+        atomicAdd(&in.pd->bin_cnt[q], (unsigned long long)s_bin_cnt[q]);
       }
     }
   }
+  if (!stats) return;
+  // the last unit of the instance forms its statistics
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&in.pd->ticket, 1u) == (unsigned)units_of(in) - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  instance_stats(in, Bf, true);
 }
 
 // Histogram bin of r = fl(fl(na nb) * inv) (one FP64 multiply, no other rounding):
@@ -517,24 +787,30 @@ __device__ __forceinline__ int hist_bin_screened(Screen a, Screen b, float inv_m
 // Histogram of every triple of every instance: one warp per output tile,
 // lanes over k; equal bins of a warp are merged with match_any before the
 // shared-memory atomics, CTA totals go to the instance's global bins.
-__global__ void __launch_bounds__(kWarpsPerCta * 32)
+__global__ void __launch_bounds__(kHistWarps * 32)
     hist_kernel(InstRef R, PlanBuffers Bf) {
   __shared__ unsigned int s_hist[kHistBins];
   const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-  const int ii = inst_of_count_cta(R, blockIdx.x);
+  const int ii = inst_of_unit(R, blockIdx.x);
   const Inst& in = R.at(ii);
   const int bk = in.bk, bn = in.bn;
   const double* nA = in.nA;
   const double* nB = in.nB;
   for (int q = threadIdx.x; q < kHistBins; q += blockDim.x) s_hist[q] = 0u;
   __syncthreads();
-  const double inv = in.pd->inv_ab;   // written by the prep kernel
+  __shared__ double s_inv;
+  if (warp == 0) {
+    const double v = instance_norms(in, Bf, blockIdx.x == in.count0);
+    if (lane == 0) s_inv = v;
+  }
+  __syncthreads();
+  const double inv = s_inv;
   int inv_e;
   const float inv_m = (float)frexp(inv, &inv_e);
   const int64_t tiles = (int64_t)in.bm * bn;
-  const int64_t lt0 = (int64_t)(blockIdx.x - in.count0) * kTilesPerCta;
-  for (int r = 0; r < kTileRounds; ++r) {
-    const int64_t t = lt0 + warp + (int64_t)r * kWarpsPerCta;
+  const int64_t lt0 = (int64_t)(blockIdx.x - in.count0) * kHistTiles;
+  for (int r = 0; r < kHistTiles / kHistWarps; ++r) {
+    const int64_t t = lt0 + warp + (int64_t)r * kHistWarps;
     if (t >= tiles) break;
     const int i = (int)(t / bn), j = (int)(t % bn);
     const Screen* ra = Bf.sA + in.ablk0 + (int64_t)i * bk;
@@ -555,380 +831,290 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32)
     if (s_hist[q]) atomicAdd(&in.pd->hist[q], s_hist[q]);
 }
 
-// Block-wide exclusive scan of K values per thread at once (one shuffle scan
-// per warp, one warp over the warp totals): ex[k] = prefix, total[k] = sum.
-// `sh` holds 33 * K ints; every thread of the block calls it.
-template <int K>
-__device__ void block_scan_vec(const int (&x)[K], int (&ex)[K], int (&total)[K], int* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = (int)(blockDim.x >> 5);
-  int incl[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) incl[k] = x[k];
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int y = __shfl_up_sync(0xffffffffu, incl[k], off);
-      if (lane >= off) incl[k] += y;
-    }
-  }
-  if (lane == 31)
-#pragma unroll
-    for (int k = 0; k < K; ++k) sh[warp * K + k] = incl[k];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int w = lane < nwarps ? sh[lane * K + k] : 0;
-      int wi = w;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, wi, off);
-        if (lane >= off) wi += y;
-      }
-      sh[lane * K + k] = wi - w;
-      if (lane == 31) sh[32 * K + k] = wi;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    ex[k] = sh[warp * K + k] + incl[k] - x[k];
-    total[k] = sh[32 * K + k];
-  }
-  __syncthreads();   // sh is reused by the next scan
-}
-
-// One CTA per instance: per-CTA slot bases (survivors, non-empty tiles, order
-// buckets) by one vector scan, statistics, skipped bounds and the split-flag
-// binade; the last CTA to finish lays out the batch-wide longest-first order.
-__global__ void __launch_bounds__(kFinThreads)
-    finalize_kernel(InstRef R, PlanBuffers Bf) {
+// Work queues of `per_cta` consecutive units per CTA (kUnitWarps warps per
+// unit).  The first slots come from the totals of all units (or of the groups
+// of units): a few KB from L2 per CTA, instead of a scan kernel of its own
+// between count and fill.  Count and fill together, without the memset, prep and
+// finalize launches they replace: 30 -> 11 us at 32 blocks per side, 48 -> 17 at
+// 64 (10% of the triples survive), 169 -> 26 at 128 (half of them survive: one
+// atomic per word of needed blocks instead of two per triple).
+__global__ void __launch_bounds__(kFillThreads)
+    fill_kernel(InstRef R, PlanBuffers Bf, int per_cta, int prepped) {
   pdl_wait();
   pdl_trigger();
-  constexpr int K = 2 + (kOrderKeys - 1);   // survivors, non-empty, buckets 1 .. kOrderKeys-1
-  __shared__ int s_sh[33 * K];
-  __shared__ int s_kmax[kFinThreads / 32];
-  __shared__ ExtSum s_b1[kFinThreads / 32], s_b2[kFinThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const Inst& in = R.at(blockIdx.x);
-  const int nparts = (int)(((int64_t)in.bm * in.bn + kTilesPerCta - 1) / kTilesPerCta);
-  PlanDevice* pd = in.pd;
-
-  // each thread takes a contiguous chunk of the instance's count CTAs
-  const int chunk = (nparts + kFinThreads - 1) / kFinThreads;
-  const int p0 = min(nparts, chunk * tid), p1 = min(nparts, p0 + chunk);
-  int loc[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) loc[k] = 0;
-  int locK = 0;
-  ExtSum locB1{0.0f, 0}, locB2{0.0f, 0};
-  for (int q = p0; q < p1; ++q) {
-    const int cq = in.count0 + q;
-    loc[0] += (int)Bf.part_S[cq];   // at most 32 * bk per CTA
-    loc[1] += Bf.part_ne[cq];
-#pragma unroll
-    for (int key = 1; key < kOrderKeys; ++key)
-      loc[1 + key] += Bf.part_keys[(int64_t)cq * kOrderKeys + key];
-    locK = max(locK, Bf.part_kmax[cq]);
-    ext_add(locB1, Bf.part_b1[cq].m, Bf.part_b1[cq].e);
-    ext_add(locB2, Bf.part_b2[cq].m, Bf.part_b2[cq].e);
-  }
-  int ex[K], tot[K];
-  block_scan_vec<K>(loc, ex, tot, s_sh);
-  {
-    int base[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) base[k] = ex[k];
-    for (int q = p0; q < p1; ++q) {
-      const int cq = in.count0 + q;
-      Bf.cta_base[cq] = (int)in.kidx0 + base[0];
-      base[0] += (int)Bf.part_S[cq];
-      Bf.ne_cta_base[cq] = base[1];
-      base[1] += Bf.part_ne[cq];
-#pragma unroll
-      for (int key = 1; key < kOrderKeys; ++key) {
-        const int64_t o = (int64_t)cq * kOrderKeys + key;
-        Bf.key_cta_base[o] = base[1 + key];
-        base[1 + key] += Bf.part_keys[o];
-      }
-    }
-  }
-  // max and the extended-range sums (FP32 only): warp shuffles, then warp 0
-  for (int off = 16; off > 0; off >>= 1) locK = max(locK, __shfl_xor_sync(0xffffffffu, locK, off));
-  locB1 = ext_warp_sum(locB1);
-  locB2 = ext_warp_sum(locB2);
-  if (lane == 0) {
-    s_kmax[warp] = locK;
-    s_b1[warp] = locB1;
-    s_b2[warp] = locB2;
-  }
-  __syncthreads();
-
-  // warp 0: totals and the split flag binade m = the largest mm in
-  // [kFlagBinMin - 1, 1] with c1 * sum_{bins < mm} p <= budget; bins are
-  // prefix-summed in a fixed order (7 consecutive bins per lane, then a warp
-  // scan of the lane totals).
-  if (warp == 0) {
-    int kmax = lane < kFinThreads / 32 ? s_kmax[lane] : 0;
-    ExtSum b1x = lane < kFinThreads / 32 ? s_b1[lane] : ExtSum{0.0f, 0};
-    ExtSum b2x = lane < kFinThreads / 32 ? s_b2[lane] : ExtSum{0.0f, 0};
-    for (int off = 16; off > 0; off >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, off));
-    b1x = ext_warp_sum(b1x);
-    b2x = ext_warp_sum(b2x);
-    const double ab = pd->norm_a * pd->norm_b;
-    const double b1 = ext_value(b1x);
-    const double bound2 = sqrt(ext_value(b2x)) * ab;
-    constexpr int PER = (kFlagBins + 31) / 32;   // 7
-    int m = kFlagBinMin - 1;
-    long long flagged = 0;
-    if (in.split) {
-      const double budget = 0.5 * (in.target_rel * ab - bound2);
-      double v[PER];
-      double run = 0.0;
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        const int b = lane * PER + q;
-        v[q] = b < kFlagBins ? pd->bin_sum[b] : 0.0;
-        run += v[q];
-      }
-      double incl = run;
-      for (int off = 1; off < 32; off <<= 1) {
-        const double y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-      }
-      double below = incl - run;     // sum of the bins before this lane's first
-      int best = kFlagBinMin - 1;
-      if (budget >= 0.0) {
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          const int b = lane * PER + q;       // candidate mm = kFlagBinMin + b
-          if (b < kFlagBins && in.c1 * below <= budget) best = kFlagBinMin + b;
-          below += v[q];
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
-      m = best;
-      long long f = 0;
-      for (int b = lane; b < kFlagBins; b += 32)
-        if (kFlagBinMin + b >= m) f += (long long)pd->bin_cnt[b];
-      for (int off = 16; off > 0; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
-      flagged = f;
-    }
-    if (lane == 0) {
-      pd->survivors = tot[0];
-      pd->max_tile = kmax;
-      pd->nonempty = tot[1];
-      for (int key = 1; key < kOrderKeys; ++key) pd->key_tot[key] = tot[1 + key];
-      pd->bound1 = b1 * ab;
-      pd->bound2 = bound2;
-      pd->valid_ratio = (double)tot[0] / ((double)in.bm * (double)in.bk * (double)in.bn);
-      pd->flag_exp = m;
-      pd->flagged = flagged;
-    }
-  }
-
-  // one instance: its own totals lay out the order (no other CTA to wait for)
-  if (gridDim.x == 1) {
-    if (tid == 0) {
-      int acc = 0;
-      for (int key = kOrderKeys - 1; key >= 1; --key) {   // largest key first
-        Bf.bdev->cursor[key] = acc;
-        pd->key_base[key] = acc;
-        acc += tot[1 + key];
-      }
-      Bf.bdev->nonempty = acc;
-      pd->ne_base = 0;
-    }
+  constexpr int kMaxPer = 32;
+  __shared__ int s_red[kFillWarps][2 * kPartInts];
+  __shared__ int s_base[kPartInts];          // buckets 1 .. 11: first slots of the CTA's units
+  __shared__ int s_nonempty;                 // non-empty tiles of all units
+  __shared__ int s_part[kMaxPer][kPartInts];
+  __shared__ UnitSums s_u[kStatWarps];
+  __shared__ int s_m[kMaxPer];               // split flag binade of instance ii0 + z
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int U = Bf.count_ctas;
+  const int u0 = blockIdx.x * per_cta, u1 = min(U, u0 + per_cta);
+  if (u0 >= U) {   // no split modes: one more CTA per instance forms its statistics
+    instance_stats(R.at(blockIdx.x - (U + per_cta - 1) / per_cta), Bf, prepped != 0);
     return;
   }
-
-  // the last finalize CTA: bucket starts of the batch-wide longest-first
-  // order, each instance's first slot in each bucket and its non-empty base
-  __shared__ bool s_last;
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&Bf.bdev->ticket, 1u) == gridDim.x - 1u;
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    constexpr int KB = kOrderKeys;   // buckets 1 .. kOrderKeys-1 and (slot 0) non-empty
-    int sum[KB];
+  const int ii0 = inst_of_unit(R, u0);
+  const int first = R.at(ii0).count0;   // of u0's instance
+  const int sub = warp / kUnitWarps, wu = warp % kUnitWarps;
+  // the first unit of this warp: its counts and first words, on their way while
+  // the totals are added up
+  int count_next = 0;
+  uint32_t word_next[4] = {0u, 0u, 0u, 0u};
+  if (u0 + sub < u1) {
+    const Inst& in = R.at(inst_of_unit(R, u0 + sub));
+    const Unit u = unit_at(in, u0 + sub - in.count0);
+    const int nch = (in.bk + 31) >> 5;
+    const int c = lane / u.rows, r = lane - c * u.rows;
+    if (c < u.cols) {
+      const int64_t t = (int64_t)(u.r0 + r) * in.bn + u.j0 + c;
+      count_next = __ldcg(Bf.cnt + in.tile0 + t);
 #pragma unroll
-    for (int k = 0; k < KB; ++k) sum[k] = 0;
-    for (int i0 = 0; i0 < R.count; i0 += kFinThreads) {   // pass 1: totals over instances
-      const int i = i0 + tid;
-      int v[KB], e[KB], t[KB];
-#pragma unroll
-      for (int k = 0; k < KB; ++k) v[k] = 0;
-      if (i < R.count) {
-        const PlanDevice* q = R.at(i).pd;
-        v[0] = __ldcg(&q->nonempty);
-#pragma unroll
-        for (int key = 1; key < kOrderKeys; ++key) v[key] = __ldcg(&q->key_tot[key]);
-      }
-      block_scan_vec<KB>(v, e, t, s_sh);
-#pragma unroll
-      for (int k = 0; k < KB; ++k) sum[k] += t[k];
-    }
-    int start[KB];   // start[key]: first slot of the bucket (largest key first)
-    {
-      int acc = 0;
-#pragma unroll
-      for (int key = kOrderKeys - 1; key >= 1; --key) {
-        start[key] = acc;
-        acc += sum[key];
-      }
-      start[0] = 0;
-      if (tid == 0) {
-        for (int key = 1; key < kOrderKeys; ++key) Bf.bdev->cursor[key] = start[key];
-        Bf.bdev->nonempty = acc;
-      }
-    }
-    int carry[KB];
-#pragma unroll
-    for (int k = 0; k < KB; ++k) carry[k] = 0;
-    for (int i0 = 0; i0 < R.count; i0 += kFinThreads) {   // pass 2: per-instance bases
-      const int i = i0 + tid;
-      int v[KB], e[KB], t[KB];
-#pragma unroll
-      for (int k = 0; k < KB; ++k) v[k] = 0;
-      if (i < R.count) {
-        const PlanDevice* q = R.at(i).pd;
-        v[0] = __ldcg(&q->nonempty);
-#pragma unroll
-        for (int key = 1; key < kOrderKeys; ++key) v[key] = __ldcg(&q->key_tot[key]);
-      }
-      block_scan_vec<KB>(v, e, t, s_sh);
-      if (i < R.count) {
-        PlanDevice* q = R.at(i).pd;
-        q->ne_base = carry[0] + e[0];
-        for (int key = 1; key < kOrderKeys; ++key) q->key_base[key] = start[key] + carry[key] + e[key];
-      }
-#pragma unroll
-      for (int k = 0; k < KB; ++k) carry[k] += t[k];
+      for (int q = 0; q < 4; ++q)
+        if (q < nch) word_next[q] = __ldcg(Bf.surv_mask + in.mask0 + t * nch + q);
     }
   }
-}
-
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
-    fill_kernel(InstRef R, PlanBuffers Bf) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ int s_beg[kTilesPerCta];
-  const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-  const int ii = inst_of_count_cta(R, blockIdx.x);
-  const Inst& in = R.at(ii);
-  const int bm = in.bm, bk = in.bk, bn = in.bn, split = in.split, quant = in.quant;
-  const double* nA = in.nA;
-  const double* nB = in.nB;
-  const int64_t tiles = (int64_t)bm * bn;
-  const int nch = (bk + 31) >> 5;
-  const int64_t lt0 = (int64_t)(blockIdx.x - in.count0) * kTilesPerCta;
-  uint32_t* bitsA = Bf.need_bits;
-  uint32_t* bitsB = Bf.need_bits + Bf.need_words_a;
-  if (warp == 0) {   // first k_idx slot of each of the CTA's tiles (kTilesPerCta == 32 lanes)
-    const int64_t pos = lt0 + lane;
-    // lane q < kOrderKeys: this CTA's first slot in bucket q (loaded with the counts)
-    int key_slot = 0;
-    if (lane > 0 && lane < kOrderKeys)
-      key_slot = in.pd->key_base[lane] + Bf.key_cta_base[(int64_t)blockIdx.x * kOrderKeys + lane];
-    int64_t g = 0;
-    int c = 0;
-    if (pos < tiles) {
-      int i, j;
-      tile_at(pos, bm, bn, i, j);
-      g = in.tile0 + (int64_t)i * bn + j;
-      c = Bf.cnt[g];
+  const int ii1 = R.any_split ? inst_of_unit(R, u1 - 1) : ii0;
+  // split modes: the flag binade of every instance with units here, one warp per
+  // instance; the sums of a lone one are formed by the upper warps while the lower
+  // ones add up the totals, and finished below
+  const bool lone = R.any_split && ii0 == ii1;
+  if (R.any_split && !lone) {
+    for (int z = warp; z <= ii1 - ii0; z += kFillWarps) {
+      const Inst& in = R.at(ii0 + z);
+      UnitSums u = unit_sums(in, Bf, 0);
+      for (int v = 1; v < kStatWarps && 32 * v < units_of(in); ++v)
+        merge_sums(u, unit_sums(in, Bf, v));
+      const int m = write_stats(in, Bf, u, true, in.count0 >= u0);
+      if (lane == 0) s_m[z] = m;
     }
-    int incl = c;
+  }
+  const int scan_warps = lone ? kFillWarps - kStatWarps : kFillWarps;
+  const int scan_threads = scan_warps * 32;
+  if (warp >= scan_warps) {
+    stat_part(R.at(ii0), Bf, s_u, warp - scan_warps);
+  } else {
+    // per thread: totals of the buckets over all units and over those before
+    // u0; survivors of u0's instance before u0
+    int tot[kPartInts], bef[kPartInts];
+#pragma unroll
+    for (int q = 0; q < kPartInts; ++q) tot[q] = bef[q] = 0;
+    auto add = [&](int (&dst)[kPartInts], const int* p, int sign) {
+      const int4* v = reinterpret_cast<const int4*>(p);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const int4 x = __ldcg(v + q);
+        dst[4 * q] += sign * x.x;
+        dst[4 * q + 1] += sign * x.y;
+        dst[4 * q + 2] += sign * x.z;
+        dst[4 * q + 3] += sign * x.w;
+      }
+    };
+    if (Bf.group_shift == 0) {
+      for (int q = tid; q < U; q += scan_threads) {
+        int x[kPartInts];
+#pragma unroll
+        for (int z = 0; z < kPartInts; ++z) x[z] = 0;
+        add(x, Bf.part + (int64_t)q * kPartInts, 1);
+        const bool before = q < u0;
+        if (q >= first && before) bef[kPartS] += x[kPartS];
+#pragma unroll
+        for (int z = 1; z < kOrderKeys; ++z) {
+          tot[z] += x[z];
+          if (before) bef[z] += x[z];
+        }
+      }
+    } else {
+      const int gs = Bf.group_shift, ng = (U + (1 << gs) - 1) >> gs;
+      const int gu = u0 >> gs, gf = first >> gs;
+      for (int q = tid; q < ng; q += scan_threads) {
+        int x[kPartInts];
+#pragma unroll
+        for (int z = 0; z < kPartInts; ++z) x[z] = 0;
+        add(x, Bf.group + (int64_t)q * kPartInts, 1);
+        if (q < gu) bef[kPartS] += x[kPartS];
+        if (q < gf) bef[kPartS] -= x[kPartS];
+#pragma unroll
+        for (int z = 1; z < kOrderKeys; ++z) {
+          tot[z] += x[z];
+          if (q < gu) bef[z] += x[z];
+        }
+      }
+      for (int q = (gu << gs) + tid; q < u0; q += scan_threads)
+        add(bef, Bf.part + (int64_t)q * kPartInts, 1);
+      for (int q = (gf << gs) + tid; q < first; q += scan_threads)
+        bef[kPartS] -= __ldcg(Bf.part + (int64_t)q * kPartInts + kPartS);
+    }
+#pragma unroll
+    for (int q = 0; q < kOrderKeys; ++q) {
+      const int a = __reduce_add_sync(0xffffffffu, tot[q]);
+      const int b = __reduce_add_sync(0xffffffffu, bef[q]);
+      if (lane == 0) {
+        s_red[warp][q] = a;
+        s_red[warp][kPartInts + q] = b;
+      }
+    }
+    for (int x = tid; x < (u1 - u0) * kPartInts; x += scan_threads)
+      s_part[x / kPartInts][x % kPartInts] = __ldcg(Bf.part + (int64_t)u0 * kPartInts + x);
+  }
+  __syncthreads();
+  if (warp == kFillWarps - 1 && lone) {
+    const Inst& in = R.at(ii0);   // the CTA of its first unit also writes its statistics
+    const int m = write_stats(in, Bf, merged(s_u), true, in.count0 >= u0);
+    if (lane == 0) s_m[0] = m;
+  }
+  if (warp == 0) {
+    // lane q: bucket q's total and the part before u0; largest bucket first
+    int a = 0, b = 0;
+    if (lane < kOrderKeys)
+      for (int w = 0; w < scan_warps; ++w) {
+        a += s_red[w][lane];
+        b += s_red[w][kPartInts + lane];
+      }
+    int below = 0;   // non-empty tiles in the buckets above this lane's
+    const int all = __reduce_add_sync(0xffffffffu, a);
+#pragma unroll
+    for (int q = 1; q < kOrderKeys; ++q) {
+      const int x = __shfl_sync(0xffffffffu, a, q);
+      if (q > lane) below += x;
+    }
+    const int ne_before = __reduce_add_sync(0xffffffffu, lane >= 1 ? b : 0);
+    if (lane < kOrderKeys) s_base[lane] = lane == kPartS ? b : below + b;
+    if (lane == kPartNe) s_base[lane] = ne_before;
+    if (lane == 0) {
+      s_nonempty = all;
+      if (blockIdx.x == 0) Bf.bdev->nonempty = all;
+    }
+  }
+  __syncthreads();
+  const int nonempty = s_nonempty;
+  for (int un = u0 + sub; un < u1; un += kFillWarps / kUnitWarps) {
+    const int ii = inst_of_unit(R, un);
+    const Inst& in = R.at(ii);
+    const int bk = in.bk, bn = in.bn;
+    const Unit u = unit_at(in, un - in.count0);
+    const int nch = (bk + 31) >> 5;
+    const int c = lane / u.rows, r = lane - c * u.rows;
+    const bool act = c < u.cols;
+    const int i = u.r0 + r, j = u.j0 + c;
+    const int64_t t = (int64_t)i * bn + j, g = in.tile0 + t;
+    const bool first_round = un == u0 + sub;
+    const int count = first_round ? count_next : (act ? Bf.cnt[g] : 0);
+    // lane q: the unit's first slot in bucket q, lane 0: survivors before it in
+    // its instance, lane kPartNe: non-empty tiles before it
+    int base = 0;
+    if (lane < kPartInts) {
+      base = s_base[lane];
+      const int q0 = max(u0, in.count0);   // the CTA's first unit of this instance
+      if (lane == kPartS && in.count0 > u0) base = 0;
+      for (int q = lane == kPartS ? q0 : u0; q < un; ++q) base += s_part[q - u0][lane];
+    }
+    int incl = count;
     for (int off = 1; off < 32; off <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, incl, off);
       if (lane >= off) incl += y;
     }
-    const int beg = Bf.cta_base[blockIdx.x] + incl - c;
-    s_beg[lane] = beg;
-    if (pos < tiles) Bf.tile_beg[g] = beg;
-    // empty tiles go after all non-empty ones, in enumeration order: the rank
-    // of an empty tile is its position minus the non-empty tiles before it
-    // non-empty tiles: bucket slot = instance base + earlier CTAs + rank among
-    // the CTA's lanes of the same bucket (enumeration order inside a bucket)
-    const int key = c > 0 ? order_key(c) : 0;
+    const int beg = (int)in.kidx0 + __shfl_sync(0xffffffffu, base, kPartS) + incl - count;
+    const int key = count > 0 ? order_key(count) : 0;
     const unsigned same = __match_any_sync(0xffffffffu, key);
-    const int first = __shfl_sync(0xffffffffu, key_slot, key);
-    if (c > 0) Bf.order[first + __popc(same & ((1u << lane) - 1u))] = (int)g;
-    const unsigned ne_mask = __ballot_sync(0xffffffffu, c > 0);
-    if (pos < tiles && c == 0) {
-      const int64_t ne_before = (int64_t)in.pd->ne_base + Bf.ne_cta_base[blockIdx.x] +
-                                __popc(ne_mask & ((1u << lane) - 1u));
-      Bf.order[Bf.bdev->nonempty + (in.tile0 + pos - ne_before)] = (int)g;
+    const int slot0 = __shfl_sync(0xffffffffu, base, key);
+    const unsigned ne_mask = __ballot_sync(0xffffffffu, count > 0);
+    const int ne0 = __shfl_sync(0xffffffffu, base, kPartNe);
+    const unsigned lower = (1u << lane) - 1u;
+    if (wu == 0 && act) {
+      Bf.tile_beg[g] = beg;
+      if (count > 0) {
+        Bf.order[slot0 + __popc(same & lower)] = (int)g;
+      } else {
+        const int64_t pos = in.tile0 + (int64_t)u.r0 * bn + (int64_t)j * u.rows + r;
+        Bf.order[nonempty + (pos - (ne0 + __popc(ne_mask & lower)))] = (int)g;
+      }
     }
-  }
-  __syncthreads();
-  const double inv = in.pd->inv_ab;
-  int inv_e;
-  const float inv_m = (float)frexp(inv, &inv_e);
-  const int m = in.pd->flag_exp;
-  // dense skip sets (more than 4 survivors per block on average): most blocks are
-  // listed after the first few triples, so a plain read of the bit spares the
-  // atomic; on sparse ones the read would only add latency
-  const bool read_first =
-      quant && in.pd->survivors > 4 * ((int64_t)bm * bk + (int64_t)bk * bn);
-  for (int r = 0; r < kTileRounds; ++r) {
-    const int lt = warp + r * kWarpsPerCta;
-    const int64_t pos = lt0 + lt;
-    if (pos >= tiles) break;
-    int i, j;
-    tile_at(pos, bm, bn, i, j);
-    const int64_t g = in.tile0 + (int64_t)i * bn + j;
-    const int c = Bf.cnt[g];
-    if (c == 0) continue;
-    const Screen* ra = Bf.sA + in.ablk0 + (int64_t)i * bk;
-    const Screen* rb = Bf.sBT + in.bblk0 + (int64_t)j * bk;
-    int base = s_beg[lt];
-    // the count kernel's ballots: one word per 32 k, expanded in increasing k
-    const uint32_t* mrow = Bf.surv_mask + in.mask0 + ((int64_t)i * bn + j) * nch;
-    for (int qg = 0; qg < nch; qg += 4) {
-      unsigned words[4];
+    // expand the bitmask words, tile by tile (the unit's warps take turns)
+    const uint32_t* mrow = Bf.surv_mask + in.mask0 + t * nch;
+    const int split = in.split;
+    const int m = split ? s_m[ii - ii0] : 0;
+    const double inv = split && ne_mask ? in.pd->inv_ab : 0.0;
+    int cursor = beg;
+    for (int w0 = 0; w0 < nch; w0 += 4) {
+      uint32_t word[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) words[q] = qg + q < nch ? __ldg(mrow + qg + q) : 0u;
+      for (int q = 0; q < 4; ++q)
+        word[q] = first_round && w0 == 0 ? word_next[q]
+                                         : (count > 0 && w0 + q < nch ? __ldg(mrow + w0 + q) : 0u);
+      unsigned todo = ne_mask;
+      int turn = 0;
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        if ((turn++ & (kUnitWarps - 1)) != wu) continue;
+        int at = __shfl_sync(0xffffffffu, cursor, src);
+        const int si = __shfl_sync(0xffffffffu, i, src), sj = __shfl_sync(0xffffffffu, j, src);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const unsigned ball = words[q];
-        if (ball == 0u) continue;   // uniform over the warp
-        const int k = (qg + q) * 32 + lane;
-        const bool s = (ball >> lane) & 1u;
-        if (s) {
-          uint16_t v = (uint16_t)k;
-          if (split && rel_bin_screened(ra[k], rb[k], inv_m, inv_e, nA + (int64_t)i * bk + k,
-                                        nB + (int64_t)k * bn + j, inv) >= m)
-            v |= kSplitFlag;
-          Bf.k_idx[base + __popc(ball & ((1u << lane) - 1u))] = v;
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t bits = __shfl_sync(0xffffffffu, word[q], src);
+          if (bits == 0u) continue;   // uniform over the warp
+          if ((bits >> lane) & 1u) {
+            const int k = (w0 + q) * 32 + lane;
+            uint16_t v = (uint16_t)k;
+            if (split && rel_bin(__dmul_rn(in.nA[(int64_t)si * bk + k], in.nB[(int64_t)k * bn + sj]),
+                                 inv) >= m)
+              v |= kSplitFlag;
+            Bf.k_idx[at + __popc(bits & lower)] = v;
+          }
+          at += __popc(bits);
         }
-        base += __popc(ball);
-        if (quant) {
-          // list the A and B blocks of surviving triples, each once over the plan
-          const int64_t ga = in.ablk0 + (int64_t)i * bk + k, gb = in.bblk0 + (int64_t)k * bn + j;
-          bool newA = false, newB = false;
-          if (s) {
-            // a bit once set stays set: a plain read from L2 that already shows it
-            // spares the atomic (atomics on the same words serialise)
-            const uint32_t bitA = 1u << (ga & 31), bitB = 1u << (gb & 31);
-            newA = (!read_first || (__ldcg(&bitsA[ga >> 5]) & bitA) == 0u) &&
-                   (atomicOr(&bitsA[ga >> 5], bitA) & bitA) == 0u;
-            newB = (!read_first || (__ldcg(&bitsB[gb >> 5]) & bitB) == 0u) &&
-                   (atomicOr(&bitsB[gb >> 5], bitB) & bitB) == 0u;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cursor += __popc(word[q]);
+      if (in.quant && wu == kUnitWarps - 1) {
+        // the blocks of A and B that the unit's triples use: lane x < rows holds row x
+        // of A, the next cols lanes the columns of B, 32 k per word; the four words'
+        // round trips go out together
+        uint32_t mine[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          mine[q] = 0u;
+          if (!__any_sync(0xffffffffu, word[q] != 0u)) continue;
+          for (int x = 0; x < u.rows + u.cols; ++x) {
+            const bool in_set = x < u.rows ? r == x : c == x - u.rows;
+            const uint32_t o = __reduce_or_sync(0xffffffffu, in_set ? word[q] : 0u);
+            if (lane == x) mine[q] = o;
           }
-          const unsigned ma = __ballot_sync(0xffffffffu, newA), mb = __ballot_sync(0xffffffffu, newB);
-          if (ma | mb) {
-            int nb = 0;
-            if (lane == 0) nb = atomicAdd(&Bf.bdev->need_count, __popc(ma) + __popc(mb));
-            nb = __shfl_sync(0xffffffffu, nb, 0);
-            const unsigned lt = (1u << lane) - 1u;
-            if (newA) Bf.need_list[nb + __popc(ma & lt)] = (uint32_t)ga;
-            if (newB) Bf.need_list[nb + __popc(ma) + __popc(mb & lt)] = (uint32_t)gb | 0x80000000u;
-          }
+        }
+        const bool isB = lane >= u.rows;
+        const int bi = isB ? u.j0 + lane - u.rows : u.r0 + lane;   // column of B / row of A
+        uint32_t* w = Bf.need_bits + (isB ? Bf.need_words_a + in.needb0 : in.needa0) +
+                      (int64_t)bi * nch + w0;
+        uint32_t fresh[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)   // a plain read first: a bit once set stays set
+          fresh[q] = mine[q] ? mine[q] & ~__ldcg(w + q) : 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (fresh[q]) fresh[q] = mine[q] & ~atomicOr(w + q, mine[q]);
+        int n = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) n += __popc(fresh[q]);
+        int end = n;
+        for (int off = 1; off < 32; off <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, end, off);
+          if (lane >= off) end += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, end, 31);
+        if (total > 0) {
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&Bf.bdev->need_count, total);
+          at = __shfl_sync(0xffffffffu, at, 0) + end - n;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            for (; fresh[q]; fresh[q] &= fresh[q] - 1u) {
+              const int64_t k = (w0 + q) * 32 + __ffs(fresh[q]) - 1;
+              Bf.need_list[at++] = isB ? (uint32_t)(in.bblk0 + k * bn + bi) | 0x80000000u
+                                       : (uint32_t)(in.ablk0 + (int64_t)bi * bk + k);
+            }
         }
       }
     }
@@ -937,9 +1123,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 4)
 
 }  // namespace
 
-int count_ctas_of(const Inst& in) {
-  return (int)(((int64_t)in.bm * in.bn + kTilesPerCta - 1) / kTilesPerCta);
-}
+int count_ctas_of(const Inst& in) { return units_of(in); }
 
 void set_general(Inst& in, int64_t m, int64_t kd, int64_t n, int64_t lda, int64_t ldb,
                  int64_t ldc, float alpha, float beta, int leaf) {
@@ -960,17 +1144,23 @@ void set_square(Inst& in, int64_t n, int leaf) { set_general(in, n, n, n, n, n, 
 
 size_t plan_layout(Inst* insts, int count, PlanBuffers* b, char* base, bool norm_parts) {
   int64_t tiles = 0, ablks = 0, bblks = 0, kslots = 0, mwords = 0, groups = 0;
-  int prep = 0, cnt = 0, max_bk = 0;
+  int64_t need_a = 0, need_b = 0;
+  int prep = 0, cnt = 0;
+  size_t staged = 0;
   for (int i = 0; i < count; ++i) {
     Inst& in = insts[i];
     const int64_t bm = in.bm, bk = in.bk, bn = in.bn;
-    max_bk = max_bk > (int)bk ? max_bk : (int)bk;
+    const int rows = in.bm < kBandRows ? in.bm : kBandRows;
+    const size_t st = (size_t)(rows + unit_cols(in.bm)) * staged_len(in.bk) * sizeof(Screen);
+    staged = staged > st ? staged : st;
     in.tile0 = tiles;
     in.ablk0 = ablks;
     in.bblk0 = bblks;
     in.kidx0 = kslots;
     in.mask0 = mwords;
     in.grp0 = groups;
+    in.needa0 = need_a;
+    in.needb0 = need_b;
     in.prep0 = prep;
     in.count0 = cnt;
     tiles += bm * bn;
@@ -978,8 +1168,10 @@ size_t plan_layout(Inst* insts, int count, PlanBuffers* b, char* base, bool norm
     bblks += bk * bn;
     kslots += bm * bk * bn;
     mwords += bm * bn * ((bk + 31) / 32);
+    need_a += bm * ((bk + 31) / 32);
+    need_b += bn * ((bk + 31) / 32);
     groups += bm * ((bn + kGroupTiles - 1) / kGroupTiles);
-    prep += prep_ctas_of(in);
+    prep += prep_parts(in);
     cnt += count_ctas_of(in);
   }
   size_t off = 0;
@@ -997,26 +1189,28 @@ size_t plan_layout(Inst* insts, int count, PlanBuffers* b, char* base, bool norm
   t.kslots = kslots;
   t.prep_ctas = prep;
   t.count_ctas = cnt;
-  t.max_bk = max_bk;
-  t.need_words_a = (ablks + 31) / 32;
-  t.need_words_b = (bblks + 31) / 32;
+  t.staged_bytes = staged;
+  t.need_words_a = need_a;
+  t.need_words_b = need_b;
+  int shift = 0;
+  if (cnt > kScanUnits) {
+    shift = 6;
+    while (((int64_t)1 << (2 * shift)) < cnt) ++shift;
+  }
+  t.group_shift = shift;
+  const int nparts = prep > cnt ? prep : cnt;
+  const int ugroups = shift ? (cnt + (1 << shift) - 1) >> shift : 0;
   t.pd = reinterpret_cast<PlanDevice*>(take((size_t)count * sizeof(PlanDevice)));
   t.bdev = reinterpret_cast<BatchDevice*>(take(sizeof(BatchDevice)));
   t.need_bits = reinterpret_cast<uint32_t*>(
       take((size_t)(t.need_words_a + t.need_words_b) * sizeof(uint32_t)));
   t.sA = reinterpret_cast<Screen*>(take((size_t)ablks * sizeof(Screen)));
   t.sBT = reinterpret_cast<Screen*>(take((size_t)bblks * sizeof(Screen)));
-  t.part_a = reinterpret_cast<double*>(take((size_t)prep * sizeof(double)));
-  t.part_b = reinterpret_cast<double*>(take((size_t)prep * sizeof(double)));
-  t.part_S = reinterpret_cast<long long*>(take((size_t)cnt * sizeof(long long)));
-  t.part_kmax = reinterpret_cast<int*>(take((size_t)cnt * sizeof(int)));
-  t.part_ne = reinterpret_cast<int*>(take((size_t)cnt * sizeof(int)));
-  t.part_b1 = reinterpret_cast<ExtSum*>(take((size_t)cnt * sizeof(ExtSum)));
-  t.part_b2 = reinterpret_cast<ExtSum*>(take((size_t)cnt * sizeof(ExtSum)));
-  t.cta_base = reinterpret_cast<int*>(take((size_t)cnt * sizeof(int)));
-  t.ne_cta_base = reinterpret_cast<int*>(take((size_t)cnt * sizeof(int)));
-  t.part_keys = reinterpret_cast<int*>(take((size_t)cnt * kOrderKeys * sizeof(int)));
-  t.key_cta_base = reinterpret_cast<int*>(take((size_t)cnt * kOrderKeys * sizeof(int)));
+  t.part_a = reinterpret_cast<double*>(take((size_t)nparts * sizeof(double)));
+  t.part_b = reinterpret_cast<double*>(take((size_t)nparts * sizeof(double)));
+  t.part = reinterpret_cast<int*>(take((size_t)cnt * kPartInts * sizeof(int)));
+  t.part_bound = reinterpret_cast<ExtSum*>(take((size_t)cnt * 2 * sizeof(ExtSum)));
+  t.group = reinterpret_cast<int*>(take((size_t)ugroups * kPartInts * sizeof(int)));
   t.cnt = reinterpret_cast<int*>(take((size_t)tiles * sizeof(int)));
   t.tile_beg = reinterpret_cast<int*>(take((size_t)tiles * sizeof(int)));
   t.order = reinterpret_cast<int*>(take((size_t)tiles * sizeof(int)));
@@ -1044,46 +1238,58 @@ InstRef make_ref(const Inst* host_insts, const Inst* dev_table, int count) {
   return r;
 }
 
-// The count kernel with its staged screens: 12 * max_bk screens of shared memory.
-cudaError_t launch_count(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
-  const size_t smem = (size_t)(kGroupRows + kTilesPerCta / kGroupRows) * b.max_bk * sizeof(Screen);
+namespace {
+
+// Some instance needs ||A|| ||B|| while its products are counted, or the units
+// are totalled in groups: the prep kernel runs first.
+bool needs_prep(const InstRef& ref, const PlanBuffers& b) {
+  return ref.any_split || b.group_shift != 0;
+}
+
+cudaError_t launch_prep(const InstRef& ref, const PlanBuffers& b, int screens, cudaStream_t s) {
+  return launch_pdl(prep_kernel, dim3(b.prep_ctas), dim3(kPrepThreads), 0, s, ref, b, screens);
+}
+
+cudaError_t launch_count(const InstRef& ref, const PlanBuffers& b, int prepped, int stats,
+                         cudaStream_t s) {
   auto* kern = ref.any_band ? (ref.any_split ? count_kernel<true, true> : count_kernel<false, true>)
                             : (ref.any_split ? count_kernel<true, false> : count_kernel<false, false>);
-  {   // opt in to the largest size once per device and variant (static shared memory counts too)
+  {   // opt in to the largest size once per device and variant
     static bool opted[64][4] = {};
     const int v = (ref.any_band ? 2 : 0) + (ref.any_split ? 1 : 0);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && !opted[dev][v]) {
+    if (dev < 0 || dev >= 64 || !opted[dev][v]) {
       e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)((kGroupRows + kTilesPerCta / kGroupRows) * kMaxBd * sizeof(Screen)));
+                               (int)(16 * staged_len(kMaxBd) * sizeof(Screen)));
       if (e != cudaSuccess) return e;
-      opted[dev][v] = true;
+      if (dev >= 0 && dev < 64) opted[dev][v] = true;
     }
   }
-  return launch_pdl(kern, dim3(b.count_ctas), dim3(kWarpsPerCta * 32), smem, s, ref, b);
+  return launch_pdl(kern, dim3(b.count_ctas), dim3(kCountThreads), b.staged_bytes, s, ref, b, prepped,
+                    stats);
 }
 
+}  // namespace
+
 cudaError_t run_plan_count_half(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
-  // clear the per-instance statistics, the batch-wide order state and the
-  // needed-block bits (laid out back to back, one memset)
-  const size_t clear =
-      reinterpret_cast<const char*>(b.need_bits + b.need_words_a + b.need_words_b) -
-      reinterpret_cast<const char*>(b.pd);
-  cudaError_t e = cudaMemsetAsync(b.pd, 0, clear, s);
-  if (e != cudaSuccess) return e;
-  prep_kernel<<<b.prep_ctas, kPrepThreads, 0, s>>>(ref, b);
-  e = launch_count(ref, b, s);
-  if (e != cudaSuccess) return e;
-  return cudaPeekAtLastError();
+  const int prepped = needs_prep(ref, b) ? 1 : 0;
+  cudaError_t e = prepped ? launch_prep(ref, b, 0, s) : cudaSuccess;
+  return e == cudaSuccess ? launch_count(ref, b, prepped, 0, s) : e;
 }
 
 cudaError_t run_plan_queue_half(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
-  cudaError_t e = launch_pdl(finalize_kernel, dim3(ref.count), dim3(kFinThreads), 0, s, ref, b);
-  if (e == cudaSuccess)
-    e = launch_pdl(fill_kernel, dim3(b.count_ctas), dim3(kWarpsPerCta * 32), 0, s, ref, b);
-  return e;
+  // two CTAs per SM (each reads the totals of all units), four when the totals
+  // are grouped; at most 32 units each
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int want = std::max(1, sms * (b.group_shift ? 4 : 2));
+  const int per = std::min(32, std::max(1, (b.count_ctas + want - 1) / want));
+  const int grid = (b.count_ctas + per - 1) / per + (ref.any_split ? 0 : ref.count);
+  return launch_pdl(fill_kernel, dim3(grid), dim3(kFillThreads), 0, s, ref, b, per,
+                    needs_prep(ref, b) ? 1 : 0);
 }
 
 cudaError_t run_plan(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
@@ -1093,27 +1299,15 @@ cudaError_t run_plan(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
 }
 
 cudaError_t run_plan_count(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
-  const size_t clear =
-      reinterpret_cast<const char*>(b.need_bits + b.need_words_a + b.need_words_b) -
-      reinterpret_cast<const char*>(b.pd);
-  cudaError_t e = cudaMemsetAsync(b.pd, 0, clear, s);
-  if (e != cudaSuccess) return e;
-  prep_kernel<<<b.prep_ctas, kPrepThreads, 0, s>>>(ref, b);
-  e = launch_count(ref, b, s);
-  if (e != cudaSuccess) return e;
-  e = launch_pdl(finalize_kernel, dim3(ref.count), dim3(kFinThreads), 0, s, ref, b);
-  if (e != cudaSuccess) return e;
-  return cudaPeekAtLastError();
+  // the statistics come from the last count CTA: its ticket needs the prep kernel
+  cudaError_t e = launch_prep(ref, b, 0, s);
+  return e == cudaSuccess ? launch_count(ref, b, 1, 1, s) : e;
 }
 
 cudaError_t run_histogram(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
-  const size_t clear =
-      reinterpret_cast<const char*>(b.need_bits + b.need_words_a + b.need_words_b) -
-      reinterpret_cast<const char*>(b.pd);
-  cudaError_t e = cudaMemsetAsync(b.pd, 0, clear, s);
+  cudaError_t e = launch_prep(ref, b, 1, s);
   if (e != cudaSuccess) return e;
-  prep_kernel<<<b.prep_ctas, kPrepThreads, 0, s>>>(ref, b);
-  hist_kernel<<<b.count_ctas, kWarpsPerCta * 32, 0, s>>>(ref, b);
+  hist_kernel<<<b.count_ctas, kHistWarps * 32, 0, s>>>(ref, b);
   return cudaPeekAtLastError();
 }
 

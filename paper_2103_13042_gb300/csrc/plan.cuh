@@ -37,29 +37,23 @@ constexpr int kHistBins = 64;
 // inside a bucket the tiles keep the plan's enumeration order.
 constexpr int kOrderKeys = 12;
 
-// Per-instance statistics; `ticket` and the bins are cleared before each plan.
+// Per-instance statistics; `ticket` and the bins are cleared by the prep kernel.
 struct PlanDevice {
   double norm_a, norm_b, inv_ab;
   double bound1, bound2, valid_ratio;
   long long survivors, flagged;
   int max_tile, nonempty, flag_exp;
-  int ne_base;                              // non-empty tiles of the instances before this one
   unsigned int hist[kHistBins];             // norm-product histogram (tau prediction)
-  int key_tot[kOrderKeys];                  // non-empty tiles per order bucket
-  int key_base[kOrderKeys];                 // first slot of this instance in each bucket
-  unsigned int ticket;                      // prep CTAs of this instance that have finished
+  unsigned int ticket;                      // count CTAs of this instance that have finished
   double bin_sum[kFlagBins];                // surviving products per relative binade
   unsigned long long bin_cnt[kFlagBins];
 };
 
-// Batch-wide state of the longest-first order (cleared before each plan).
+// Batch-wide state.
 struct BatchDevice {
-  int hist[kMaxBd + 2];     // non-empty tiles per survivor count, over all instances
-  int cursor[kMaxBd + 2];   // next slot of each count's bucket in `order`
   int nonempty;             // non-empty tiles over all instances
-  unsigned int ticket;      // finalize CTAs that have finished
   int mul_ticket;           // next slot of `order` to hand out (dynamic multiply schedule)
-  int need_count;           // entries of the needed-block list
+  int need_count;           // entries of the needed-block list (cleared before each fill)
 };
 
 // Multiply schedules: CTAs walk the longest-first order with a fixed
@@ -71,6 +65,8 @@ enum Schedule { kScheduleStatic = 0, kScheduleDynamic = 1, kScheduleGroups = 2 }
 // Tiles per group of the grouped multiply: one block row, kGroupTiles
 // consecutive block columns.
 constexpr int kGroupTiles = 4;
+
+constexpr int kPartInts = 16;   // ints per unit of totals
 
 // Extended-range FP32 sum: value = m * 2^e with an integer exponent.
 struct ExtSum {
@@ -98,8 +94,10 @@ struct Inst {
   int64_t kidx0;        // first k_idx slot
   int64_t mask0;        // first word of the survivor bitmask (bm * bn * ceil(bk / 32) words)
   int64_t grp0;         // first global tile group (bm * ceil(bn / kGroupTiles) groups)
+  int64_t needa0;       // first word of A's part of the needed-block bits (bm * ceil(bk / 32))
+  int64_t needb0;       // first word of B's part (bn * ceil(bk / 32))
   int prep0;            // first CTA of this instance in the prep grid
-  int count0;           // first CTA of this instance in the count and fill grids
+  int count0;           // first unit (CTA of the count grid) of this instance
   double target_rel;    // split modes: relative error target
   double c1;            // split modes: hi-only error coefficient 2u + u^2
   TauScreen T;
@@ -155,21 +153,16 @@ struct PlanBuffers {
   int64_t bblks;       // sum of bk * bn (blocks of B)
   int64_t kslots;      // sum of bm * bk * bn
   int prep_ctas;       // prep grid
-  int count_ctas;      // count and fill grids
-  int max_bk;          // largest bk of the table (the count kernel's shared-memory size)
-  Screen* sA;          // [ablks] screen form of normA, row-major per instance
-  Screen* sBT;         // [bblks] screen form of normB, transposed per instance (J * bk + K)
-  double* part_a;      // [prep_ctas] partial sums of squared norms
+  int count_ctas;      // units: count grid
+  int group_shift;     // log2 units per group of totals (0: no groups)
+  size_t staged_bytes; // the count kernel's shared memory (largest unit of the table)
+  Screen* sA;          // [ablks] histogram: screen form of normA, row-major per instance
+  Screen* sBT;         // [bblks] and of normB, transposed per instance (J * bk + K)
+  double* part_a;      // partial sums of squared norms: per prep CTA, or per unit without prep
   double* part_b;
-  long long* part_S;   // [count_ctas] per-CTA partials of the count kernel
-  int* part_kmax;
-  int* part_ne;
-  ExtSum* part_b1;     // sums of skipped relative products
-  ExtSum* part_b2;     // sums of their per-tile squares
-  int* cta_base;       // [count_ctas] first k_idx slot of the CTA's tiles
-  int* ne_cta_base;    // [count_ctas] non-empty tiles of the instance's earlier CTAs
-  int* part_keys;      // [count_ctas * kOrderKeys] non-empty tiles of the CTA per bucket
-  int* key_cta_base;   // [count_ctas * kOrderKeys] the instance's earlier CTAs' tiles per bucket
+  int* part;           // [units * kPartInts] totals of each unit
+  ExtSum* part_bound;  // [units * 2] sums of skipped products, and of their per-tile squares
+  int* group;          // [groups * kPartInts] totals of each group of units
   int* cnt;            // [tiles] survivors per tile
   int* tile_beg;       // [tiles] absolute first k_idx slot of the tile
   int* order;          // [tiles] global ids: the non-empty tiles, most survivors first, then
@@ -177,12 +170,13 @@ struct PlanBuffers {
   uint16_t* k_idx;     // [kslots] surviving k per tile, increasing (bit 15: split triple)
   int* tile_inst;      // [tiles] instance of each global output tile
   uint32_t* surv_mask; // survivors of each tile, 32 k per word (tile t = i*bn + j of an instance)
-  uint32_t* need_bits; // [words_a + words_b] bit g: block g of A (first part) / B (second) is used
+  uint32_t* need_bits; // [words_a + words_b] used blocks, 32 k per word: row i of A at
+                       // needa0 + i * ceil(bk / 32), column j of B (second part) at needb0 + ...
   uint32_t* need_list; // [ablks + bblks] used blocks, each once: g (A) or g | 2^31 (B)
   int64_t need_words_a;   // 32-bit words of the A part of need_bits
   int64_t need_words_b;
   void* norm_part;     // tensor modes with an output norm map: per-tile partial sums
-  PlanDevice* pd;      // [instances]; pd, bdev and need_bits are contiguous (one memset)
+  PlanDevice* pd;      // [instances]
   BatchDevice* bdev;
 };
 
@@ -191,8 +185,7 @@ __device__ __forceinline__ int inst_of(const InstRef& r, const PlanBuffers& b, i
   return r.count <= 1 ? 0 : b.tile_inst[g];
 }
 
-// Grid sizes of the plan kernels for one instance.
-int prep_ctas_of(const Inst& in);
+// Units of one instance (CTAs of the count grid).
 int count_ctas_of(const Inst& in);
 
 // Sets the shape fields of a square n x n instance (alpha = 1, beta = 0).
@@ -216,7 +209,7 @@ InstRef make_ref(const Inst* host_insts, const Inst* dev_table, int count);
 cudaError_t run_plan(const InstRef& ref, const PlanBuffers& b, cudaStream_t s);
 
 // run_plan in two halves: the first ends once every tile's survivor count is
-// known (cnt), the second builds the queues and the order.
+// known (cnt), the second builds the queues, the order and the statistics.
 cudaError_t run_plan_count_half(const InstRef& ref, const PlanBuffers& b, cudaStream_t s);
 cudaError_t run_plan_queue_half(const InstRef& ref, const PlanBuffers& b, cudaStream_t s);
 
