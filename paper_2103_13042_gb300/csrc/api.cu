@@ -156,6 +156,11 @@ spamm_status_t engine_free(Engine& e) {
 
 namespace {
 
+// The multiply writes the empty tiles too: no zero-fill on the side stream.
+bool own_zeros(const Engine& e, const InstRef& ref) {
+  return e.precision == SPAMM_FP32 && simt_writes_zeros(ref, e.buf, e.leaf);
+}
+
 // The multiply of the non-empty tiles (operand rounding first in tensor modes).
 cudaError_t multiply_nonempty(Engine& e, const InstRef& ref, int32_t* status, cudaStream_t s,
                               cudaEvent_t after_round) {
@@ -165,7 +170,7 @@ cudaError_t multiply_nonempty(Engine& e, const InstRef& ref, int32_t* status, cu
   if (err != cudaSuccess) return err;
   if (e.precision == SPAMM_FP32) {
     if (after_round) err = cudaEventRecord(after_round, s);
-    if (err == cudaSuccess) err = launch_multiply_simt(ref, e.buf, e.leaf, e.schedule, s);
+    if (err == cudaSuccess) err = launch_multiply_simt(ref, e.buf, e.leaf, e.schedule, own_zeros(e, ref), s);
   } else {
     err = launch_quantize(e.precision, e.leaf, ref, e.buf, e.img, s);
     if (err == cudaSuccess && after_round) err = cudaEventRecord(after_round, s);
@@ -180,6 +185,7 @@ cudaError_t multiply_nonempty(Engine& e, const InstRef& ref, int32_t* status, cu
 
 cudaError_t engine_multiply(Engine& e, const InstRef& ref, int32_t* status, cudaStream_t s,
                             cudaEvent_t after_round) {
+  if (own_zeros(e, ref)) return multiply_nonempty(e, ref, status, s, after_round);
   // empty tiles (zeros, HBM-write bound) on the side stream, overlapped with
   // the rounding and multiply of the non-empty tiles (disjoint parts of C)
   cudaError_t err = cudaEventRecord(e.fork, s);
@@ -193,6 +199,11 @@ cudaError_t engine_multiply(Engine& e, const InstRef& ref, int32_t* status, cuda
 
 cudaError_t engine_plan_multiply(Engine& e, const InstRef& ref, int32_t* status, cudaStream_t s,
                                  cudaEvent_t after_plan, cudaEvent_t after_round) {
+  if (own_zeros(e, ref)) {
+    cudaError_t err = run_plan(ref, e.buf, s);
+    if (err == cudaSuccess && after_plan) err = cudaEventRecord(after_plan, s);
+    return err == cudaSuccess ? multiply_nonempty(e, ref, status, s, after_round) : err;
+  }
   // The zeros of the empty tiles (HBM-write bound) overlap the rounding and the
   // multiply; one big instance, whose zeros take longest, starts them as soon as the
   // counting half is done.  Elsewhere that costs more than it gains: the zeros slow

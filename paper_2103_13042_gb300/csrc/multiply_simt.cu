@@ -1,97 +1,174 @@
 // Plain FP32 multiply on the SIMT cores (Section 3.3's FP32 multiplication
 // kernel; the baseline the tensor-core modes are measured against).
 //
-// Persistent CTAs walk the non-empty tiles of all instances (most survivors
-// first) with a grid stride; the caller writes the empty tiles with the
-// coalesced zero-fill kernel.  A non-empty tile (i, j) streams its
-// surviving k in 32-wide slices of the inner dimension: the A slice
-// A[i, k][:, s:s+32] is stored transposed and the B slice B[k, j][s:s+32, :]
-// as is, both in shared memory, double buffered through registers so the next
-// slice's global loads overlap the current slice's FMAs.  Each of the 256
-// threads keeps a (leaf/16) x (leaf/16) register tile of C and accumulates
-// in FP32 FMA over every surviving k.  Empty tiles are written as zeros with
-// coalesced float4 stores (beta = 0) by that kernel.
+// One persistent CTA per SM holds several independent groups of warps; a group
+// multiplies one tile at a time: 1 warp at leaf 32, 2 at 64, 8 at 128.  The
+// non-empty tiles of all instances (most survivors first) are dealt over the SMs
+// with a fixed stride; inside an SM its groups take them from a shared-memory
+// counter, so a group that met short tiles takes more of them (a fixed deal to
+// every group left a third of the warps idle on average).  A warp owns 32 x 64
+// entries of the tile (32 x 32 at leaf 32), a thread 8 rows x 8 (4) columns: rows
+// ty + 4 u, columns 4 tx .. 4 tx + 3 and 32 further on, so that the distinct
+// addresses of every shared-memory read fall into different banks.
+// The surviving k are streamed in slices of 16 of the inner dimension through a
+// three-stage ring filled by asynchronous copies (16 bytes where rows are
+// aligned, else 4; entries outside the matrix are filled with zeros), A as rows,
+// B as rows: neither is transposed.  The products accumulate in FP32 FMA over the
+// surviving k in increasing order, two columns per instruction (packed
+// fma.rn.f32x2: the same FP32 rate, half the issue slots).  Bound by the FP32 pipe
+// on dense skip sets: 45, 48 and 41 TFLOP/s at leaf 32, 64 and 128 (n = 4096,
+// 30% of the triples; 256 threads per tile with transposed A slices: 19, 30 and
+// 29), 41 at leaf 64 with unaligned rows (26).
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace spamm {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kSlice = 32;
+constexpr int kSlice = 16;
+constexpr int kStages = 3;
+constexpr int kLdA = kSlice + 4;   // floats per staged row of A: 16-byte rows, four rows apart in
+                                   // different banks
+// Outputs up to this size: the multiply writes the empty tiles itself (a second
+// kernel on a side stream costs more than their stores)
+constexpr int64_t kOwnZeroBytes = (int64_t)64 << 20;
 
 template <int LEAF>
 struct SimtTile {
-  static constexpr int TM = LEAF / 16;                    // C rows (and cols) per thread
-  static constexpr int kLoadsA = LEAF * kSlice / 4 / kThreads;  // float4 per thread per slice
+  static constexpr int kWarps = LEAF == 128 ? 8 : (LEAF == 64 ? 2 : 1);
+  static constexpr int kThreads = 32 * kWarps;
+  static constexpr int TN = LEAF == 32 ? 4 : 8;                      // columns per thread
+  static constexpr int kWarpCols = 8 * TN;                           // 64, 32 at leaf 32
+  static constexpr int kStageFloats = LEAF * kLdA + kSlice * LEAF;   // A rows, then B rows
+  static constexpr size_t kSmem = (size_t)kStages * kStageFloats * sizeof(float);
+  static constexpr int kPieces = LEAF * kSlice / 4 / kThreads;       // 16-byte pieces per thread
+    // groups per CTA, one CTA per SM: 168 registers per thread at leaf 32 and 64 (8 and 16
+  // groups at 128 registers spill: 37 and 42 TFLOP/s against 48 and 45)
+  static constexpr int kGroups = LEAF == 128 ? 1 : (LEAF == 64 ? 6 : 12);
+  static constexpr int kCtaThreads = kGroups * kThreads;
+  static constexpr size_t kCtaSmem = kGroups * kSmem;
+  static_assert(kCtaSmem <= 227 * 1024 && kCtaThreads <= 1024 && kGroups <= 15, "CTA shape");
 };
 
-// Loads 4 consecutive floats of row r, columns c..c+3 of a rows x cols matrix
-// with leading dimension ld, zero outside it.
-__device__ __forceinline__ float4 load4(const float* __restrict__ M, int64_t rows, int64_t cols,
-                                        int64_t ld, int64_t r, int64_t c, bool vec) {
-  if (r >= rows) return make_float4(0.f, 0.f, 0.f, 0.f);
-  const float* p = M + r * ld + c;
-  if (vec && c + 3 < cols) return __ldg(reinterpret_cast<const float4*>(p));
-  float4 v;
-  v.x = c < cols ? __ldg(p) : 0.f;
-  v.y = c + 1 < cols ? __ldg(p + 1) : 0.f;
-  v.z = c + 2 < cols ? __ldg(p + 2) : 0.f;
-  v.w = c + 3 < cols ? __ldg(p + 3) : 0.f;
-  return v;
+// Copies 16 (4) bytes, `bytes` of them from src and the rest zeros.
+__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
 }
 
-// TM consecutive floats from 16-byte (TM >= 4) or 8-byte (TM = 2) aligned shared memory.
-template <int TM>
-__device__ __forceinline__ void read_row(const float* p, float* out) {
-  if constexpr (TM >= 4) {
+// Stages rows [r, r + ROWS) x columns [c, c + COLS) of a rows x cols matrix with
+// leading dimension ld as ROWS rows of LD floats.
+template <int ROWS, int COLS, int LD, int THREADS>
+__device__ __forceinline__ void stage(float* dst, const float* __restrict__ M, int64_t rows,
+                                      int64_t cols, int64_t ld, int64_t r, int64_t c, bool vec) {
+  constexpr int kPerRow = COLS / 4;
+  const int tid = threadIdx.x % THREADS;
+  if (vec) {
 #pragma unroll
-    for (int v = 0; v < TM; v += 4) {
-      const float4 x = *reinterpret_cast<const float4*>(p + v);
-      out[v] = x.x; out[v + 1] = x.y; out[v + 2] = x.z; out[v + 3] = x.w;
+    for (int l = 0; l < ROWS * kPerRow / THREADS; ++l) {
+      const int p = tid + l * THREADS, pr = p / kPerRow, pc = p % kPerRow * 4;
+      const int64_t left = r + pr < rows ? cols - (c + pc) : 0;
+      const int bytes = left >= 4 ? 16 : (left > 0 ? (int)left * 4 : 0);
+      copy16(dst + pr * LD + pc, bytes ? M + (r + pr) * ld + c + pc : M, bytes);
     }
   } else {
-    const float2 x = *reinterpret_cast<const float2*>(p);
-    out[0] = x.x; out[1] = x.y;
+#pragma unroll 4
+    for (int l = 0; l < ROWS * COLS / THREADS; ++l) {
+      const int p = tid + l * THREADS, pr = p / COLS, pc = p % COLS;
+      const bool in = r + pr < rows && c + pc < cols;
+      copy4(dst + pr * LD + pc, in ? M + (r + pr) * ld + c + pc : M, in ? 4 : 0);
+    }
   }
 }
 
-template <int TM>
-__device__ __forceinline__ void write_row(float* p, const float* v) {
-  if constexpr (TM >= 4) {
-#pragma unroll
-    for (int q = 0; q < TM; q += 4)
-      *reinterpret_cast<float4*>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-  } else {
-    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-  }
+// Two FP32 FMAs, each rounded to nearest.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t pair(float x, float y) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ void unpair(uint64_t d, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(d));
 }
 
+// The barrier of one group (hardware barrier 1 + group).
 template <int LEAF>
-__global__ void __launch_bounds__(kThreads) simt_kernel(InstRef R, PlanBuffers Bf, int dynamic) {
-  pdl_wait();
-  using T = SimtTile<LEAF>;
-  constexpr int TM = T::TM;
-  constexpr int kLoads = T::kLoadsA;
-  // A slice transposed: sA[buf][s][r] (r = row within the leaf), B slice sB[buf][s][c]
-  extern __shared__ __align__(16) float smem[];
-  float (*sA)[kSlice][LEAF + 4] = reinterpret_cast<float (*)[kSlice][LEAF + 4]>(smem);
-  float (*sB)[kSlice][LEAF + 4] =
-      reinterpret_cast<float (*)[kSlice][LEAF + 4]>(smem + 2 * kSlice * (LEAF + 4));
+__device__ __forceinline__ void tile_sync(int group) {
+  if constexpr (SimtTile<LEAF>::kWarps == 1)
+    __syncwarp();
+  else
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(SimtTile<LEAF>::kThreads) : "memory");
+}
 
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int64_t ne = Bf.bdev->nonempty;   // empty tiles are zero-filled by another kernel
-
-  __shared__ int s_next;
-  for (int64_t w = blockIdx.x;; w += gridDim.x) {
-    if (dynamic) {   // next tile from the global counter (its use ends at the loop's barrier)
-      if (tid == 0) s_next = atomicAdd(&Bf.bdev->mul_ticket, 1);
-      __syncthreads();
-      w = s_next;
+// An empty tile of an instance with beta = 0: zeros, and the tile's norm.
+template <int LEAF>
+__device__ __forceinline__ void zero_tile(const Inst& in, int64_t t, int tid) {
+  constexpr int kThreads = SimtTile<LEAF>::kThreads;
+  const int i = (int)(t / in.bn), j = (int)(t - (int64_t)i * in.bn);
+  const int64_t r0 = (int64_t)i * LEAF, c0 = (int64_t)j * LEAF;
+  const int rows = (int)min((int64_t)LEAF, in.m - r0), cols = (int)min((int64_t)LEAF, in.n - c0);
+  float* p = in.C + r0 * in.ldc + c0;
+  if ((in.ldc & 3) == 0 && (cols & 3) == 0) {
+    constexpr int kPerRow = LEAF / 4;
+    for (int x = tid; x < rows * kPerRow; x += kThreads) {
+      const int r = x / kPerRow, c = x % kPerRow * 4;
+      if (c < cols)
+        *reinterpret_cast<float4*>(p + r * in.ldc + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (w >= ne) break;
+  } else {
+    for (int x = tid; x < rows * LEAF; x += kThreads)
+      if (x % LEAF < cols) p[x / LEAF * in.ldc + x % LEAF] = 0.0f;
+  }
+  if (in.nC && tid == 0) in.nC[t] = 0.0;
+}
+
+// zeros: also write the tiles without survivors (every instance has beta = 0).
+template <int LEAF>
+__global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
+    simt_kernel(InstRef R, PlanBuffers Bf, int dynamic, int zeros) {
+  using T = SimtTile<LEAF>;
+  constexpr int TN = T::TN, kHalves = TN / 4;
+  extern __shared__ __align__(16) float smem_all[];
+  __shared__ int s_taken;               // tiles of this SM handed to its groups
+  __shared__ int s_next[T::kGroups];
+  __shared__ SumSq s_norm[T::kGroups][T::kWarps];
+  const int group = threadIdx.x / T::kThreads, tid = threadIdx.x % T::kThreads;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int tx = lane & 7, ty = lane >> 3;
+  constexpr int kWarpsAcross = LEAF / T::kWarpCols;
+  const int wr = warp / kWarpsAcross * 32, wc = warp % kWarpsAcross * T::kWarpCols;
+  float* smem = smem_all + (size_t)group * kStages * T::kStageFloats;
+  if (threadIdx.x == 0) s_taken = 0;
+  __syncthreads();
+  pdl_wait();
+  const int64_t ne = Bf.bdev->nonempty, all = zeros ? Bf.tiles : ne;
+
+  for (;;) {
+    if (tid == 0)   // dynamic: from the table's counter (it hands out non-empty tiles only)
+      s_next[group] = dynamic ? atomicAdd(&Bf.bdev->mul_ticket, 1) : atomicAdd(&s_taken, 1);
+    tile_sync<LEAF>(group);   // also: the previous tile's readers are done with the ring
+    const int64_t w = dynamic ? s_next[group] : blockIdx.x + (int64_t)s_next[group] * gridDim.x;
+    if (w >= (dynamic ? ne : all)) break;
     const int g = Bf.order[w];
     const Inst& in = R.at(inst_of(R, Bf, g));
+    if (w >= ne) {
+      zero_tile<LEAF>(in, g - in.tile0, tid);
+      tile_sync<LEAF>(group);   // s_next is rewritten next
+      continue;
+    }
+    const int beg = Bf.tile_beg[g], cnt = Bf.cnt[g];
     const int bn = in.bn;
     const int64_t m = in.m, kd = in.kd, n = in.n;
     const int64_t lda = in.lda, ldb = in.ldb, ldc = in.ldc;
@@ -99,107 +176,138 @@ __global__ void __launch_bounds__(kThreads) simt_kernel(InstRef R, PlanBuffers B
     const float* __restrict__ B = in.B;
     float* __restrict__ C = in.C;
     const bool vec_a = (lda % 4) == 0, vec_b = (ldb % 4) == 0, vec_c = (ldc % 4) == 0;
-    const uint16_t* __restrict__ k_idx = Bf.k_idx;
+    const uint16_t* __restrict__ k_idx = Bf.k_idx + beg;
     const int64_t t = g - in.tile0;
     const int i = (int)(t / bn), j = (int)(t % bn);
-    const int beg = Bf.tile_beg[g], end = beg + Bf.cnt[g];
     const int64_t r0 = (int64_t)i * LEAF, c0 = (int64_t)j * LEAF;
 
-    float acc[TM][TM];
+    uint64_t acc[8][TN / 2];
 #pragma unroll
-    for (int a = 0; a < TM; ++a)
+    for (int u = 0; u < 8; ++u)
 #pragma unroll
-      for (int b = 0; b < TM; ++b) acc[a][b] = 0.f;
+      for (int v = 0; v < TN / 2; ++v) acc[u][v] = 0ull;
 
-    const int nslices = (end - beg) * (LEAF / kSlice);
-    float4 ra[kLoads], rb[kLoads];
-
-    // slice q -> (k, s0): A rows r0.., cols k*LEAF + s0..; B rows k*LEAF + s0.., cols c0..
+    constexpr int kPerK = LEAF / kSlice;
+    const int nslices = cnt * kPerK;
+    int k_ahead = __ldg(k_idx) & 0x3ff;   // the inner block of the next slice to stage
+    // a tile inside the matrix: this thread's pieces (or entries) of a slice start at
+    // fixed distances from two pointers
+    const bool inside = r0 + LEAF <= m && c0 + LEAF <= n;
+    constexpr int kThr = T::kThreads, kPc = kSlice / 4, kPl = LEAF / 4;
+    const int pa = vec_a ? tid / kPc : tid / kSlice, ca = vec_a ? tid % kPc * 4 : tid % kSlice;
+    const int pb = vec_b ? tid / kPl : tid / LEAF, cb = vec_b ? tid % kPl * 4 : tid % LEAF;
+    const float* base_a = A + (r0 + pa) * lda + ca;
+    const float* base_b = B + (int64_t)pb * ldb + c0 + cb;
     auto fetch = [&](int q) {
-      const int k = k_idx[beg + q / (LEAF / kSlice)] & 0x3ff;
-      const int s0 = (q % (LEAF / kSlice)) * kSlice;
+      if (q < nslices) {
+        const int64_t k0 = (int64_t)k_ahead * LEAF + (q % kPerK) * kSlice;
+        float* s = smem + (q % kStages) * T::kStageFloats;
+        float* sb = s + LEAF * kLdA;
+        if (inside && k0 + kSlice <= kd) {
+          const float* src = base_a + k0;
+          if (vec_a) {
+            constexpr int kStep = kThr / kPc;
 #pragma unroll
-      for (int l = 0; l < kLoads; ++l) {
-        const int e = (tid + l * kThreads) * 4;      // element index in the slice
-        // A slice: LEAF rows x 32 cols, float4 along the columns
-        const int ar = e / kSlice, ac = e % kSlice;
-        ra[l] = load4(A, m, kd, lda, r0 + ar, (int64_t)k * LEAF + s0 + ac, vec_a);
-        // B slice: 32 rows x LEAF cols, float4 along the columns
-        const int br = e / LEAF, bc = e % LEAF;
-        rb[l] = load4(B, kd, n, ldb, (int64_t)k * LEAF + s0 + br, c0 + bc, vec_b);
-      }
-    };
-    auto stash = [&](int buf) {
-#pragma unroll
-      for (int l = 0; l < kLoads; ++l) {
-        const int e = (tid + l * kThreads) * 4;
-        const int ar = e / kSlice, ac = e % kSlice;
-        sA[buf][ac + 0][ar] = ra[l].x;
-        sA[buf][ac + 1][ar] = ra[l].y;
-        sA[buf][ac + 2][ar] = ra[l].z;
-        sA[buf][ac + 3][ar] = ra[l].w;
-        const int br = e / LEAF, bc = e % LEAF;
-        *reinterpret_cast<float4*>(&sB[buf][br][bc]) = rb[l];
-      }
-    };
-
-    fetch(0);
-    __syncthreads();  // previous tile's readers are done with both buffers
-    stash(0);
-    __syncthreads();
-    for (int q = 0; q < nslices; ++q) {
-      const int buf = q & 1;
-      if (q + 1 < nslices) fetch(q + 1);
+            for (int l = 0; l < LEAF / kStep; ++l, src += kStep * lda)
+              copy16(s + (pa + l * kStep) * kLdA + ca, src, 16);
+          } else {
+            constexpr int kStep = kThr / kSlice;
 #pragma unroll 8
-      for (int s = 0; s < kSlice; ++s) {
-        float a[TM], b[TM];
-        read_row<TM>(&sA[buf][s][ty * TM], a);
-        read_row<TM>(&sB[buf][s][tx * TM], b);
+            for (int l = 0; l < LEAF / kStep; ++l, src += kStep * lda)
+              copy4(s + (pa + l * kStep) * kLdA + ca, src, 4);
+          }
+          src = base_b + k0 * ldb;
+          if (vec_b) {
+            constexpr int kStep = kThr / kPl;
 #pragma unroll
-        for (int u = 0; u < TM; ++u)
-#pragma unroll
-          for (int v = 0; v < TM; ++v) acc[u][v] = __fmaf_rn(a[u], b[v], acc[u][v]);
+            for (int l = 0; l < kSlice / kStep; ++l, src += kStep * ldb)
+              copy16(sb + (pb + l * kStep) * LEAF + cb, src, 16);
+          } else {
+            constexpr int kStep = kThr / LEAF;
+#pragma unroll 8
+            for (int l = 0; l < kSlice / kStep; ++l, src += kStep * ldb)
+              copy4(sb + (pb + l * kStep) * LEAF + cb, src, 4);
+          }
+        } else {
+          stage<LEAF, kSlice, kLdA, kThr>(s, A, m, kd, lda, r0, k0, vec_a);
+          stage<kSlice, LEAF, LEAF, kThr>(sb, B, kd, n, ldb, k0, c0, vec_b);
+        }
+        if (q % kPerK == kPerK - 1 && q + 1 < nslices) k_ahead = __ldg(k_idx + q / kPerK + 1) & 0x3ff;
       }
-      if (q + 1 < nslices) stash(buf ^ 1);
-      __syncthreads();
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int q = 0; q < kStages - 1; ++q) fetch(q);
+    for (int q = 0; q < nslices; ++q) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+      tile_sync<LEAF>(group);   // slice q is here; slice q - 1 has been read
+      fetch(q + kStages - 1);
+      const float* sa = smem + (q % kStages) * T::kStageFloats + (wr + ty) * kLdA;
+      const float* sb = smem + (q % kStages) * T::kStageFloats + LEAF * kLdA + wc + tx * 4;
+#pragma unroll
+      for (int s2 = 0; s2 < kSlice; s2 += 2) {
+        float2 a[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a[u] = *reinterpret_cast<const float2*>(sa + 4 * u * kLdA + s2);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          uint64_t b[TN / 2];
+#pragma unroll
+          for (int h = 0; h < kHalves; ++h) {
+            const ulonglong2 x =
+                *reinterpret_cast<const ulonglong2*>(sb + (s2 + e) * LEAF + 32 * h);
+            b[2 * h] = x.x;
+            b[2 * h + 1] = x.y;
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const float f = e == 0 ? a[u].x : a[u].y;
+            const uint64_t aa = pair(f, f);
+#pragma unroll
+            for (int v = 0; v < TN / 2; ++v) acc[u][v] = fma2(aa, b[v], acc[u][v]);
+          }
+        }
+      }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
 
     // epilogue: C = alpha * acc + beta * C (the old C is read only when beta != 0)
     const float alpha = in.alpha, beta = in.beta;
+    SumSq ss = sumsq_empty();
 #pragma unroll
-    for (int u = 0; u < TM; ++u) {
-      const int64_t r = r0 + ty * TM + u;
-      const int64_t c = c0 + tx * TM;
-      float* p = C + r * ldc + c;
+    for (int u = 0; u < 8; ++u) {
+      const int64_t r = r0 + wr + ty + 4 * u;
       const bool row_in = r < m;
-      if (beta != 0.0f && row_in) {
+      float x[TN];
 #pragma unroll
-        for (int q = 0; q < TM; ++q)
-          acc[u][q] = c + q < n ? __fmaf_rn(beta, p[q], __fmul_rn(alpha, acc[u][q])) : 0.0f;
-      } else {
+      for (int v = 0; v < TN / 2; ++v) unpair(acc[u][v], x[2 * v], x[2 * v + 1]);
 #pragma unroll
-        for (int q = 0; q < TM; ++q) acc[u][q] = __fmul_rn(alpha, acc[u][q]);
+      for (int h = 0; h < kHalves; ++h) {
+        const int64_t c = c0 + wc + 32 * h + tx * 4;
+        float* p = C + r * ldc + c;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float& y = x[4 * h + q];
+          y = __fmul_rn(alpha, y);
+          if (beta != 0.0f) y = row_in && c + q < n ? __fmaf_rn(beta, p[q], y) : 0.0f;
+        }
+        if (!row_in) continue;
+        if (vec_c && c + 3 < n) {
+          *reinterpret_cast<float4*>(p) = make_float4(x[4 * h], x[4 * h + 1], x[4 * h + 2], x[4 * h + 3]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (c + q < n) p[q] = x[4 * h + q];
+        }
       }
-      if (!row_in) continue;
-      if (vec_c && c + TM - 1 < n) {
-        write_row<TM>(p, acc[u]);
-      } else {
+      if (in.nC) {   // C's norm map for a chained product: the row's stored values
 #pragma unroll
-        for (int q = 0; q < TM; ++q)
-          if (c + q < n) p[q] = acc[u][q];
+        for (int q = 0; q < TN; ++q)
+          if (!(row_in && c0 + wc + 32 * (q / 4) + tx * 4 + q % 4 < n)) x[q] = 0.0f;
+        sumsq_group<TN>(ss, x);
       }
     }
-    if (in.nC) {   // C's norm map for a chained product: the tile's stored values
-      float v[TM * TM];
-#pragma unroll
-      for (int u = 0; u < TM; ++u)
-#pragma unroll
-        for (int q = 0; q < TM; ++q) {
-          const bool inside = r0 + ty * TM + u < m && c0 + tx * TM + q < n;
-          v[u * TM + q] = inside ? acc[u][q] : 0.0f;
-        }
-      SumSq ss = sumsq_empty();
-      sumsq_group<TM * TM>(ss, v);
+    if (in.nC) {
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
         const float h = __shfl_xor_sync(0xffffffffu, ss.hi, off);
@@ -207,42 +315,61 @@ __global__ void __launch_bounds__(kThreads) simt_kernel(InstRef R, PlanBuffers B
         const int e = __shfl_xor_sync(0xffffffffu, ss.e, off);
         sumsq_merge_any(ss, h, l, e);
       }
-      __shared__ SumSq s_norm[kThreads / 32];
-      if ((tid & 31) == 0) s_norm[tid / 32] = ss;
-      __syncthreads();
+      if (lane == 0) s_norm[group][warp] = ss;
+      tile_sync<LEAF>(group);
       if (tid == 0) {
-        SumSq tot = s_norm[0];
-        for (int w = 1; w < kThreads / 32; ++w) sumsq_merge_any(tot, s_norm[w].hi, s_norm[w].lo, s_norm[w].e);
+        SumSq tot = s_norm[group][0];
+        for (int w2 = 1; w2 < T::kWarps; ++w2) {
+          const SumSq o = s_norm[group][w2];
+          sumsq_merge_any(tot, o.hi, o.lo, o.e);
+        }
         in.nC[t] = sumsq_sqrt(tot);
       }
     }
   }
+  if (!dynamic) return;
+  // dynamic order: the empty tiles are dealt with a fixed stride
+  for (int64_t w = ne + blockIdx.x * T::kGroups + group; w < all; w += (int64_t)gridDim.x * T::kGroups) {
+    const int g = Bf.order[w];
+    const Inst& in = R.at(inst_of(R, Bf, g));
+    zero_tile<LEAF>(in, g - in.tile0, tid);
+  }
 }
 
 template <int LEAF>
-cudaError_t launch(const InstRef& ref, const PlanBuffers& b, int schedule, cudaStream_t s) {
-  constexpr size_t smem = 4 * kSlice * (LEAF + 4) * sizeof(float);
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncSetAttribute(simt_kernel<LEAF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, simt_kernel<LEAF>, kThreads, smem);
-  const int grid = (int)std::max<int64_t>(
-      1, std::min<int64_t>(b.tiles, (int64_t)sms * std::max(1, per_sm)));
-  cudaError_t e = launch_pdl(simt_kernel<LEAF>, dim3(grid), dim3(kThreads), smem, s, ref, b,
-                             (int)(schedule == kScheduleDynamic));
+cudaError_t launch(const InstRef& ref, const PlanBuffers& b, int schedule, bool zeros,
+                   cudaStream_t s) {
+  using T = SimtTile<LEAF>;
+  static int sms[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  return cudaPeekAtLastError();
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (sms[dev] == 0) {
+    int count = 0;
+    e = cudaFuncSetAttribute(simt_kernel<LEAF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)T::kCtaSmem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    sms[dev] = std::max(1, count);
+  }
+  const int grid = (int)std::min<int64_t>(b.tiles, (int64_t)sms[dev]);
+  return launch_pdl(simt_kernel<LEAF>, dim3(grid), dim3(T::kCtaThreads), T::kCtaSmem, s, ref, b,
+                    (int)(schedule == kScheduleDynamic), zeros ? 1 : 0);
 }
 
 }  // namespace
 
+bool simt_writes_zeros(const InstRef& ref, const PlanBuffers& b, int leaf) {
+  return !ref.any_scaled && b.tiles * leaf * leaf * (int64_t)sizeof(float) <= kOwnZeroBytes;
+}
+
 cudaError_t launch_multiply_simt(const InstRef& ref, const PlanBuffers& b, int leaf,
-                                 int schedule, cudaStream_t s) {
+                                 int schedule, bool zeros, cudaStream_t s) {
   switch (leaf) {
-    case 32: return launch<32>(ref, b, schedule, s);
-    case 64: return launch<64>(ref, b, schedule, s);
-    case 128: return launch<128>(ref, b, schedule, s);
+    case 32: return launch<32>(ref, b, schedule, zeros, s);
+    case 64: return launch<64>(ref, b, schedule, zeros, s);
+    case 128: return launch<128>(ref, b, schedule, zeros, s);
     default: return cudaErrorInvalidValue;
   }
 }

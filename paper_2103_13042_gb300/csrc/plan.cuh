@@ -258,8 +258,13 @@ cudaError_t launch_normmap_jobs(const NormJob* dev_jobs, int n_vec, int units_ve
                                 cudaStream_t side = nullptr, cudaEvent_t fork = nullptr,
                                 cudaEvent_t join = nullptr);
 
+// FP32 multiply of the non-empty tiles; zeros: of the empty ones too (where
+// simt_writes_zeros says so).
 cudaError_t launch_multiply_simt(const InstRef& ref, const PlanBuffers& b, int leaf,
-                                 int schedule, cudaStream_t s);
+                                 int schedule, bool zeros, cudaStream_t s);
+// Every instance has beta = 0 and the outputs are small: no kernel of their own
+// for the empty tiles.
+bool simt_writes_zeros(const InstRef& ref, const PlanBuffers& b, int leaf);
 
 // Per-tile partial sums of squares of the tensor-core epilogue (output norm
 // maps): one per epilogue warp of a tile, merged by launch_norm_out_finish.

@@ -104,7 +104,7 @@ spamm_status_t band_error(Engine& e, const double* nA, const double* nB, const f
   const InstRef ref = make_ref(e.insts.data(), nullptr, 1);
   cudaError_t ce = run_plan(ref, e.buf, s);
   in.band = 0;
-  if (ce == cudaSuccess) ce = launch_multiply_simt(ref, e.buf, e.leaf, kScheduleStatic, s);
+  if (ce == cudaSuccess) ce = launch_multiply_simt(ref, e.buf, e.leaf, kScheduleStatic, false, s);
   if (ce == cudaSuccess) ce = launch_zero_empty_tiles(ref, e.buf, e.leaf, s);
   if (ce != cudaSuccess) return cuda_fail();
   double norm = 0.0;
