@@ -523,6 +523,38 @@ __device__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepp
 // 128 bytes of a shared-memory wavefront.
 __host__ __device__ __forceinline__ int staged_len(int bk) { return ((bk + 31) & ~31) + 2; }
 
+// A unit's screens into shared memory (rows of A, then columns of B, their
+// exponents relative to eT), by kCountThreads threads.
+__device__ __forceinline__ void stage_unit(const Inst& in, const Unit& u, Screen* sa, Screen* sb,
+                                           int eT) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int bk = in.bk, bn = in.bn, len = staged_len(bk), kpad = len - 2;
+  const double* __restrict__ nA = in.nA;
+  const double* __restrict__ nB = in.nB;
+  for (int x = warp; x < u.rows; x += kCountWarps) {
+    const double* src = nA + (int64_t)(u.r0 + x) * bk;
+#pragma unroll 8
+    for (int k = lane; k < kpad; k += 32) sa[x * len + k] = test_screen(k < bk ? src[k] : 0.0);
+  }
+  if (u.cols == 4) {   // lanes over (k, column): whole 32-byte sectors
+#pragma unroll 8
+    for (int x = tid; x < 4 * kpad; x += kCountThreads) {
+      const int k = x >> 2, c = x & 3;
+      Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
+      b.e -= eT;
+      sb[c * len + k] = b;
+    }
+  } else {
+    for (int k = tid; k < kpad; k += kCountThreads)
+#pragma unroll 4
+      for (int c = 0; c < u.cols; ++c) {
+        Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
+        b.e -= eT;
+        sb[c * len + k] = b;
+      }
+  }
+}
+
 // One CTA per unit.  A lane owns a tile, so nothing is reduced across lanes per
 // tile and a word of the survivor mask is built in a register; about 25
 // instructions per triple and lane, bound by issue and by the latency of staging
@@ -563,28 +595,7 @@ __global__ void __launch_bounds__(kCountThreads)
   const int len = staged_len(bk), kpad = len - 2;
   Screen* sa = s_scr;
   Screen* sb = s_scr + u.rows * len;
-  for (int x = warp; x < u.rows; x += kCountWarps) {
-    const double* src = nA + (int64_t)(u.r0 + x) * bk;
-#pragma unroll 8
-    for (int k = lane; k < kpad; k += 32) sa[x * len + k] = test_screen(k < bk ? src[k] : 0.0);
-  }
-  if (u.cols == 4) {   // lanes over (k, column): whole 32-byte sectors
-#pragma unroll 8
-    for (int x = tid; x < 4 * kpad; x += kCountThreads) {
-      const int k = x >> 2, c = x & 3;
-      Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
-      b.e -= T.e;
-      sb[c * len + k] = b;
-    }
-  } else {
-    for (int k = tid; k < kpad; k += kCountThreads)
-#pragma unroll 4
-      for (int c = 0; c < u.cols; ++c) {
-        Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
-        b.e -= T.e;
-        sb[c * len + k] = b;
-      }
-  }
+  stage_unit(in, u, sa, sb, T.e);
   if (split) {
     for (int i = tid; i < kFlagBins; i += kCountThreads) {
       s_bin_sum[i] = 0.0;
@@ -753,6 +764,183 @@ __global__ void __launch_bounds__(kCountThreads)
   if (!s_last) return;
   __threadfence();
   instance_stats(in, Bf, true);
+}
+
+// ---------------------------------------------------------------------------
+// Certified reference tau: the largest grid point -60 + 60 x / 2^36 (log10 of tau
+// relative to ||A|| ||B||) whose skipped-product bound bound2 is at most ref_rel
+// ||A|| ||B||, by the 36 decisions of a bisection, four of them per pass: a pass
+// forms bound2 at the 15 inner points of the current interval at once (a triple's
+// product falls between two of them and is added to that gap's sum of its tile;
+// a tile's bound at a point is the sum of the gaps below it), and its last CTA
+// takes the four decisions and lays out the next points.  No host round trip in
+// between: 36 counting half-plans with a synchronisation each took 1.0 ms at 64
+// blocks per side, this takes 0.2.
+// ---------------------------------------------------------------------------
+
+// Grid point x as a threshold.
+__device__ __forceinline__ double cert_tau(double ab, long long x) {
+  return ab * exp10(ldexp((double)(15 * (x - (1ll << 36))), -34));
+}
+
+// Norms (after prep), the first points and cleared sums: one warp.
+__global__ void cert_init_kernel(InstRef R, PlanBuffers Bf, double ref_rel) {
+  pdl_wait();
+  pdl_trigger();
+  const Inst& in = R.at(0);
+  CertState* cs = Bf.cert;
+  const int lane = threadIdx.x;
+  (void)instance_norms(in, Bf, true);
+  __syncwarp();
+  const double ab = in.pd->norm_a * in.pd->norm_b;
+  if (lane < kCertPoints) {
+    cs->tau[lane] = cert_tau(ab, (long long)(lane + 1) << 32);
+    cs->sum[lane] = 0.0;
+  }
+  if (lane == 0) {
+    cs->lo = 0;
+    cs->step = 1ll << 32;
+    cs->ab = ab;
+    cs->limit = ref_rel * ab;
+    cs->ticket = 0u;
+  }
+}
+
+// One pass: one CTA per unit.
+__global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, PlanBuffers Bf) {
+  pdl_wait();
+  pdl_trigger();
+  extern __shared__ __align__(16) Screen s_scr[];
+  __shared__ double s_tau[kCertPoints];
+  __shared__ int s_exp[kCertPoints];
+  __shared__ float s_gap[kCountWarps][kCertPoints][32];   // sums of the gaps, relative to 2^s_exp
+  __shared__ float s_S[kCountWarps][32];
+  __shared__ int s_E[kCountWarps][32];
+  __shared__ bool s_last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const Inst& in = R.at(0);
+  CertState* cs = Bf.cert;
+  const Unit u = unit_at(in, blockIdx.x);
+  const int bk = in.bk, bn = in.bn, len = staged_len(bk), nch = (len - 2) >> 5;
+  Screen* sa = s_scr;
+  Screen* sb = s_scr + u.rows * len;
+  stage_unit(in, u, sa, sb, 0);
+  if (tid < kCertPoints) {
+    s_tau[tid] = cs->tau[tid];
+    s_exp[tid] = test_screen(cs->tau[tid]).e;
+  }
+  for (int x = tid; x < kCountWarps * kCertPoints * 32; x += kCountThreads)
+    (&s_gap[0][0][0])[x] = 0.0f;
+  __syncthreads();
+  // FP32 windows around the lowest and the highest point (1 -+ 2^-20): products
+  // outside them need no FP64
+  const Screen t0 = test_screen(s_tau[0]), t1 = test_screen(s_tau[kCertPoints - 1]);
+  const float lo0 = t0.m * (1.0f - 9.5367431640625e-7f), hi1 = t1.m * (1.0f + 9.5367431640625e-7f);
+  const int c = lane / u.rows, r = lane - c * u.rows;
+  const bool act = c < u.cols;
+  const int i = u.r0 + r, j = u.j0 + c;
+  SkipSum sk{0.0f, kSkipStart};
+  if (act) {
+    const double* pa = in.nA + (int64_t)i * bk;
+    const double* pb = in.nB + j;
+    for (int w = warp; w < nch; w += kCountWarps) {
+      const int end = min(32, bk - w * 32);
+      for (int z0 = 0; z0 < end; z0 += 8) {
+        float q[8];
+        int D[8];
+#pragma unroll
+        for (int z = 0; z < 8; ++z) {
+          const int k = w * 32 + z0 + z;
+          const Screen a = sa[r * len + k], b = sb[c * len + k];
+          const float q0 = __fmul_rn(a.m, b.m);
+          const int E = a.e + b.e;
+          q[z] = q0;
+          D[z] = E;                                                 // below every point
+          if (screen_value(q0, E - t0.e) < lo0) continue;
+          D[z] = kSkipNone;                                         // survives the lowest point
+          if (z0 + z >= end || screen_value(q0, E - t1.e) >= hi1) continue;
+          const double p = __dmul_rn(pa[k], pb[(int64_t)k * bn]);   // between the points
+          int gap = 0;                                              // points at or below p
+#pragma unroll
+          for (int b2 = 8; b2 > 0; b2 >>= 1)
+            if (gap + b2 <= kCertPoints && !(p < s_tau[gap + b2 - 1])) gap += b2;
+          if (gap == 0) D[z] = E;
+          else if (gap < kCertPoints) s_gap[warp][gap - 1][lane] +=
+                __fmul_rn(q0, pow2f_or_zero(min(0, E - s_exp[gap] - 2)));
+        }
+        skip_add<8>(sk, q, D);
+      }
+    }
+  }
+  s_S[warp][lane] = sk.S;
+  s_E[warp][lane] = sk.Emax;
+  __syncthreads();
+  if (warp == 0) {
+    int emax = kSkipNone;
+#pragma unroll
+    for (int w = 0; w < kCountWarps; ++w) emax = max(emax, s_E[w][lane]);
+    float S = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kCountWarps; ++w)
+      S = __fmaf_rn(s_S[w][lane], pow2f_or_zero(max(s_E[w][lane] - emax, -127)), S);
+    ExtSum cum = S > 0.0f ? ExtSum{S, emax} : ExtSum{0.0f, 0};
+    for (int p = 0; p < kCertPoints; ++p) {
+      if (p > 0) {
+        float g = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kCountWarps; ++w) g += s_gap[w][p - 1][lane];
+        ext_add(cum, g, s_exp[p] + 2);
+      }
+      // a sum's own binade keeps its square inside the FP32 range
+      const float m = cum.m > 0.0f ? ldexpf(cum.m, -fexp(cum.m)) : 0.0f;
+      const ExtSum sq = ext_warp_sum_fast(ExtSum{__fmul_rn(m, m), 2 * (cum.e + (cum.m > 0.0f ? fexp(cum.m) : 0))});
+      if (lane == 0 && sq.m > 0.0f) atomicAdd(&cs->sum[p], ext_value(sq));
+    }
+  }
+  // the last CTA takes the pass's four decisions
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&cs->ticket, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!s_last || warp != 0) return;
+  __threadfence();
+  const double x = sqrt(lane < kCertPoints ? __ldcg(&cs->sum[lane]) : 0.0);
+  const unsigned ok = __ballot_sync(0xffffffffu, lane < kCertPoints && x <= cs->limit);
+  int at = 0;                        // point 0 is the interval's lower end
+#pragma unroll
+  for (int b2 = 8; b2 > 0; b2 >>= 1)
+    if ((ok >> (at + b2 - 1)) & 1u) at += b2;
+  const long long step = cs->step, lo = cs->lo + at * step, next = step >> 4;
+  __syncwarp();
+  if (lane < kCertPoints) {
+    if (next > 0) cs->tau[lane] = cert_tau(cs->ab, lo + (lane + 1) * next);
+    cs->sum[lane] = 0.0;
+  }
+  if (lane == 0) {
+    cs->lo = lo;
+    cs->step = next;
+    cs->ticket = 0u;
+  }
+}
+
+// Sum of squared tile norms over the tiles with survivors (one CTA).
+__global__ void __launch_bounds__(1024) tile_norms_kernel(InstRef R, PlanBuffers Bf) {
+  pdl_wait();
+  __shared__ double s_w[32];
+  const Inst& in = R.at(0);
+  const int64_t tiles = (int64_t)in.bm * in.bn;
+  double x = 0.0;
+#pragma unroll 4
+  for (int64_t t = threadIdx.x; t < tiles; t += 1024)
+    if (Bf.cnt[t] > 0) x = __fma_rn(in.nC[t], in.nC[t], x);
+  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = x;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    x = s_w[threadIdx.x];
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    if (threadIdx.x == 0) Bf.cert->norm = sqrt(x);
+  }
 }
 
 // Histogram bin of r = fl(fl(na nb) * inv) (one FP64 multiply, no other rounding):
@@ -1211,6 +1399,7 @@ size_t plan_layout(Inst* insts, int count, PlanBuffers* b, char* base, bool norm
   t.part = reinterpret_cast<int*>(take((size_t)cnt * kPartInts * sizeof(int)));
   t.part_bound = reinterpret_cast<ExtSum*>(take((size_t)cnt * 2 * sizeof(ExtSum)));
   t.group = reinterpret_cast<int*>(take((size_t)ugroups * kPartInts * sizeof(int)));
+  t.cert = reinterpret_cast<CertState*>(take(sizeof(CertState)));
   t.cnt = reinterpret_cast<int*>(take((size_t)tiles * sizeof(int)));
   t.tile_beg = reinterpret_cast<int*>(take((size_t)tiles * sizeof(int)));
   t.order = reinterpret_cast<int*>(take((size_t)tiles * sizeof(int)));
@@ -1302,6 +1491,29 @@ cudaError_t run_plan_count(const InstRef& ref, const PlanBuffers& b, cudaStream_
   // the statistics come from the last count CTA: its ticket needs the prep kernel
   cudaError_t e = launch_prep(ref, b, 0, s);
   return e == cudaSuccess ? launch_count(ref, b, 1, 1, s) : e;
+}
+
+cudaError_t run_certify(const InstRef& ref, const PlanBuffers& b, double ref_rel, cudaStream_t s) {
+  static bool opted[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!opted[dev]) {
+    e = cudaFuncSetAttribute(cert_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(16 * staged_len(kMaxBd) * sizeof(Screen)));
+    if (e != cudaSuccess) return e;
+    opted[dev] = true;
+  }
+  e = launch_prep(ref, b, 0, s);
+  if (e == cudaSuccess) e = launch_pdl(cert_init_kernel, dim3(1), dim3(32), 0, s, ref, b, ref_rel);
+  for (int pass = 0; pass < kCertBits / 4 && e == cudaSuccess; ++pass)
+    e = launch_pdl(cert_pass_kernel, dim3(b.count_ctas), dim3(kCountThreads), b.staged_bytes, s, ref, b);
+  return e;
+}
+
+cudaError_t run_tile_norms(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {
+  return launch_pdl(tile_norms_kernel, dim3(1), dim3(1024), 0, s, ref, b);
 }
 
 cudaError_t run_histogram(const InstRef& ref, const PlanBuffers& b, cudaStream_t s) {

@@ -66,6 +66,19 @@ enum Schedule { kScheduleStatic = 0, kScheduleDynamic = 1, kScheduleGroups = 2 }
 // consecutive block columns.
 constexpr int kGroupTiles = 4;
 
+// Certified reference tau (tau selection): state of its passes, and the norm of a
+// band product.
+constexpr int kCertBits = 36;      // decisions of the bisection, four per pass
+constexpr int kCertPoints = 15;    // thresholds per pass
+struct CertState {
+  double tau[kCertPoints];         // the pass's thresholds, increasing
+  double sum[kCertPoints];         // bound2 squared at each
+  double ab, limit;                // ||A|| ||B||, the largest admissible bound2
+  double norm;                     // run_tile_norms: the product's Frobenius norm
+  long long lo, step;              // grid point of the interval's lower end, distance of the points
+  unsigned int ticket;             // CTAs of the pass that have finished
+};
+
 constexpr int kPartInts = 16;   // ints per unit of totals
 
 // Extended-range FP32 sum: value = m * 2^e with an integer exponent.
@@ -163,6 +176,7 @@ struct PlanBuffers {
   int* part;           // [units * kPartInts] totals of each unit
   ExtSum* part_bound;  // [units * 2] sums of skipped products, and of their per-tile squares
   int* group;          // [groups * kPartInts] totals of each group of units
+  CertState* cert;
   int* cnt;            // [tiles] survivors per tile
   int* tile_beg;       // [tiles] absolute first k_idx slot of the tile
   int* order;          // [tiles] global ids: the non-empty tiles, most survivors first, then
@@ -215,6 +229,13 @@ cudaError_t run_plan_queue_half(const InstRef& ref, const PlanBuffers& b, cudaSt
 
 // The plan's counting half (statistics, survivors per tile; no queues).
 cudaError_t run_plan_count(const InstRef& ref, const PlanBuffers& b, cudaStream_t s);
+
+// Certified reference tau of a single instance: afterwards cert->lo is the grid
+// point (tau = ||A|| ||B|| 10^(-60 + 60 lo / 2^36)) and cert->ab = ||A|| ||B||.
+cudaError_t run_certify(const InstRef& ref, const PlanBuffers& b, double ref_rel, cudaStream_t s);
+// cert->norm = the Frobenius norm of a single instance's product from its output
+// norm map nC (tiles with survivors; the others are zero).
+cudaError_t run_tile_norms(const InstRef& ref, const PlanBuffers& b, cudaStream_t s);
 
 // Clears the statistics, builds the screen forms and norms (as run_plan's
 // first step) and the per-instance norm-product histograms (pd[i].hist).

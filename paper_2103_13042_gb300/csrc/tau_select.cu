@@ -11,8 +11,9 @@
 //     at most ref_rel ||A|| ||B||.
 //  2. error: for tau > tau_ref, AB - SpAMM(tau) = C_band + (AB - SpAMM(tau_ref))
 //     with C_band the product over the band tau_ref <= p < tau, so e(tau) is
-//     ||C_band||_F / (||A|| ||B||) to within ref_rel.  C_band is one band plan,
-//     one FP32 multiply into caller scratch and one Frobenius reduction.
+//     ||C_band||_F / (||A|| ||B||) to within ref_rel.  C_band is one band plan and
+//     one FP32 multiply into caller scratch; its norm comes from the tile norms
+//     the multiply writes.
 //  3. select: the network's tau (spamm_tau_predict) checked once; on a miss, or
 //     without a network, bisection on e: bracket [lo, hi] from tau0 =
 //     target ||A|| ||B|| by factors of 10 (up while e(hi) <= target, or down
@@ -26,8 +27,6 @@ using namespace spamm;
 
 namespace {
 
-constexpr int kCertifySteps = 36;
-constexpr double kCertifyLo = -60.0;   // log10 of the smallest relative tau tried
 constexpr int kBisectMaxEvals = 40;
 constexpr double kBisectRatio = 1.01;
 
@@ -57,31 +56,33 @@ spamm_status_t count_stats(Engine& e, const double* nA, const double* nB, double
 
 spamm_status_t certify(Engine& e, const double* nA, const double* nB, double ref_rel,
                        cudaStream_t s, double* tau_ref, double* ab_out) {
-  PlanDevice h;
-  spamm_status_t st = count_stats(e, nA, nB, 0.0, s, &h);
-  if (st != SPAMM_OK) return st;
-  const double ab = h.norm_a * h.norm_b;
-  *ab_out = ab;
-  if (!(ab > 0.0) || std::isinf(ab)) {   // a zero (or non-finite) operand: nothing to certify
+  Inst& in = e.insts[0];
+  in.nA = nA;
+  in.nB = nB;
+  in.band = 0;
+  in.split = 0;
+  in.quant = 0;
+  if (run_certify(make_ref(e.insts.data(), nullptr, 1), e.buf, ref_rel, s) != cudaSuccess)
+    return cuda_fail();
+  CertState h;
+  SPAMM_CUDA_TRY(cudaMemcpyAsync(&h, e.buf.cert, sizeof(h), cudaMemcpyDeviceToHost, s));
+  SPAMM_CUDA_TRY(cudaStreamSynchronize(s));
+  *ab_out = h.ab;
+  if (!(h.ab > 0.0) || std::isinf(h.ab)) {   // a zero (or non-finite) operand: nothing to certify
     *tau_ref = 0.0;
     return SPAMM_OK;
   }
-  double lo = kCertifyLo, hi = 0.0;
-  for (int it = 0; it < kCertifySteps; ++it) {
-    const double mid = 0.5 * (lo + hi);
-    st = count_stats(e, nA, nB, ab * std::pow(10.0, mid), s, &h);
-    if (st != SPAMM_OK) return st;
-    if (h.bound2 <= ref_rel * ab) lo = mid;
-    else hi = mid;
-  }
-  *tau_ref = ab * std::pow(10.0, lo);
+  // -60 + 60 lo / 2^36 (exact)
+  *tau_ref = h.ab * std::pow(10.0, std::ldexp((double)(15 * (h.lo - (1ll << 36))), -34));
   return SPAMM_OK;
 }
 
-// e(tau) relative to ||A|| ||B|| (0 at or below tau_ref).
+// e(tau) relative to ||A|| ||B|| (0 at or below tau_ref).  The multiply writes the
+// norm of every tile it stores, so the band product is neither completed with
+// zeros nor read back.
 spamm_status_t band_error(Engine& e, const double* nA, const double* nB, const float* A,
-                          const float* B, float* scratch, int64_t n, double tau, double tau_ref,
-                          double ab, cudaStream_t s, double* err) {
+                          const float* B, float* scratch, double tau, double tau_ref, double ab,
+                          cudaStream_t s, double* err) {
   if (!(tau > tau_ref) || !(ab > 0.0)) {
     *err = 0.0;
     return SPAMM_OK;
@@ -95,7 +96,7 @@ spamm_status_t band_error(Engine& e, const double* nA, const double* nB, const f
   in.lda = in.ldb = in.ldc = in.n;
   in.alpha = 1.0f;
   in.beta = 0.0f;
-  in.nC = nullptr;
+  in.nC = reinterpret_cast<double*>(e.buf.sA);   // bm * bk = bm * bn doubles, free here
   in.T = make_tau_screen(tau_ref);
   in.T_hi = make_tau_screen(tau);
   in.band = 1;
@@ -103,13 +104,14 @@ spamm_status_t band_error(Engine& e, const double* nA, const double* nB, const f
   in.quant = 0;
   const InstRef ref = make_ref(e.insts.data(), nullptr, 1);
   cudaError_t ce = run_plan(ref, e.buf, s);
-  in.band = 0;
   if (ce == cudaSuccess) ce = launch_multiply_simt(ref, e.buf, e.leaf, kScheduleStatic, false, s);
-  if (ce == cudaSuccess) ce = launch_zero_empty_tiles(ref, e.buf, e.leaf, s);
+  if (ce == cudaSuccess) ce = run_tile_norms(ref, e.buf, s);
+  in.band = 0;
+  in.nC = nullptr;
   if (ce != cudaSuccess) return cuda_fail();
   double norm = 0.0;
-  const spamm_status_t st = spamm_frobenius_diff(scratch, nullptr, n * n, &norm, s);
-  if (st != SPAMM_OK) return st;
+  SPAMM_CUDA_TRY(cudaMemcpyAsync(&norm, &e.buf.cert->norm, sizeof(double), cudaMemcpyDeviceToHost, s));
+  SPAMM_CUDA_TRY(cudaStreamSynchronize(s));
   *err = norm / ab;
   return SPAMM_OK;
 }
@@ -156,7 +158,7 @@ spamm_status_t spamm_tau_error(spamm_plan_t plan, const double* normA, const dou
   PlanDevice h;
   st = count_stats(plan->eng, normA, normB, 0.0, s, &h);   // ||A||, ||B|| from the norm maps
   if (st != SPAMM_OK) return st;
-  return band_error(plan->eng, normA, normB, A, B, scratch, plan->n, tau, tau_ref,
+  return band_error(plan->eng, normA, normB, A, B, scratch, tau, tau_ref,
                     h.norm_a * h.norm_b, s, err);
 }
 
@@ -179,7 +181,7 @@ spamm_status_t spamm_tau_select(spamm_plan_t plan, const double* normA, const do
   double last_err = 0.0;
   auto err_at = [&](double t, double* out) -> spamm_status_t {
     ++n_eval;
-    return band_error(e, normA, normB, A, B, scratch, plan->n, t, tau_ref, ab, s, out);
+    return band_error(e, normA, normB, A, B, scratch, t, tau_ref, ab, s, out);
   };
   auto finish = [&](double t, double et) {
     *tau = t;
