@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "lib", "libspamm.so")
 
@@ -140,15 +141,23 @@ def _check(code: int, where: str):
         raise SpammError(code, where)
 
 
+_raw_stream = None   # torch's raw current-stream query, where it has one (no Stream object built)
+
+
 def _stream(stream):
     if stream is None:
+        global _raw_stream
         import torch
+        if _raw_stream is None:
+            _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", False)
+        if _raw_stream:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return getattr(stream, "cuda_stream", stream)
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 # Tensor checks.  The C ABI sees bare pointers, so it cannot tell a CPU tensor, a wrong dtype,
@@ -176,19 +185,39 @@ def _index_of(t) -> int:
     return t.device.index if t.device.index is not None else 0
 
 
-def _tensor(t, where: str, name: str, dtype, numel=None, square=None, min_numel=None):
-    """Pointer of ``t`` after checking device, dtype, contiguity and size.
+# The checks run on every call, ten tensors of a norm map and a product, so a tensor that
+# passes takes the short way: plain attribute reads, the current device asked once per
+# call (about 0.6 us per tensor; the explaining form below took 2 to 3).
+
+def _here(t, dev: int) -> bool:
+    """t is on the current device ``dev``."""
+    if _DEVICE_TYPE == "cuda":
+        return t.is_cuda and t.get_device() == dev
+    return t.device.type == _DEVICE_TYPE and _index_of(t) == dev
+
+
+def _tensor(t, where: str, name: str, dtype, numel=None, square=None, min_numel=None, dev=None):
+    """Address of ``t`` after checking device, dtype, contiguity and size.
 
     ``numel``: the exact element count; ``min_numel``: the least one; ``square``: the side n
-    of an n x n matrix."""
+    of an n x n matrix; ``dev``: the current device index, when the caller already has it."""
+    if dev is None:
+        dev = _current_index()
+    try:
+        if (t.dtype is dtype and t.is_contiguous() and _here(t, dev) and
+                (numel is None or t.numel() == numel) and
+                (square is None or t.shape == (square, square)) and
+                (min_numel is None or t.numel() >= min_numel)):
+            return t.data_ptr()
+    except (AttributeError, TypeError):
+        pass
     import torch
     if not isinstance(t, torch.Tensor):
         _bad(where, f"{name} is not a tensor")
     if t.device.type != _DEVICE_TYPE:
         _bad(where, f"{name} is on {t.device}, not on the GPU")
-    cur = _current_index()
-    if _index_of(t) != cur:
-        _bad(where, f"{name} is on {t.device}, but the current device is {cur}")
+    if _index_of(t) != dev:
+        _bad(where, f"{name} is on {t.device}, but the current device is {dev}")
     if t.dtype != dtype:
         _bad(where, f"{name} is {t.dtype}, expected {dtype}")
     if not t.is_contiguous():
@@ -199,57 +228,53 @@ def _tensor(t, where: str, name: str, dtype, numel=None, square=None, min_numel=
         _bad(where, f"{name} has {t.numel()} elements, expected {numel}")
     if min_numel is not None and t.numel() < min_numel:
         _bad(where, f"{name} has {t.numel()} elements, expected at least {min_numel}")
-    return ctypes.c_void_p(t.data_ptr())
-
-
-_F32 = None
-
-
-def _mat_ptr(t, where: str, name, n: int, dev=None) -> int:
-    """Address of an n x n contiguous FP32 tensor on the current GPU (fast path; _tensor names
-    the fault).  ``dev``: the current device index, when the caller already has it."""
-    global _F32
-    if _F32 is None:
-        import torch
-        _F32 = torch.float32
-    if dev is None:
-        dev = _current_index()
-    try:
-        ok = (t.dtype is _F32 and t.shape == (n, n) and t.is_contiguous() and
-              (t.is_cuda and t.get_device() == dev if _DEVICE_TYPE == "cuda" else
-               t.device.type == _DEVICE_TYPE and _index_of(t) == dev))
-    except AttributeError:
-        ok = False
-    if not ok:
-        if not isinstance(name, str):             # ("As", i): formatted only on failure
-            name = "%s[%d]" % name
-        return _tensor(t, where, name, _F32, square=n).value
     return t.data_ptr()
 
 
-def _mat(t, where: str, name: str, n: int):
-    return ctypes.c_void_p(_mat_ptr(t, where, name, n))
+_F32 = _F64 = None
 
 
-def _rowmajor(t, where: str, name: str, rows: int, cols: int):
-    """(pointer, leading dimension) of a rows x cols FP32 GPU tensor whose rows are contiguous
+def _dtypes():
+    """Loads torch's float32 and float64 into _F32 and _F64 (torch is imported on first use)."""
+    global _F32, _F64
+    import torch
+    _F32, _F64 = torch.float32, torch.float64
+
+
+def _mat(t, where: str, name: str, n: int, dev=None) -> int:
+    """Address of an n x n contiguous FP32 tensor on the current GPU."""
+    if _F32 is None:
+        _dtypes()
+    return _tensor(t, where, name, _F32, square=n, dev=dev)
+
+
+def _rowmajor(t, where: str, name: str, rows: int, cols: int, dev=None):
+    """(address, leading dimension) of a rows x cols FP32 GPU tensor whose rows are contiguous
     (a row-major matrix or a view of one: stride(1) == 1, stride(0) >= cols)."""
+    if dev is None:
+        dev = _current_index()
+    if _F32 is None:
+        _dtypes()
+    try:
+        if t.dtype is _F32 and _here(t, dev) and t.shape == (rows, cols):
+            s0, s1 = t.stride()
+            ld = s0 if rows > 1 else max(cols, s0)
+            if (s1 == 1 or cols <= 1) and ld >= cols:
+                return t.data_ptr(), ld
+    except (AttributeError, TypeError, ValueError):
+        pass
     import torch
     if not isinstance(t, torch.Tensor):
         _bad(where, f"{name} is not a tensor")
     if t.device.type != _DEVICE_TYPE:
         _bad(where, f"{name} is on {t.device}, not on the GPU")
-    cur = _current_index()
-    if _index_of(t) != cur:
-        _bad(where, f"{name} is on {t.device}, but the current device is {cur}")
+    if _index_of(t) != dev:
+        _bad(where, f"{name} is on {t.device}, but the current device is {dev}")
     if t.dtype != torch.float32:
         _bad(where, f"{name} is {t.dtype}, expected torch.float32")
     if t.dim() != 2 or t.shape[0] != rows or t.shape[1] != cols:
         _bad(where, f"{name} has shape {tuple(t.shape)}, expected ({rows}, {cols})")
-    ld = t.stride(0) if rows > 1 else max(cols, t.stride(0))
-    if (t.stride(1) != 1 and cols > 1) or ld < cols:
-        _bad(where, f"{name} rows are not contiguous (strides {tuple(t.stride())})")
-    return ctypes.c_void_p(t.data_ptr()), ld
+    _bad(where, f"{name} rows are not contiguous (strides {tuple(t.stride())})")
 
 
 def _side(t, where: str, name: str) -> int:
@@ -259,9 +284,10 @@ def _side(t, where: str, name: str) -> int:
     return int(t.shape[0])
 
 
-def _norms(t, where: str, name: str, bd: int):
-    import torch
-    return _tensor(t, where, name, torch.float64, numel=bd * bd)
+def _norms(t, where: str, name: str, bd: int, dev=None):
+    if _F64 is None:
+        _dtypes()
+    return _tensor(t, where, name, _F64, numel=bd * bd, dev=dev)
 
 
 _PARAMS = None
@@ -305,17 +331,18 @@ def spamm_normmap(X, leaf: int, out=None, stream=None):
 
 def spamm_normmap_pair(A, B, leaf: int, outA=None, outB=None, stream=None):
     """Norm maps of both n x n operands of a product in one launch -> (normA, normB)."""
-    import torch
-    w = "spamm_normmap_pair"
+    w, dev = "spamm_normmap_pair", _current_index()
     n = _side(A, w, "A")
-    a, b = _mat(A, w, "A", n), _mat(B, w, "B", n)
+    a, b = _mat(A, w, "A", n, dev), _mat(B, w, "B", n, dev)
     bd = num_blocks(n, leaf) if leaf > 0 else 0
-    if outA is None:
-        outA = torch.empty((bd, bd), dtype=torch.float64, device=A.device)
-    if outB is None:
-        outB = torch.empty((bd, bd), dtype=torch.float64, device=A.device)
-    _check(lib().spamm_normmap_pair(a, b, n, leaf, _norms(outA, w, "normA", bd),
-                                    _norms(outB, w, "normB", bd), _stream(stream)), w)
+    if outA is None or outB is None:
+        import torch
+        if outA is None:
+            outA = torch.empty((bd, bd), dtype=torch.float64, device=A.device)
+        if outB is None:
+            outB = torch.empty((bd, bd), dtype=torch.float64, device=A.device)
+    _check(lib().spamm_normmap_pair(a, b, n, leaf, _norms(outA, w, "normA", bd, dev),
+                                    _norms(outB, w, "normB", bd, dev), _stream(stream)), w)
     return outA, outB
 
 
@@ -368,13 +395,15 @@ class Plan:
                                 float(target_rel_err), _stream(stream)), w)
         return self
 
-    def _na(self, t, w):
-        import torch
-        return _tensor(t, w, "normA", torch.float64, numel=self.bm * self.bk)
+    def _na(self, t, w, dev=None):
+        if _F64 is None:
+            _dtypes()
+        return _tensor(t, w, "normA", _F64, numel=self.bm * self.bk, dev=dev)
 
-    def _nb(self, t, w):
-        import torch
-        return _tensor(t, w, "normB", torch.float64, numel=self.bk * self.bn)
+    def _nb(self, t, w, dev=None):
+        if _F64 is None:
+            _dtypes()
+        return _tensor(t, w, "normB", _F64, numel=self.bk * self.bn, dev=dev)
 
     def stats(self, stream=None) -> dict:
         s = Stats()
@@ -394,19 +423,19 @@ class Plan:
         return tp, kk[:st["survivors"]]
 
     def multiply(self, A, B, C, stream=None):
-        w, n = "spamm_multiply", self.n
-        _check(lib().spamm_multiply(self.handle, _mat(A, w, "A", n), _mat(B, w, "B", n),
-                                    _mat(C, w, "C", n), _stream(stream)), w)
+        w, n, dev = "spamm_multiply", self.n, _current_index()
+        _check(lib().spamm_multiply(self.handle, _mat(A, w, "A", n, dev), _mat(B, w, "B", n, dev),
+                                    _mat(C, w, "C", n, dev), _stream(stream)), w)
         return C
 
     def plan_multiply(self, normA, normB, tau: float, A, B, C, target_rel_err: float = 1e-5,
                       stream=None):
         """plan() then multiply() in one call (zero-fill of empty tiles overlapped)."""
-        w, n = "spamm_plan_multiply", self.n
-        _check(lib().spamm_plan_multiply(self.handle, self._na(normA, w), self._nb(normB, w),
-                                         float(tau),
-                                         float(target_rel_err), _mat(A, w, "A", n),
-                                         _mat(B, w, "B", n), _mat(C, w, "C", n),
+        w, n, dev = "spamm_plan_multiply", self.n, _current_index()
+        _check(lib().spamm_plan_multiply(self.handle, self._na(normA, w, dev),
+                                         self._nb(normB, w, dev), float(tau),
+                                         float(target_rel_err), _mat(A, w, "A", n, dev),
+                                         _mat(B, w, "B", n, dev), _mat(C, w, "C", n, dev),
                                          _stream(stream)), w)
         return C
 
@@ -513,49 +542,52 @@ class GeneralPlan(Plan):
                "spamm_plan_workspace_size_general")
         return b.value
 
-    def _nc(self, t, w):
-        import torch
-        return None if t is None else _tensor(t, w, "normC", torch.float64,
-                                               numel=self.bm * self.bn)
+    def _nc(self, t, w, dev=None):
+        if t is None:
+            return None
+        if _F64 is None:
+            _dtypes()
+        return _tensor(t, w, "normC", _F64, numel=self.bm * self.bn, dev=dev)
 
     def multiply(self, A, B, C, alpha: float = 1.0, beta: float = 0.0, normC=None, stream=None):
         """C = alpha * (pruned A B) + beta * C; A, B, C may be row-major views (contiguous rows).
         normC (float64 [bm, bn], optional) receives C's norm map as stored."""
-        w = "spamm_multiply_general"
-        a, lda = _rowmajor(A, w, "A", self.m, self.k)
-        b, ldb = _rowmajor(B, w, "B", self.k, self.n)
-        c, ldc = _rowmajor(C, w, "C", self.m, self.n)
+        w, dev = "spamm_multiply_general", _current_index()
+        a, lda = _rowmajor(A, w, "A", self.m, self.k, dev)
+        b, ldb = _rowmajor(B, w, "B", self.k, self.n, dev)
+        c, ldc = _rowmajor(C, w, "C", self.m, self.n, dev)
         _check(lib().spamm_multiply_general(self.handle, a, lda, b, ldb, c, ldc, float(alpha),
-                                            float(beta), self._nc(normC, w), _stream(stream)), w)
+                                            float(beta), self._nc(normC, w, dev),
+                                            _stream(stream)), w)
         return C
 
     def plan_multiply(self, normA, normB, tau: float, A, B, C, target_rel_err: float = 1e-5,
                       alpha: float = 1.0, beta: float = 0.0, normC=None, stream=None):
-        w = "spamm_plan_multiply_general"
-        a, lda = _rowmajor(A, w, "A", self.m, self.k)
-        b, ldb = _rowmajor(B, w, "B", self.k, self.n)
-        c, ldc = _rowmajor(C, w, "C", self.m, self.n)
-        _check(lib().spamm_plan_multiply_general(self.handle, self._na(normA, w),
-                                                 self._nb(normB, w), float(tau),
+        w, dev = "spamm_plan_multiply_general", _current_index()
+        a, lda = _rowmajor(A, w, "A", self.m, self.k, dev)
+        b, ldb = _rowmajor(B, w, "B", self.k, self.n, dev)
+        c, ldc = _rowmajor(C, w, "C", self.m, self.n, dev)
+        _check(lib().spamm_plan_multiply_general(self.handle, self._na(normA, w, dev),
+                                                 self._nb(normB, w, dev), float(tau),
                                                  float(target_rel_err), a, lda, b, ldb, c, ldc,
-                                                 float(alpha), float(beta), self._nc(normC, w),
-                                                 _stream(stream)), w)
+                                                 float(alpha), float(beta),
+                                                 self._nc(normC, w, dev), _stream(stream)), w)
         return C
 
 
 def spamm_normmap_rect(X, leaf: int, out=None, stream=None):
     """Leaf Frobenius norms of a rows x cols FP32 device matrix (contiguous rows, any leading
     dimension) -> FP64 [ceil(rows/leaf), ceil(cols/leaf)] tensor."""
-    import torch
-    w = "spamm_normmap_rect"
+    w, dev = "spamm_normmap_rect", _current_index()
     if getattr(X, "dim", lambda: 0)() != 2:
         _bad(w, "X must be a 2-D tensor")
-    rows, cols = int(X.shape[0]), int(X.shape[1])
-    x, ld = _rowmajor(X, w, "X", rows, cols)
+    rows, cols = X.shape
+    x, ld = _rowmajor(X, w, "X", rows, cols, dev)
     br, bc = (num_blocks(rows, leaf), num_blocks(cols, leaf)) if leaf > 0 else (0, 0)
     if out is None:
+        import torch
         out = torch.empty((br, bc), dtype=torch.float64, device=X.device)
-    o = _tensor(out, w, "out", torch.float64, numel=br * bc)
+    o = _tensor(out, w, "out", _F64, numel=br * bc, dev=dev)
     _check(lib().spamm_normmap_rect(x, rows, cols, ld, leaf, o, _stream(stream)), w)
     return out
 
@@ -610,6 +642,10 @@ def spamm_multiply_fp32_noalloc(A, B, C, leaf: int, tau: float, stream=None):
     return C
 
 
+_PROBLEM = struct.Struct("=QQQqd")
+assert _PROBLEM.size == ctypes.sizeof(Problem)
+
+
 def _problems(As, Bs, Cs, taus, where: str, ns=None):
     """The problem table; every operand checked (n x n FP32 on the GPU, n = ns[i] if given).
     Cs may be None (no outputs: C stays NULL)."""
@@ -618,15 +654,26 @@ def _problems(As, Bs, Cs, taus, where: str, ns=None):
         _bad(where, "As, Bs, Cs and taus differ in length")
     if ns is not None and count != len(ns):
         _bad(where, f"{count} problems for a batch of {len(ns)}")
+    if _F32 is None:
+        _dtypes()
     arr = (Problem * count)()
-    dev = _current_index()
+    f32, dev, on_gpu, pack = _F32, _current_index(), _DEVICE_TYPE == "cuda", _PROBLEM.pack_into
+    ops = (("As", As), ("Bs", Bs)) if Cs is None else (("As", As), ("Bs", Bs), ("Cs", Cs))
+    at = [0, 0, 0]
     for i in range(count):
-        A = As[i]
-        n = _side(A, where, f"As[{i}]") if ns is None else ns[i]
-        arr[i] = Problem(_mat_ptr(A, where, ("As", i), n, dev),
-                         _mat_ptr(Bs[i], where, ("Bs", i), n, dev),
-                         None if Cs is None else _mat_ptr(Cs[i], where, ("Cs", i), n, dev),
-                         n, float(taus[i]))
+        n = _side(As[i], where, f"As[{i}]") if ns is None else ns[i]
+        shape = (n, n)
+        for k, (name, ts) in enumerate(ops):
+            t = ts[i]
+            try:
+                if on_gpu and (t.dtype is f32 and t.is_cuda and t.get_device() == dev and
+                               t.is_contiguous() and t.shape == shape):
+                    at[k] = t.data_ptr()
+                    continue
+            except AttributeError:
+                pass
+            at[k] = _mat(t, where, f"{name}[{i}]", n, dev)   # names the fault
+        pack(arr, _PROBLEM.size * i, at[0], at[1], at[2], n, float(taus[i]))
     return arr
 
 
