@@ -14,17 +14,18 @@
 // memory), the prediction from a histogram (one CTA per instance), one Adam
 // step, and the gradient and the training loop, both on one cluster of up to
 // 16 CTAs: every CTA keeps the weights in its shared memory and takes every
-// 16th chunk of 16 samples; the partial gradients are summed in a fixed order
-// through distributed shared memory, each CTA taking 1/16 of the parameters,
-// updating them (Adam, the moments in registers) and writing them back to
-// every CTA's weights.  A 256-sample step is 13 MFLOP: on one SM that alone is
-// 25 us, and the exchange (8449 values per CTA, two cluster barriers) costs
-// about 2 us.
+// 16th chunk of 16 samples.  In the training loop each CTA sends every other
+// its sixteenth of the partial gradient (one bulk copy into that CTA's shared
+// memory, completion counted on its mbarrier), sums the sixteen parts of its own
+// share in a fixed order, updates those weights (Adam, the moments in registers)
+// and sends them to every CTA.  A 256-sample step is 13 MFLOP: on one SM that
+// alone is 25 us.  Waits are bounded as in the multiply.
 #include <cmath>
 
 #include <cooperative_groups.h>
 
 #include "plan.cuh"
+#include "tc_common.cuh"
 
 namespace spamm {
 namespace mlp {
@@ -75,13 +76,17 @@ __global__ void __launch_bounds__(128) forward_kernel(const float* __restrict__ 
   Y[s] = forward_one(W, x);
 }
 
-// Adam with bias-corrected moments (beta1 0.9, beta2 0.999, eps 1e-8).
+// Adam with bias-corrected moments (beta1 0.9, beta2 0.999, eps 1e-8).  Zero moments
+// (weights of features that never occur, padding) are kept out of the divisions and
+// the square root: a zero operand there takes a slow path, for the whole warp.
 __device__ __forceinline__ void adam_update(float& w, float g, float& m, float& v, float lr,
                                             float c1, float c2) {
   m = 0.9f * m + 0.1f * g;
   v = 0.999f * v + 0.001f * g * g;
-  const float mhat = m / c1, vhat = v / c2;
-  w -= lr * mhat / (sqrtf(vhat) + 1e-8f);
+  const bool m0 = m == 0.0f, v0 = v == 0.0f;
+  const float mhat = (m0 ? 1.0f : m) / c1, root = sqrtf((v0 ? 1.0f : v) / c2);
+  const float step = lr * mhat / ((v0 ? 0.0f : root) + 1e-8f);
+  w -= m0 ? 0.0f : step;
 }
 
 __global__ void adam_kernel(float* __restrict__ W, const float* __restrict__ grad,
@@ -96,27 +101,39 @@ __global__ void adam_kernel(float* __restrict__ W, const float* __restrict__ gra
   v[p] = vv;
 }
 
-constexpr int kThreads = 256;
-constexpr int kChunk = 16;    // samples per chunk: 4 per warp pair
+constexpr int kThreads = 512;
+constexpr int kChunk = 16;    // samples per chunk: 2 per warp pair
 constexpr int kLd = 68;       // row stride in shared memory: 16-byte rows, conflict-free columns
+
+// The parameters as the cluster holds them: padded rows, whole 16-byte groups.  The
+// partial gradients and the exchange use the same layout; the padding stays zero,
+// but for b3[1], where the gradient carries the loss.
+struct Params {
+  float w1[kH * kLd], w2[kH * kLd], b1[kH], b2[kH], w3[kH], b3[4];
+  float pad[60];              // to equal shares of 16 (or 8) CTAs
+};
+constexpr int kGroups = sizeof(Params) / 16;                  // float4 groups
+constexpr int kLossSlot = 2 * kH * kLd + 3 * kH + 1;
+static_assert(sizeof(Params) % (16 * 16) == 0, "equal shares of whole groups");
 
 // Shared memory of one CTA of the gradient cluster.
 struct Net {
-  float w1[kH * kLd], w2[kH * kLd], b1[kH], b2[kH], w3[kH], b3[4];
+  Params w, part;             // weights; this CTA's partial gradient
   float x[2][kChunk * kLd];   // the chunk's samples, and the next chunk's on their way
   float h1[kChunk * kLd], h2[kChunk * kLd], g1[kChunk * kLd], g2[kChunk * kLd];
-  float y[2][kChunk], g3[kChunk], loss[kThreads / 32];
-  float part[kParams + 3];    // this CTA's partial gradient, then its partial loss
+  float y[2][kChunk], g3[kChunk], loss[kThreads / 32], gb3[kThreads / 32], half[4 * kH];
+  Params recv;                // this CTA's share of every CTA's partial gradient, by rank
+  uint64_t bar[2];            // all shares / all weights have arrived
+  int abort_flag, gave_up;    // a wait ran out
 };
 
-// Shared-memory slot of parameter p (the flat order of the weights).
-__device__ __forceinline__ float& weight(Net& n, int p) {
-  if (p < kOffB1) return n.w1[p / kIn * kLd + p % kIn];
-  if (p < kOffW2) return n.b1[p - kOffB1];
-  if (p < kOffB2) return n.w2[(p - kOffW2) / kH * kLd + (p - kOffW2) % kH];
-  if (p < kOffW3) return n.b2[p - kOffB2];
-  if (p < kOffB3) return n.w3[p - kOffW3];
-  return n.b3[0];
+// Place of parameter p (the flat order of the weights) in Params, in floats.
+__device__ __forceinline__ int place(int p) {
+  constexpr int kW2 = kH * kLd, kB1 = 2 * kH * kLd;
+  if (p < kOffB1) return p / kIn * kLd + p % kIn;
+  if (p < kOffW2) return kB1 + p - kOffB1;
+  if (p < kOffB2) return kW2 + (p - kOffW2) / kH * kLd + (p - kOffW2) % kH;
+  return kB1 + kH + p - kOffB2;   // b2, w3, b3 follow each other
 }
 
 __device__ __forceinline__ void copy4(float* dst, const float* src) {
@@ -126,36 +143,104 @@ __device__ __forceinline__ void copy4(float* dst, const float* src) {
                : "memory");
 }
 
-// Starts the copies of the samples c0 .. c0 + kChunk - 1 (zeros past `count`).
+// Row of this warp's sample of the chunk at c0: -1 past `count`.
+__device__ __forceinline__ int sample_row(const int* __restrict__ idx, int c0, int count) {
+  const int s = c0 + (int)(threadIdx.x >> 5);
+  return s < count ? (idx ? idx[s] : s) : -1;
+}
+
+// Starts the copies of a chunk's samples, one row per warp (-1: zeros).
 __device__ __forceinline__ void fetch(Net& n, int buf, const float* __restrict__ Xg,
-                                      const float* __restrict__ Yg, const int* __restrict__ idx,
-                                      int c0, int count) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < kChunk / 8; ++q) {   // a warp takes whole rows
-    const int s = warp + 8 * q;
-    float* dst = n.x[buf] + s * kLd;
-    if (c0 + s < count) {
-      const int row = idx ? idx[c0 + s] : c0 + s;
-      const float* src = Xg + (int64_t)row * kIn;
-      copy4(dst + lane, src + lane);
-      copy4(dst + lane + 32, src + lane + 32);
-      if (lane == 0) copy4(dst + 64, src + 64);
-      if (lane == 1) copy4(&n.y[buf][s], Yg + row);
-    } else {
-      dst[lane] = 0.0f;
-      dst[lane + 32] = 0.0f;
-      if (lane == 0) dst[64] = 0.0f;
-      if (lane == 1) n.y[buf][s] = 0.0f;
-    }
+                                      const float* __restrict__ Yg, int row) {
+  static_assert(kChunk == kThreads / 32, "a row per warp");
+  const int s = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* dst = n.x[buf] + s * kLd;
+  if (row >= 0) {
+    const float* src = Xg + (int64_t)row * kIn;
+    copy4(dst + lane, src + lane);
+    copy4(dst + lane + 32, src + lane + 32);
+    if (lane == 0) copy4(dst + 64, src + 64);
+    if (lane == 1) copy4(&n.y[buf][s], Yg + row);
+  } else {
+    dst[lane] = 0.0f;
+    dst[lane + 32] = 0.0f;
+    if (lane == 0) dst[64] = 0.0f;
+    if (lane == 1) n.y[buf][s] = 0.0f;
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// acc[4][4] += outer products of four columns of G and four of H over the chunk.
-__device__ __forceinline__ void outer4(const float* __restrict__ G, const float* __restrict__ H,
-                                       float (&acc)[4][4]) {
-#pragma unroll 4
+// A layer's products are cut into tiles of 4 units x 4 samples, the sum of a tile's
+// 16 values over eight neighbouring lanes (8 of the 64 terms each): 8 shared-memory
+// loads feed 64 FMAs, where a thread per unit and two samples needs 24 and is bound
+// by shared memory.  fold leaves each lane two of the values, all eight lanes' terms
+// summed in a fixed tree: unit lane / 2 of the tile, samples 2 (lane % 2) and the next.
+__device__ __forceinline__ void fold(float (&v)[16], int lane, float (&out)[2]) {
+#pragma unroll
+  for (int half = 8, bit = 4; half >= 2; half >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int q = 0; q < half; ++q) {
+      const float keep = up ? v[q + half] : v[q], send = up ? v[q] : v[q + half];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+    }
+  }
+  out[0] = v[0];
+  out[1] = v[1];
+}
+
+// Sums over 64 columns of W's rows u4 .. u4 + 3 times H's rows s4 .. s4 + 3.
+__device__ __forceinline__ void layer(const float* __restrict__ W, const float* __restrict__ H,
+                                      int lane, float (&out)[2]) {
+  float v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int k = (lane & 7) * 4 + 32 * i;
+    float4 w[4], h[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      w[a] = *reinterpret_cast<const float4*>(W + a * kLd + k);
+      h[a] = *reinterpret_cast<const float4*>(H + a * kLd + k);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        v[a * 4 + b] = fmaf(w[a].w, h[b].w,
+                            fmaf(w[a].z, h[b].z, fmaf(w[a].y, h[b].y, fmaf(w[a].x, h[b].x, v[a * 4 + b]))));
+  }
+  fold(v, lane, out);
+}
+
+// The same with W's transpose: sums over 64 rows of W's columns u4 .. u4 + 3 (W points at
+// the first) times H's rows s4 .. s4 + 3.
+__device__ __forceinline__ void layer_t(const float* __restrict__ W, const float* __restrict__ H,
+                                        int lane, float (&out)[2]) {
+  float v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = (lane & 7) + 8 * i;
+    const float4 w = *reinterpret_cast<const float4*>(W + k * kLd);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const float h = H[b * kLd + k];
+      v[b] = fmaf(w.x, h, v[b]);
+      v[4 + b] = fmaf(w.y, h, v[4 + b]);
+      v[8 + b] = fmaf(w.z, h, v[8 + b]);
+      v[12 + b] = fmaf(w.w, h, v[12 + b]);
+    }
+  }
+  fold(v, lane, out);
+}
+
+// acc[4][4] += outer products of four columns of G and of H over the chunk.
+__device__ __forceinline__ void outer(const float* __restrict__ G, const float* __restrict__ H,
+                                      float (&acc)[4][4]) {
+#pragma unroll 8
   for (int s = 0; s < kChunk; ++s) {
     const float4 g = *reinterpret_cast<const float4*>(G + s * kLd);
     const float4 h = *reinterpret_cast<const float4*>(H + s * kLd);
@@ -169,7 +254,7 @@ __device__ __forceinline__ void outer4(const float* __restrict__ G, const float*
 
 // This CTA's share of a gradient: the chunks first, first + stride, ... of `count`
 // samples (idx: their rows, or null), divided by norm, into n.part (with the
-// loss in part[kParams]).  The first chunk is in buffer 0 or on its way (fetch);
+// loss in part.b3[1]).  The first chunk is in buffer 0 or on its way (fetch);
 // then(): called once the last chunk's samples have been read, to fetch the
 // next call's first chunk into buffer 0.  Every thread of the CTA calls it.
 template <typename Then>
@@ -178,146 +263,149 @@ __device__ __forceinline__ void cta_gradient(Net& n, const float* __restrict__ X
                                              const int* __restrict__ idx, int count, float norm,
                                              float q, int first, int stride, Then then) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int o = (warp & 1) * 32 + lane, s0 = (warp >> 1) * 4;   // one unit, four samples
-  const int ty = (t >> 4) * 4, tx = (t & 15) * 4;               // 4 x 4 weights of each matrix
-  const int part = t >> 6, pu = t & 63;   // and: column 64 of W1, b1, b2, W3 (one unit each)
-  float a1[4][4], a2[4][4], ax = 0.0f, ab3 = 0.0f, loss = 0.0f;
+  // this thread's lanes' tile of 4 units x 4 samples, and its own unit and two samples
+  const int u4 = ((warp & 7) * 2 + ((lane >> 3) & 1)) * 4, s4 = ((warp >> 3) * 2 + (lane >> 4)) * 4;
+  const int o = u4 + ((lane >> 1) & 3), s0 = s4 + (lane & 1) * 2;
+  // 4 x 4 entries of d W1 (the lower half of the CTA) or d W2
+  const int upper = t >> 8, ty = ((t >> 4) & 15) * 4, tx = (t & 15) * 4;
+  // and, over half of the chunk: column 64 of W1, b1, b2, W3 (one unit each)
+  const int part = (t >> 6) & 3, pu = t & 63;
+  float acc[4][4], ax = 0.0f, ab3 = 0.0f, loss = 0.0f;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) a1[a][b] = a2[a][b] = 0.0f;
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
   const int chunks = (count + kChunk - 1) / kChunk;
   int buf = 0;
   for (int c = first; c < chunks; c += stride) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();   // the chunk is here, and the previous one has been read
-    if (c + stride < chunks) fetch(n, buf ^ 1, Xg, Yg, idx, (c + stride) * kChunk, count);
+    if (c + stride < chunks)
+      fetch(n, buf ^ 1, Xg, Yg, sample_row(idx, (c + stride) * kChunk, count));
     const float* x = n.x[buf];
-    float z1[4], z2[4];
-    // layer 1
-#pragma unroll
-    for (int j = 0; j < 4; ++j) z1[j] = n.b1[o];
-#pragma unroll 4
-    for (int i = 0; i < 64; i += 4) {
-      const float4 w = *reinterpret_cast<const float4*>(n.w1 + o * kLd + i);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 v = *reinterpret_cast<const float4*>(x + (s0 + j) * kLd + i);
-        z1[j] = fmaf(w.w, v.w, fmaf(w.z, v.z, fmaf(w.y, v.y, fmaf(w.x, v.x, z1[j]))));
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      z1[j] = fmaf(n.w1[o * kLd + 64], x[(s0 + j) * kLd + 64], z1[j]);
-      n.h1[(s0 + j) * kLd + o] = gelu(z1[j]);
-      z2[j] = n.b2[o];
-    }
-    __syncthreads();
-    // layer 2
-#pragma unroll 4
-    for (int i = 0; i < kH; i += 4) {
-      const float4 w = *reinterpret_cast<const float4*>(n.w2 + o * kLd + i);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 v = *reinterpret_cast<const float4*>(n.h1 + (s0 + j) * kLd + i);
-        z2[j] = fmaf(w.w, v.w, fmaf(w.z, v.z, fmaf(w.y, v.y, fmaf(w.x, v.x, z2[j]))));
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) n.h2[(s0 + j) * kLd + o] = gelu(z2[j]);
-    __syncthreads();
-    // output and d loss / d y (pinball slope q for r > 0, q - 1 otherwise): two samples per warp
+    float z1[2], z2[2], g[2];
+    layer(n.w.w1 + u4 * kLd, x + s4 * kLd, lane, z1);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int s = warp * 2 + j;
-      float y = fmaf(n.w3[lane], n.h2[s * kLd + lane], n.w3[lane + 32] * n.h2[s * kLd + lane + 32]);
+      z1[j] += fmaf(n.w.w1[o * kLd + 64], x[(s0 + j) * kLd + 64], n.w.b1[o]);
+      n.h1[(s0 + j) * kLd + o] = gelu(z1[j]);
+    }
+    __syncthreads();
+    layer(n.w.w2 + u4 * kLd, n.h1 + s4 * kLd, lane, z2);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      z2[j] += n.w.b2[o];
+      n.h2[(s0 + j) * kLd + o] = gelu(z2[j]);
+    }
+    __syncthreads();
+    // output and d loss / d y (pinball slope q for r > 0, q - 1 otherwise): a sample per warp
+    {
+      const int s = warp;
+      float y = fmaf(n.w.w3[lane], n.h2[s * kLd + lane], n.w.w3[lane + 32] * n.h2[s * kLd + lane + 32]);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) y += __shfl_xor_sync(0xffffffffu, y, off);
       if (lane == 0) {
         float g = 0.0f;
         if (c * kChunk + s < count) {
-          const float r = n.y[buf][s] - (y + n.b3[0]);
+          const float r = n.y[buf][s] - (y + n.w.b3[0]);
           g = -(r > 0.0f ? q : q - 1.0f) / norm;
           loss += fmaxf(q * r, (q - 1.0f) * r) / norm;
         }
         n.g3[s] = g;
+        ab3 += g;
       }
     }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      n.g2[(s0 + j) * kLd + o] = n.g3[s0 + j] * n.w3[o] * gelu_grad(z2[j]);
+    for (int j = 0; j < 2; ++j)
+      n.g2[(s0 + j) * kLd + o] = n.g3[s0 + j] * n.w.w3[o] * gelu_grad(z2[j]);
     __syncthreads();
-    {
-      float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 4
-      for (int j0 = 0; j0 < kH; j0 += 4) {
-        float w[4];
+    layer_t(n.w.w2 + u4, n.g2 + s4 * kLd, lane, g);
 #pragma unroll
-        for (int b = 0; b < 4; ++b) w[b] = n.w2[(j0 + b) * kLd + o];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 v = *reinterpret_cast<const float4*>(n.g2 + (s0 + j) * kLd + j0);
-          g[j] = fmaf(v.w, w[3], fmaf(v.z, w[2], fmaf(v.y, w[1], fmaf(v.x, w[0], g[j]))));
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) n.g1[(s0 + j) * kLd + o] = g[j] * gelu_grad(z1[j]);
-    }
+    for (int j = 0; j < 2; ++j) n.g1[(s0 + j) * kLd + o] = g[j] * gelu_grad(z1[j]);
     __syncthreads();
-    outer4(n.g1 + ty, x + tx, a1);
-    outer4(n.g2 + ty, n.h1 + tx, a2);
+    outer((upper ? n.g2 : n.g1) + ty, (upper ? n.h1 : x) + tx, acc);
     {
-      const float* g = part < 2 ? n.g1 : (part == 2 ? n.g2 : n.h2);
-#pragma unroll 4
-      for (int s = 0; s < kChunk; ++s) {
+      const float* gs = part < 2 ? n.g1 : (part == 2 ? n.g2 : n.h2);
+#pragma unroll
+      for (int z = 0; z < kChunk / 2; ++z) {
+        const int s = upper * (kChunk / 2) + z;
         const float f = part == 0 ? x[s * kLd + 64] : (part == 3 ? n.g3[s] : 1.0f);
-        ax = fmaf(f, g[s * kLd + pu], ax);
+        ax = fmaf(f, gs[s * kLd + pu], ax);
       }
-      if (t == 0)
-        for (int s = 0; s < kChunk; ++s) ab3 += n.g3[s];
     }
     buf ^= 1;
   }
-  if (lane == 0) n.loss[warp] = loss;
+  if (lane == 0) {
+    n.loss[warp] = loss;
+    n.gb3[warp] = ab3;
+  }
+  if (upper) n.half[t & 255] = ax;
   __syncthreads();   // every thread has read the last chunk
   then();
+  float* own = (upper ? n.part.w2 : n.part.w1) + ty * kLd + tx;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
+    *reinterpret_cast<float4*>(own + a * kLd) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+  if (!upper) {
+    ax += n.half[t];
+    if (part == 0) n.part.w1[pu * kLd + 64] = ax;
+    else (part == 1 ? n.part.b1 : (part == 2 ? n.part.b2 : n.part.w3))[pu] = ax;
+  } else if (t >= kThreads - 32) {   // the warps' sums of d loss / d y and of the loss
+    float sums[2] = {lane < kThreads / 32 ? n.gb3[lane] : 0.0f, lane < kThreads / 32 ? n.loss[lane] : 0.0f};
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      n.part[kOffW1 + (ty + a) * kIn + tx + b] = a1[a][b];
-      n.part[kOffW2 + (ty + a) * kH + tx + b] = a2[a][b];
+    for (int off = 16; off > 0; off >>= 1) {
+      sums[0] += __shfl_xor_sync(0xffffffffu, sums[0], off);
+      sums[1] += __shfl_xor_sync(0xffffffffu, sums[1], off);
     }
-  const int where[4] = {kOffW1 + pu * kIn + 64, kOffB1 + pu, kOffB2 + pu, kOffW3 + pu};
-  n.part[where[part]] = ax;
-  if (t == 0) {
-    n.part[kOffB3] = ab3;
-    float l = 0.0f;
-    for (int w = 0; w < kThreads / 32; ++w) l += n.loss[w];
-    n.part[kParams] = l;
+    if (lane == 0) {
+      n.part.b3[0] = sums[0];
+      n.part.b3[1] = sums[1];
+    }
   }
 }
 
-// Parameter slots (the loss counts as one) of each CTA of a cluster of CL.
+// Groups of each CTA of a cluster of CL: one per thread.
 template <int CL>
-constexpr int slice() { return (kParams + 1 + CL - 1) / CL; }
+constexpr int slice() {
+  static_assert(kGroups / CL <= kThreads, "a group per thread");
+  return kGroups / CL;
+}
 
-// Sum of slot p's partial values over the cluster, in rank order.
+// Sum of a group's partial values over the cluster, in rank order.
 template <int CL>
-__device__ __forceinline__ float cluster_total(cooperative_groups::cluster_group& cl, Net& n, int p) {
-  float v[CL];
+__device__ __forceinline__ float4 cluster_total(cooperative_groups::cluster_group& cl, Net& n, int g) {
+  float4 v[CL];
 #pragma unroll
-  for (int r = 0; r < CL; ++r) v[r] = *cl.map_shared_rank(&n.part[p], r);
-  float g = v[0];
+  for (int r = 0; r < CL; ++r) v[r] = *cl.map_shared_rank(reinterpret_cast<float4*>(&n.part) + g, r);
+  float4 s = v[0];
 #pragma unroll
-  for (int r = 1; r < CL; ++r) g += v[r];
-  return g;
+  for (int r = 1; r < CL; ++r) {
+    s.x += v[r].x;
+    s.y += v[r].y;
+    s.z += v[r].z;
+    s.w += v[r].w;
+  }
+  return s;
+}
+
+// Weights into shared memory, the padding of weights and partial gradient cleared.
+__device__ __forceinline__ void load_weights(Net& n, const float* __restrict__ Wg) {
+  for (int q = threadIdx.x; q < 2 * kGroups; q += kThreads)
+    reinterpret_cast<float4*>(&n.w)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  for (int p = threadIdx.x; p < kParams; p += kThreads) reinterpret_cast<float*>(&n.w)[place(p)] = Wg[p];
 }
 
 // One cluster: `steps` Adam steps; step s uses the samples idx[s * batch .. (s + 1) *
-// batch).  Before (one CTA, 32-sample chunks, W2 read with 32-way bank conflicts): 235
-// us per 256-sample step; now 11.7 us.
+// batch).  A wait that runs out leaves NaN weights (nothing is allocated for a status:
+// the call may be captured).
+// 64 steps of 256 samples: 515 us, 8 us a step.  Of a step's 15.7 thousand cycles each
+// layer takes 1.6 to 2.0 (shared memory and latency), the outer products 2.3 (shared
+// memory), Adam 1.2, the two exchanges 5 (35 KB each way per CTA at the ~20 bytes per
+// clock of the cluster's network).  Before: one CTA, W2 read with 32-way bank conflicts,
+// 15.1 ms; the cluster with a thread per unit and four samples, and the exchange by
+// remote loads and stores, 746 us.
 template <int CL>
 __global__ void __launch_bounds__(kThreads, 1)
     train_kernel(float* __restrict__ Wg, float* __restrict__ mg, float* __restrict__ vg, int t0,
@@ -328,49 +416,96 @@ __global__ void __launch_bounds__(kThreads, 1)
   Net& n = *reinterpret_cast<Net*>(smem);
   auto cl = cooperative_groups::this_cluster();
   const int rank = (int)cl.block_rank(), t = threadIdx.x;
-  constexpr int kSlice = slice<CL>(), kOwn = (kSlice + kThreads - 1) / kThreads;
-  for (int p = t; p < kParams; p += kThreads) weight(n, p) = Wg[p];
-  float m[kOwn], v[kOwn];
-#pragma unroll
-  for (int r = 0; r < kOwn; ++r) {
-    const int l = t + r * kThreads, p = rank * kSlice + l;
-    const bool mine = l < kSlice && p < kParams;
-    m[r] = mine ? mg[p] : 0.0f;
-    v[r] = mine ? vg[p] : 0.0f;
+  constexpr int kSlice = slice<CL>();
+  constexpr uint32_t kBytes = kSlice * 16;
+  const int g = rank * kSlice + t;           // this thread's group
+  const bool mine = t < kSlice;
+  const int to = (t & 31) ? CL : t >> 5;     // a copy per warp: their issue is serial within one
+  if (t == 0) {
+    tc::mbar_init(&n.bar[0], 1);
+    tc::mbar_init(&n.bar[1], 1);
+    n.abort_flag = n.gave_up = 0;
+    tc::fence_mbarrier_init();
   }
-  fetch(n, 0, X, Y, idx, rank * kChunk, batch);
+  load_weights(n, Wg);
+  // the moments of this thread's group, through the (still unused) partial gradient
+  float4 m, v;
+  for (int pass = 0; pass < 2; ++pass) {
+    __syncthreads();
+    for (int p = t; p < kParams; p += kThreads)
+      reinterpret_cast<float*>(&n.part)[place(p)] = (pass ? vg : mg)[p];
+    __syncthreads();
+    const float4 x = mine ? reinterpret_cast<float4*>(&n.part)[g] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (pass) v = x;
+    else m = x;
+  }
   __syncthreads();
-  for (int s = 0; s < steps; ++s) {
-    cta_gradient(n, X, Y, idx + (int64_t)s * batch, batch, (float)batch, q, rank, CL, [&] {
-      if (s + 1 < steps)
-        fetch(n, 0, X, Y, idx + (int64_t)(s + 1) * batch, rank * kChunk, batch);
-    });
-    cl.sync();   // every CTA's partial gradient is there
+  // the padding of the partial gradient stays zero
+  for (int q = t; q < kGroups; q += kThreads)
+    reinterpret_cast<float4*>(&n.part)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  fetch(n, 0, X, Y, sample_row(idx, rank * kChunk, batch));
+  cl.sync();   // every CTA's barriers are initialised
+  uint32_t phase = 0;
+  for (int s = 0; s < steps; ++s, phase ^= 1u) {
+    const int* now = idx + (int64_t)s * batch;
+    const int row = s + 1 < steps ? sample_row(now + batch, rank * kChunk, batch) : -1;
+    cta_gradient(n, X, Y, now, batch, (float)batch, q, rank, CL, [&] { fetch(n, 0, X, Y, row); });
+    tc::fence_proxy_async_smem();
+    __syncthreads();
+    // send every CTA its share; a share's place in the receiver is free: it sent the
+    // weights this step started from after it had summed the previous shares
+    if (t == 0) tc::mbar_arrive_expect_tx(&n.bar[0], CL * kBytes);
+    if (to < CL)
+      tc::bulk_s2peer(tc::peer_addr(reinterpret_cast<float4*>(&n.recv) + rank * kSlice, to),
+                      reinterpret_cast<float4*>(&n.part) + to * kSlice, kBytes,
+                      tc::peer_addr(&n.bar[0], to));
     const int step = t0 + s + 1;
     const float c1 = 1.0f - powf(0.9f, (float)step), c2 = 1.0f - powf(0.999f, (float)step);
+    (void)wait_ab(&n.bar[0], phase, &n.abort_flag, &n.gave_up);
+    if (mine) {
+      const float4* r4 = reinterpret_cast<const float4*>(&n.recv) + t;
+      float4 d = r4[0];
 #pragma unroll
-    for (int r = 0; r < kOwn; ++r) {
-      const int l = t + r * kThreads, p = rank * kSlice + l;
-      if (l >= kSlice || p > kParams) continue;
-      const float g = cluster_total<CL>(cl, n, p);
-      if (p == kParams) {
-        if (loss_hist) loss_hist[s] = g;
-        continue;
+      for (int r = 1; r < CL; ++r) {
+        const float4 x = r4[r * kSlice];
+        d.x += x.x;
+        d.y += x.y;
+        d.z += x.z;
+        d.w += x.w;
       }
-      float w = weight(n, p);
-      adam_update(w, g, m[r], v[r], lr, c1, c2);
-#pragma unroll
-      for (int d = 0; d < CL; ++d) *cl.map_shared_rank(&weight(n, p), d) = w;
+      if (g == kLossSlot / 4) {   // b3, the loss beside it
+        if (loss_hist) loss_hist[s] = d.y;
+        d.y = 0.0f;
+      }
+      float4 w = reinterpret_cast<float4*>(&n.w)[g];
+      adam_update(w.x, d.x, m.x, v.x, lr, c1, c2);
+      adam_update(w.y, d.y, m.y, v.y, lr, c1, c2);
+      adam_update(w.z, d.z, m.z, v.z, lr, c1, c2);
+      adam_update(w.w, d.w, m.w, v.w, lr, c1, c2);
+      reinterpret_cast<float4*>(&n.w)[g] = w;
+      tc::fence_proxy_async_smem();
     }
-    cl.sync();   // the new weights are everywhere, the partial gradients read
+    __syncthreads();
+    // send the new weights to the others (which have all finished this step's
+    // gradient: their shares are here)
+    if (t == 0) tc::mbar_arrive_expect_tx(&n.bar[1], (CL - 1) * kBytes);
+    if (to < CL && to != rank)
+      tc::bulk_s2peer(tc::peer_addr(reinterpret_cast<float4*>(&n.w) + rank * kSlice, to),
+                      reinterpret_cast<float4*>(&n.w) + rank * kSlice, kBytes,
+                      tc::peer_addr(&n.bar[1], to));
+    (void)wait_ab(&n.bar[1], phase, &n.abort_flag, &n.gave_up);
   }
-#pragma unroll
-  for (int r = 0; r < kOwn; ++r) {
-    const int l = t + r * kThreads, p = rank * kSlice + l;
-    if (l < kSlice && p < kParams) {
-      Wg[p] = weight(n, p);
-      mg[p] = m[r];
-      vg[p] = v[r];
+  cl.sync();   // no CTA leaves while another sends to it
+  // weights and moments back, each CTA its own groups
+  for (int pass = 0; pass < 2; ++pass) {
+    __syncthreads();
+    if (mine) reinterpret_cast<float4*>(&n.part)[g] = pass ? v : m;
+    __syncthreads();
+    for (int p = t; p < kParams; p += kThreads) {
+      const int at = place(p);
+      if (at / 4 / kSlice != rank) continue;
+      (pass ? vg : mg)[p] = reinterpret_cast<float*>(&n.part)[at];
+      if (!pass) Wg[p] = n.gave_up ? NAN : reinterpret_cast<float*>(&n.w)[at];
     }
   }
 }
@@ -385,18 +520,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   Net& n = *reinterpret_cast<Net*>(smem);
   auto cl = cooperative_groups::this_cluster();
   const int rank = (int)cl.block_rank();
-  for (int p = threadIdx.x; p < kParams; p += kThreads) weight(n, p) = Wg[p];
-  fetch(n, 0, X, Y, nullptr, rank * kChunk, count);
+  load_weights(n, Wg);
+  fetch(n, 0, X, Y, sample_row(nullptr, rank * kChunk, count));
   __syncthreads();
   cta_gradient(n, X, Y, nullptr, count, (float)count, q, rank, CL, [] {});
   cl.sync();
+  // this CTA's groups into its (then unused) weights, from there to the flat order
   for (int l = threadIdx.x; l < slice<CL>(); l += kThreads) {
-    const int p = rank * slice<CL>() + l;
-    if (p > kParams) continue;
-    const float g = cluster_total<CL>(cl, n, p);
-    if (p == kParams) *loss = g;
-    else grad[p] = g;
+    const int g = rank * slice<CL>() + l;
+    if (g < kGroups) reinterpret_cast<float4*>(&n.w)[g] = cluster_total<CL>(cl, n, g);
   }
+  __syncthreads();
+  for (int p = threadIdx.x; p < kParams; p += kThreads) {
+    const int at = place(p);
+    if (at / 4 / slice<CL>() == rank) grad[p] = reinterpret_cast<float*>(&n.w)[at];
+  }
+  if (threadIdx.x == 0 && kLossSlot / 4 / slice<CL>() == rank) *loss = n.w.b3[1];
   cl.sync();   // no CTA leaves while its shared memory is read
 }
 

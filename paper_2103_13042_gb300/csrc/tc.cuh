@@ -101,6 +101,23 @@ __device__ __forceinline__ void bulk_wait_read0() {
 __device__ __forceinline__ void bulk_wait0() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
+// The cluster address of this CTA's shared-memory object in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_addr(const void* p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+// Bulk copy of this CTA's shared memory into a CTA of the cluster, completion
+// counted in bytes on an mbarrier of that CTA.  Addresses 16-byte aligned, bytes a
+// multiple of 16.
+__device__ __forceinline__ void bulk_s2peer(uint32_t peer_dst, const void* src, uint32_t bytes,
+                                            uint32_t peer_bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(peer_dst),
+      "r"(smem_u32(src)), "r"(bytes), "r"(peer_bar)
+      : "memory");
+}
 // Orders this thread's generic-proxy shared-memory writes before its later
 // async-proxy (bulk copy) reads of them.
 __device__ __forceinline__ void fence_proxy_async_smem() {
