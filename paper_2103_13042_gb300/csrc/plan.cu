@@ -813,6 +813,8 @@ __global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, Pla
   extern __shared__ __align__(16) Screen s_scr[];
   __shared__ double s_tau[kCertPoints];
   __shared__ int s_exp[kCertPoints];
+  __shared__ Screen s_pt[kCertPoints];
+  __shared__ float2 s_cum[kCertPoints][40];   // a tile's sum up to each point: value, exponent
   __shared__ float s_gap[kCountWarps][kCertPoints][32];   // sums of the gaps, relative to 2^s_exp
   __shared__ float s_S[kCountWarps][32];
   __shared__ int s_E[kCountWarps][32];
@@ -821,13 +823,14 @@ __global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, Pla
   const Inst& in = R.at(0);
   CertState* cs = Bf.cert;
   const Unit u = unit_at(in, blockIdx.x);
-  const int bk = in.bk, bn = in.bn, len = staged_len(bk), nch = (len - 2) >> 5;
+  const int bk = in.bk, bn = in.bn, len = staged_len(bk);
   Screen* sa = s_scr;
   Screen* sb = s_scr + u.rows * len;
   stage_unit(in, u, sa, sb, 0);
   if (tid < kCertPoints) {
     s_tau[tid] = cs->tau[tid];
-    s_exp[tid] = test_screen(cs->tau[tid]).e;
+    s_pt[tid] = test_screen(cs->tau[tid]);
+    s_exp[tid] = s_pt[tid].e;
   }
   for (int x = tid; x < kCountWarps * kCertPoints * 32; x += kCountThreads)
     (&s_gap[0][0][0])[x] = 0.0f;
@@ -835,7 +838,8 @@ __global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, Pla
   // FP32 windows around the lowest and the highest point (1 -+ 2^-20): products
   // outside them need no FP64
   const Screen t0 = test_screen(s_tau[0]), t1 = test_screen(s_tau[kCertPoints - 1]);
-  const float lo0 = t0.m * (1.0f - 9.5367431640625e-7f), hi1 = t1.m * (1.0f + 9.5367431640625e-7f);
+  constexpr float kBelow = 1.0f - 9.5367431640625e-7f, kAbove = 1.0f + 9.5367431640625e-7f;
+  const float lo0 = t0.m * kBelow, hi1 = t1.m * kAbove;
   const int c = lane / u.rows, r = lane - c * u.rows;
   const bool act = c < u.cols;
   const int i = u.r0 + r, j = u.j0 + c;
@@ -843,38 +847,59 @@ __global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, Pla
   if (act) {
     const double* pa = in.nA + (int64_t)i * bk;
     const double* pb = in.nB + j;
-    for (int w = warp; w < nch; w += kCountWarps) {
-      const int end = min(32, bk - w * 32);
-      for (int z0 = 0; z0 < end; z0 += 8) {
-        float q[8];
-        int D[8];
+    for (int k0 = warp * 8; k0 < bk; k0 += 8 * kCountWarps) {
+      float q[8];
+      int D[8];
 #pragma unroll
-        for (int z = 0; z < 8; ++z) {
-          const int k = w * 32 + z0 + z;
-          const Screen a = sa[r * len + k], b = sb[c * len + k];
-          const float q0 = __fmul_rn(a.m, b.m);
-          const int E = a.e + b.e;
-          q[z] = q0;
-          D[z] = E;                                                 // below every point
-          if (screen_value(q0, E - t0.e) < lo0) continue;
-          D[z] = kSkipNone;                                         // survives the lowest point
-          if (z0 + z >= end || screen_value(q0, E - t1.e) >= hi1) continue;
-          const double p = __dmul_rn(pa[k], pb[(int64_t)k * bn]);   // between the points
-          int gap = 0;                                              // points at or below p
+      for (int z = 0; z < 8; ++z) {
+        const int k = k0 + z;
+        const Screen a = sa[r * len + k], b = sb[c * len + k];
+        const float q0 = __fmul_rn(a.m, b.m);
+        const int E = a.e + b.e;
+        q[z] = q0;
+        D[z] = E;                                                 // below every point
+        if (screen_value(q0, E - t0.e) < lo0) continue;
+        D[z] = kSkipNone;                                         // survives the lowest point
+        if (k >= bk || screen_value(q0, E - t1.e) >= hi1) continue;
+        // between the points: how many are at or below the product; FP64 (and the
+        // norms from memory) only next to a point
+        int gap = 0;
+        bool near = false;
+#pragma unroll
+        for (int b2 = 8; b2 > 0; b2 >>= 1) {
+          if (gap + b2 > kCertPoints) continue;
+          const Screen t = s_pt[gap + b2 - 1];
+          const float v = screen_value(q0, E - t.e);
+          if (v >= t.m * kAbove) gap += b2;
+          else if (v >= t.m * kBelow) near = true;
+        }
+        if (near) {
+          const double p = __dmul_rn(pa[k], pb[(int64_t)k * bn]);
+          gap = 0;
 #pragma unroll
           for (int b2 = 8; b2 > 0; b2 >>= 1)
             if (gap + b2 <= kCertPoints && !(p < s_tau[gap + b2 - 1])) gap += b2;
-          if (gap == 0) D[z] = E;
-          else if (gap < kCertPoints) s_gap[warp][gap - 1][lane] +=
-                __fmul_rn(q0, pow2f_or_zero(min(0, E - s_exp[gap] - 2)));
         }
-        skip_add<8>(sk, q, D);
+        if (gap == 0) D[z] = E;
+        else if (gap < kCertPoints) s_gap[warp][gap - 1][lane] +=
+              __fmul_rn(q0, pow2f_or_zero(min(0, E - s_exp[gap] - 2)));
       }
+      skip_add<8>(sk, q, D);
     }
   }
   s_S[warp][lane] = sk.S;
   s_E[warp][lane] = sk.Emax;
   __syncthreads();
+  for (int p = warp; p < kCertPoints - 1; p += kCountWarps) {   // every gap over the warps
+    float g = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kCountWarps; ++w) g += s_gap[w][p][lane];
+    s_gap[0][p][lane] = g;
+  }
+  __syncthreads();
+  // the tiles' sums up to every point (a lane per tile), then the points' sums of
+  // squares, eight threads each, in the order of a warp's butterfly (both by one warp,
+  // a point after the other, took 11 of a pass's 24 us)
   if (warp == 0) {
     int emax = kSkipNone;
 #pragma unroll
@@ -885,17 +910,43 @@ __global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, Pla
       S = __fmaf_rn(s_S[w][lane], pow2f_or_zero(max(s_E[w][lane] - emax, -127)), S);
     ExtSum cum = S > 0.0f ? ExtSum{S, emax} : ExtSum{0.0f, 0};
     for (int p = 0; p < kCertPoints; ++p) {
-      if (p > 0) {
-        float g = 0.0f;
-#pragma unroll
-        for (int w = 0; w < kCountWarps; ++w) g += s_gap[w][p - 1][lane];
-        ext_add(cum, g, s_exp[p] + 2);
-      }
-      // a sum's own binade keeps its square inside the FP32 range
-      const float m = cum.m > 0.0f ? ldexpf(cum.m, -fexp(cum.m)) : 0.0f;
-      const ExtSum sq = ext_warp_sum_fast(ExtSum{__fmul_rn(m, m), 2 * (cum.e + (cum.m > 0.0f ? fexp(cum.m) : 0))});
-      if (lane == 0 && sq.m > 0.0f) atomicAdd(&cs->sum[p], ext_value(sq));
+      if (p > 0) ext_add(cum, s_gap[0][p - 1][lane], s_exp[p] + 2);
+      s_cum[p][lane] = make_float2(cum.m, __int_as_float(cum.e));
     }
+  }
+  __syncthreads();
+  static_assert(kCountThreads >= 8 * (kCertPoints + 1), "eight threads per point");
+  const int pt = tid >> 3, sub = tid & 7;
+  if (warp < (kCertPoints + 1) / 4) {   // whole warps: point kCertPoints is empty
+    constexpr int kNone = -(1 << 29);
+    float sq[4];
+    int e[4], eb[4], emax = kNone;
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {   // tiles sub, sub + 16, sub + 8, sub + 24
+      const float2 x = pt < kCertPoints ? s_cum[pt][sub + (z & 1) * 16 + (z >> 1) * 8] : make_float2(0.0f, 0.0f);
+      // a sum's own binade keeps its square inside the FP32 range
+      const int own = x.x > 0.0f ? fexp(x.x) : 0;
+      const float m = x.x > 0.0f ? ldexpf(x.x, -own) : 0.0f;
+      sq[z] = __fmul_rn(m, m);
+      e[z] = 2 * (__float_as_int(x.y) + own);
+      eb[z] = sq[z] > 0.0f ? e[z] + fexp(sq[z]) : kNone;
+      emax = max(emax, eb[z]);
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
+    float v[4];
+#pragma unroll
+    for (int z = 0; z < 4; ++z)
+      v[z] = eb[z] != kNone && eb[z] >= emax - 40 ? sq[z] * pow2f(e[z] - (emax - 40)) : 0.0f;
+    float sum = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    ExtSum r{sum, emax - 40};
+    while (r.m >= 1099511627776.0f) {   // keep the mantissa below 2^40
+      r.m *= pow2f(-40);
+      r.e += 40;
+    }
+    if (sub == 0 && sum > 0.0f) atomicAdd(&cs->sum[pt], ext_value(r));
   }
   // the last CTA takes the pass's four decisions
   __threadfence();
