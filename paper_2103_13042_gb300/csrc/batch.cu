@@ -30,6 +30,7 @@ struct spamm_batch_s {
   size_t insts_offset = 0;       // offset of the Inst table inside it
   int n_vec_jobs = 0;            // norm-map jobs with 16-byte aligned rows (listed first)
   int units_vec = 0, units_other = 0;
+  int64_t entries = 0, max_n = 0;   // of all operands; the widest one's columns
   std::vector<int> job_slot;     // table slot of job 2 i + op (op 0: A, 1: B)
   std::vector<int> job_unit0;    // its first unit in its part of the table
   void* staging = nullptr;       // pinned host copy of the tables being uploaded
@@ -132,8 +133,8 @@ cudaError_t enqueue(spamm_batch_s* b, cudaStream_t s, bool timing) {
   cudaError_t e = timing ? cudaEventRecord(b->phase[0], s) : cudaSuccess;
   if (e == cudaSuccess)
     e = launch_normmap_jobs(b->jobs_dev, b->n_vec_jobs, b->units_vec, 2 * b->count - b->n_vec_jobs,
-                            b->units_other, b->eng.leaf, b->status, s, b->eng.side, b->eng.fork,
-                            b->eng.join);
+                            b->units_other, b->entries, b->max_n, b->eng.leaf, b->status, s,
+                            b->eng.side, b->eng.fork, b->eng.join);
   if (e == cudaSuccess && timing) e = cudaEventRecord(b->phase[1], s);
   if (e == cudaSuccess)
     e = engine_plan_multiply(b->eng, ref, b->status, s, timing ? b->phase[2] : nullptr,
@@ -213,6 +214,10 @@ spamm_status_t spamm_batch_create(spamm_batch_t* batch, const int64_t* n, int32_
   b->job_slot.resize(2 * (size_t)count);
   b->job_unit0.resize(2 * (size_t)count);
   int slot = 0;
+  for (int32_t i = 0; i < count; ++i) {
+    b->entries += 2 * n[i] * n[i];
+    b->max_n = std::max<int64_t>(b->max_n, n[i]);
+  }
   for (int pass = 0; pass < 2; ++pass) {
     const bool vec_pass = pass == 0;
     int64_t units = 0;
@@ -400,8 +405,8 @@ spamm_status_t spamm_batch_tau_predict(spamm_batch_t b, const spamm_problem_t* p
   if (st != SPAMM_OK) return st;
   const InstRef ref = batch_ref(b);
   cudaError_t err = launch_normmap_jobs(b->jobs_dev, b->n_vec_jobs, b->units_vec,
-                                        2 * b->count - b->n_vec_jobs, b->units_other, b->eng.leaf,
-                                        b->status, s);
+                                        2 * b->count - b->n_vec_jobs, b->units_other, b->entries,
+                                        b->max_n, b->eng.leaf, b->status, s);
   if (err == cudaSuccess) err = run_histogram(ref, b->eng.buf, s);
   if (err == cudaSuccess) err = launch_tau_from_hist(ref, weights, b->eng.feat_dev, b->eng.tau_dev, s);
   if (err != cudaSuccess) {

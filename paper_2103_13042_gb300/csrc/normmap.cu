@@ -98,21 +98,27 @@ constexpr uint64_t kStagedDrainNs = 100000000ull;   // 100 ms for the abort drai
 struct StagedJobs {
   const NormJob* table;
   int count, units;
+  int64_t entries;   // of all operands
+  int slices;        // pieces of 128 columns of a window (of the widest operand's)
   NormJob one[2];
 };
 
+// The last job with unit0 <= u, by a whole warp: 32 candidates at a time.
+__device__ __forceinline__ NormJob find_job(const NormJob* table, int count, int u) {
+  int lo = 0, n = count;
+  while (n > 1) {
+    const int step = (n + 31) / 32, at = lo + (int)(threadIdx.x & 31) * step;
+    const bool ok = at < lo + n && table[at].unit0 <= u;   // lane 0's always is
+    const int z = (31 - __clz(__ballot_sync(0xffffffffu, ok))) * step;
+    n = min(step, n - z);
+    lo += z;
+  }
+  return table[lo];
+}
+
 __device__ __forceinline__ NormJob job_of(const StagedJobs& J, int u) {
-  if (J.table == nullptr) {
-    if (J.count > 1 && u >= J.one[1].unit0) return J.one[1];
-    return J.one[0];
-  }
-  int lo = 0, hi = J.count - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) / 2;
-    if (J.table[mid].unit0 <= u) lo = mid;
-    else hi = mid - 1;
-  }
-  return J.table[lo];
+  if (J.table) return find_job(J.table, J.count, u);
+  return J.count > 1 && u >= J.one[1].unit0 ? J.one[1] : J.one[0];
 }
 
 // Bounded wait of a whole warp: returns (uniformly) once every lane has seen
@@ -405,6 +411,95 @@ __global__ void __launch_bounds__(Cfg::kThreads, Cfg::kCtasPerSm)
   }
 }
 
+// ---------------------------------------------------------------------------
+// Few entries (kDirectEntries): bound by latency, not by bandwidth.  In the staged kernel a
+// lane sums a strip's groups of 8 rows one after the other (0.3 us each) behind row
+// copies issued one after the other.  Here a CTA takes 128 columns of a strip, a warp
+// per group: the groups' sums are independent, and merged in their order afterwards,
+// which gives the bits of the staged kernel.  Aligned and other rows in one launch
+// (two on two streams, joined by events, cost a small batch 4 us).
+// ---------------------------------------------------------------------------
+// Up to this many entries (per launch): at 1024 x 1024 it takes 3.3, 4.1 and 5.9 us at
+// leaf 32, 64 and 128 (staged: 6.1, 9.5, 15.5), at 2300 x 2300 7.0, 8.8 and 11.7 (7.8, 9.4,
+// 15.7), at 2560 x 2560 7.4, 10.1 and 13.0 (8.0, 9.3, 15.2), and beyond it falls behind at
+// leaf 32 and 64; unaligned rows about 2 us more on both sides.
+constexpr int64_t kDirectEntries = (int64_t)5 << 20;
+
+// second: the first unit of a second table of jobs, count2 jobs from J.table[J.count] on.
+template <int LEAF>
+__global__ void __launch_bounds__(LEAF * 4) normmap_direct_kernel(const StagedJobs J, int second,
+                                                                  int count2) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int kGroups = LEAF / 8, kLanesPerBlockCol = LEAF / 4;
+  __shared__ SumSq s_part[kGroups][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane >> 3;
+  int u = blockIdx.x / J.slices;
+  const bool other = u >= second;
+  if (other) u -= second;
+  const NormJob jb = other ? find_job(J.table + J.count, count2, u) : job_of(J, u);
+  const UnitPos p = unit_pos<LEAF, StagedAligned>(jb, u);
+  const int64_t col = p.col0 + (blockIdx.x % J.slices * 32 + lane) * 4;
+  if (col - lane * 4 >= jb.cols) return;   // the whole CTA
+  const int64_t left = jb.cols - col;
+  const int nv = left >= 4 ? 4 : (left > 0 ? (int)left : 0);
+  const int rows = p.rows - warp * 8;
+  const float* src = jb.X + (p.row0 + warp * 8) * jb.ld + col;
+  float v[32];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float* rp = src + q * jb.ld;
+    if (jb.vec && nv == 4) {
+      const float4 t = q < rows ? __ldg(reinterpret_cast<const float4*>(rp)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[4 * q] = t.x;
+      v[4 * q + 1] = t.y;
+      v[4 * q + 2] = t.z;
+      v[4 * q + 3] = t.w;
+    } else {
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int c = jb.vec ? z : (l8 + z) & 3;   // the staged kernel's order
+        v[4 * q + z] = q < rows && c < nv ? __ldg(rp + c) : 0.0f;
+      }
+    }
+  }
+  SumSq ss = sumsq_empty();
+  if (rows > 0) sumsq_group<32>(ss, v);
+  s_part[warp][lane] = ss;
+  __syncthreads();
+  if (warp != 0) return;
+#pragma unroll
+  for (int g = 1; g < kGroups; ++g) {
+    const SumSq o = s_part[g][lane];
+    merge_from(ss, o.hi, o.lo, o.e);
+  }
+#pragma unroll
+  for (int off = kLanesPerBlockCol / 2; off > 0; off >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, ss.hi, off);
+    const float l = __shfl_xor_sync(0xffffffffu, ss.lo, off);
+    const int e = __shfl_xor_sync(0xffffffffu, ss.e, off);
+    merge_from(ss, h, l, e);
+  }
+  if ((lane % kLanesPerBlockCol) == 0 && nv > 0)
+    jb.out[(int64_t)p.I * jb.bc + col / LEAF] = sumsq_sqrt(ss);
+}
+
+template <int LEAF>
+cudaError_t launch_direct(const StagedJobs& J, int second, int count2, cudaStream_t s) {
+  return launch_pdl(normmap_direct_kernel<LEAF>, dim3(J.units * J.slices), dim3(LEAF * 4), 0, s, J,
+                    second, count2);
+}
+
+// All units of one or two sets of jobs in one direct launch.
+cudaError_t launch_direct_leaf(int leaf, const StagedJobs& J, int second, int count2, cudaStream_t s) {
+  switch (leaf) {
+    case 32: return launch_direct<32>(J, second, count2, s);
+    case 64: return launch_direct<64>(J, second, count2, s);
+    case 128: return launch_direct<128>(J, second, count2, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 // Resident CTAs of the staged kernel on the current device (occupancy x SMs).
 template <int LEAF, class Cfg>
 cudaError_t staged_capacity(int* cap) {
@@ -450,6 +545,8 @@ cudaError_t launch_staged_jobs(const StagedJobs& J, int32_t* status, cudaStream_
 template <class Cfg>
 cudaError_t launch_leaf(int leaf, const StagedJobs& J, int32_t* status, cudaStream_t s,
                         double share = 1.0) {
+  if (J.units > 0 && J.entries <= kDirectEntries && share == 1.0)
+    return launch_direct_leaf(leaf, J, J.units, 0, s);
   switch (leaf) {
     case 32: return launch_staged_jobs<32, Cfg>(J, status, s, share);
     case 64: return launch_staged_jobs<64, Cfg>(J, status, s, share);
@@ -488,6 +585,15 @@ cudaError_t launch_normmap_wait_selftest(int32_t* status, uint64_t limit_ns, lon
   return cudaPeekAtLastError();
 }
 
+namespace {
+
+void set_entries(StagedJobs& J, int64_t entries, int64_t max_cols) {
+  J.entries = entries;
+  J.slices = (int)std::min<int64_t>((max_cols + 127) / 128, StagedAligned::kWinCols / 128);
+}
+
+}  // namespace
+
 int normjob_shape(NormJob& j, int leaf) {
   j.br = (int)num_blocks(j.rows, leaf);
   j.bc = (int)num_blocks(j.cols, leaf);
@@ -511,6 +617,7 @@ cudaError_t launch_normmap_rect(const float* X, int64_t rows, int64_t cols, int6
   j.vec = (ld % 4) == 0;
   j.unit0 = 0;
   J.units = normjob_shape(j, leaf);
+  set_entries(J, rows * cols, cols);
   return j.vec ? launch_leaf<StagedAligned>(leaf, J, status, s)
                : launch_leaf<StagedUnaligned>(leaf, J, status, s);
 }
@@ -538,13 +645,15 @@ cudaError_t launch_normmap_pair(const float* A, const float* B, int64_t n, int32
     units += normjob_shape(j, leaf);
   }
   J.units = units;
+  set_entries(J, 2 * n * n, n);
   return vec ? launch_leaf<StagedAligned>(leaf, J, status, s)
              : launch_leaf<StagedUnaligned>(leaf, J, status, s);
 }
 
 cudaError_t launch_normmap_jobs(const NormJob* dev_jobs, int n_vec, int units_vec, int n_other,
-                                int units_other, int leaf, int32_t* status, cudaStream_t s,
-                                cudaStream_t side, cudaEvent_t fork, cudaEvent_t join) {
+                                int units_other, int64_t entries, int64_t max_cols, int leaf,
+                                int32_t* status, cudaStream_t s, cudaStream_t side,
+                                cudaEvent_t fork, cudaEvent_t join) {
   StagedJobs Jv{}, Jo{};
   Jv.table = dev_jobs;
   Jv.count = n_vec;
@@ -552,7 +661,13 @@ cudaError_t launch_normmap_jobs(const NormJob* dev_jobs, int n_vec, int units_ve
   Jo.table = dev_jobs + n_vec;
   Jo.count = n_other;
   Jo.units = units_other;
+  set_entries(Jv, entries, max_cols);
+  set_entries(Jo, entries, max_cols);
   cudaError_t e = cudaSuccess;
+  if (n_vec > 0 && n_other > 0 && entries <= kDirectEntries) {
+    Jv.units = units_vec + units_other;
+    return launch_direct_leaf(leaf, Jv, units_vec, n_other, s);
+  }
   if (n_vec > 0 && n_other > 0 && side && fork && join) {
     // both kinds at once, on two streams, the resident CTAs shared in proportion
     // to the units: they end together instead of one after the other

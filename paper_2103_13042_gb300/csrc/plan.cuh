@@ -272,12 +272,13 @@ cudaError_t launch_normmap_wait_selftest(int32_t* status, uint64_t limit_ns, lon
 // Sets br, bc, nwin and lines from X, rows, cols, ld, vec and the leaf;
 // returns the job's units.
 int normjob_shape(NormJob& j, int leaf);
-// Both kinds of jobs (16-byte aligned rows, others); with a side stream and two
-// events they run at once, sharing the SMs in proportion to their units.
+// Both kinds of jobs (16-byte aligned rows, others): in one launch when they are small
+// (entries of all operands); else, with a side stream and two events, at once, sharing
+// the SMs in proportion to their units.
 cudaError_t launch_normmap_jobs(const NormJob* dev_jobs, int n_vec, int units_vec, int n_other,
-                                int units_other, int leaf, int32_t* status, cudaStream_t s,
-                                cudaStream_t side = nullptr, cudaEvent_t fork = nullptr,
-                                cudaEvent_t join = nullptr);
+                                int units_other, int64_t entries, int64_t max_cols, int leaf,
+                                int32_t* status, cudaStream_t s, cudaStream_t side = nullptr,
+                                cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
 
 // FP32 multiply of the non-empty tiles; zeros: of the empty ones too (where
 // simt_writes_zeros says so).
