@@ -368,36 +368,50 @@ __device__ __forceinline__ double instance_norms(const Inst& in, const PlanBuffe
 }
 
 // The flag binade m = the largest mm in [kFlagBinMin - 1, 1] with
-// c1 * sum_{bins < mm} p <= budget, by one warp; bins are prefix-summed in a
-// fixed order (7 consecutive bins per lane, then a warp scan of the lane totals).
-__device__ __forceinline__ int flag_binade(const Inst& in, double ab, double bound2) {
-  constexpr int PER = (kFlagBins + 31) / 32;   // 7
+// c1 * sum_{bins < mm} p <= budget, in two halves of one warp each.  flag_prefix: the
+// sums below every bin, in a fixed order (7 consecutive bins per lane, then a warp
+// scan of the lane totals).  flag_pick: they grow with the bin, so every lane tests its
+// first bin, and seven lanes the bins of the last lane that passed (a test of all seven
+// by every lane is ten times the FP64 instructions, at 64 cycles each).
+constexpr int kBinsPerLane = (kFlagBins + 31) / 32;   // 7
+
+__device__ __forceinline__ void flag_prefix(const Inst& in, double* below) {
   const int lane = threadIdx.x & 31;
-  const double budget = 0.5 * (in.target_rel * ab - bound2);
-  double v[PER];
+  double v[kBinsPerLane];
   double run = 0.0;
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int b = lane * PER + q;
+  for (int q = 0; q < kBinsPerLane; ++q) {
+    const int b = lane * kBinsPerLane + q;
     v[q] = b < kFlagBins ? __ldcg(&in.pd->bin_sum[b]) : 0.0;
-    run += v[q];
   }
+#pragma unroll
+  for (int q = 0; q < kBinsPerLane; ++q) run += v[q];
   double incl = run;
+#pragma unroll 1
   for (int off = 1; off < 32; off <<= 1) {
     const double y = __shfl_up_sync(0xffffffffu, incl, off);
     if (lane >= off) incl += y;
   }
-  double below = incl - run;     // sum of the bins before this lane's first
-  int best = kFlagBinMin - 1;
-  if (budget >= 0.0) {
+  double x = incl - run;     // sum of the bins before this lane's first
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      const int b = lane * PER + q;       // candidate mm = kFlagBinMin + b
-      if (b < kFlagBins && in.c1 * below <= budget) best = kFlagBinMin + b;
-      below += v[q];
-    }
+  for (int q = 0; q < kBinsPerLane; ++q) {
+    below[lane * kBinsPerLane + q] = x;
+    x += v[q];
   }
-  return __reduce_max_sync(0xffffffffu, best);
+  __syncwarp();
+}
+
+__device__ __forceinline__ int flag_pick(const Inst& in, double ab, double bound2,
+                                         const double* below) {
+  const int lane = threadIdx.x & 31;
+  const double budget = 0.5 * (in.target_rel * ab - bound2);
+  const bool first = budget >= 0.0 && in.c1 * below[lane * kBinsPerLane] <= budget &&
+                     lane * kBinsPerLane < kFlagBins;
+  const unsigned pass = __ballot_sync(0xffffffffu, first);
+  if (pass == 0u) return kFlagBinMin - 1;
+  const int b = (31 - __clz(pass)) * kBinsPerLane + min(lane, kBinsPerLane - 1);
+  const bool ok = b < kFlagBins && in.c1 * below[b] <= budget;
+  return kFlagBinMin + __reduce_max_sync(0xffffffffu, ok ? b : 0);
 }
 
 // One instance's sums over its units.
@@ -457,9 +471,10 @@ __device__ __forceinline__ void merge_sums(UnitSums& u, const UnitSums& v) {
 // The statistics of one instance from its sums, by one warp (one square root and
 // one division for all of them).  prepped: the count kernel left the norms in the
 // statistics; otherwise they come from the units' partial sums and are written
-// too.  Returns the split-flag binade; publish = false: only that.
+// too.  Returns the split-flag binade (below: flag_prefix's sums); publish = false:
+// only that.
 __device__ __forceinline__ int write_stats(const Inst& in, const PlanBuffers& Bf, const UnitSums& u,
-                                           bool prepped, bool publish) {
+                                           bool prepped, bool publish, const double* below) {
   const int lane = threadIdx.x & 31;
   PlanDevice* pd = in.pd;
   double x = prepped ? 0.0 : sum_norms(Bf, in.count0, units_of(in));
@@ -468,7 +483,7 @@ __device__ __forceinline__ int write_stats(const Inst& in, const PlanBuffers& Bf
   const double na = __shfl_sync(0xffffffffu, x, 0), nb = __shfl_sync(0xffffffffu, x, 1);
   const double bound2 = __shfl_sync(0xffffffffu, x, 2);
   const double ab = na * nb;
-  const int m = in.split ? flag_binade(in, ab, bound2) : kFlagBinMin - 1;
+  const int m = in.split ? flag_pick(in, ab, bound2, below) : kFlagBinMin - 1;
   if (!publish) return m;
   const double cube = (double)in.bm * (double)in.bk * (double)in.bn;
   const double quot = (lane == 0 ? 1.0 : (double)u.S) / (lane == 0 ? ab : cube);
@@ -511,11 +526,13 @@ __device__ __forceinline__ UnitSums merged(const UnitSums* parts) {
 }
 
 // The statistics of one instance by a CTA of kStatWarps warps or more.
-__device__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped) {
+__device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped) {
   __shared__ UnitSums s_u[kStatWarps];
+  __shared__ double s_below[32 * kBinsPerLane];
   if (threadIdx.x / 32 < kStatWarps) stat_part(in, Bf, s_u, threadIdx.x / 32);
+  if (threadIdx.x < 32 && in.split) flag_prefix(in, s_below);
   __syncthreads();
-  if (threadIdx.x < 32) (void)write_stats(in, Bf, merged(s_u), prepped, true);
+  if (threadIdx.x < 32) (void)write_stats(in, Bf, merged(s_u), prepped, true, s_below);
 }
 
 // Screens of one staged row or column: whole words of 32 k (the tail holds
@@ -1070,50 +1087,151 @@ __global__ void __launch_bounds__(kHistWarps * 32)
     if (s_hist[q]) atomicAdd(&in.pd->hist[q], s_hist[q]);
 }
 
+__device__ __forceinline__ void add4(int4& a, const int4& b) {
+  a.x += b.x;
+  a.y += b.y;
+  a.z += b.z;
+  a.w += b.w;
+}
+__device__ __forceinline__ int4 shfl_xor4(const int4& v, int off) {
+  return make_int4(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off),
+                   __shfl_xor_sync(0xffffffffu, v.z, off), __shfl_xor_sync(0xffffffffu, v.w, off));
+}
+
+// A lane's tile of a unit: lane c * rows + r has row r, column c.
+struct FillLane {
+  Unit u;
+  int ii, nch, c, r, i, j;
+  bool act;
+  int64_t g, mask;   // tile; its first mask word
+};
+
+__device__ __forceinline__ FillLane fill_lane(const InstRef& R, int un) {
+  FillLane f;
+  f.ii = inst_of_unit(R, un);
+  const Inst& in = R.at(f.ii);
+  f.u = unit_at(in, un - in.count0);
+  f.nch = (in.bk + 31) >> 5;
+  const int lane = threadIdx.x & 31;
+  f.c = lane / f.u.rows;
+  f.r = lane - f.c * f.u.rows;
+  f.act = f.c < f.u.cols;
+  f.i = f.u.r0 + f.r;
+  f.j = f.u.j0 + f.c;
+  const int64_t t = (int64_t)f.i * in.bn + f.j;
+  f.g = in.tile0 + t;
+  f.mask = in.mask0 + t * f.nch;
+  return f;
+}
+
+// Puts the blocks of A and B that a unit's triples use on the list of needed blocks, by
+// one warp.
+__device__ __forceinline__ void need_blocks(const InstRef& R, const PlanBuffers& Bf, const FillLane& f) {
+  const Inst& in = R.at(f.ii);
+  if (!in.quant) return;
+  const int lane = threadIdx.x & 31, bk = in.bk, nch = f.nch;
+  for (int w0 = 0; w0 < nch; w0 += 4) {
+    uint32_t word[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      word[q] = f.act && w0 + q < nch ? __ldcg(Bf.surv_mask + f.mask + w0 + q) : 0u;
+    // the blocks of A and B that the unit's triples use: lane x < rows holds row x
+    // of A, the next cols lanes the columns of B, 32 k per word; the four words'
+    // round trips go out together
+    uint32_t mine[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      mine[q] = 0u;
+      if (!__any_sync(0xffffffffu, word[q] != 0u)) continue;
+      for (int x = 0; x < f.u.rows + f.u.cols; ++x) {
+        const bool in_set = x < f.u.rows ? f.r == x : f.c == x - f.u.rows;
+        const uint32_t o = __reduce_or_sync(0xffffffffu, in_set ? word[q] : 0u);
+        if (lane == x) mine[q] = o;
+      }
+    }
+    const bool isB = lane >= f.u.rows;
+    const int bi = isB ? f.u.j0 + lane - f.u.rows : f.u.r0 + lane;   // column of B / row of A
+    uint32_t* w = Bf.need_bits + (isB ? Bf.need_words_a + in.needb0 : in.needa0) +
+                  (int64_t)bi * nch + w0;
+    uint32_t fresh[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)   // a plain read first: a bit once set stays set
+      fresh[q] = mine[q] ? mine[q] & ~__ldcg(w + q) : 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (fresh[q]) fresh[q] = mine[q] & ~atomicOr(w + q, mine[q]);
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) n += __popc(fresh[q]);
+    int end = n;
+    for (int off = 1; off < 32; off <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, end, off);
+      if (lane >= off) end += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, end, 31);
+    if (total > 0) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&Bf.bdev->need_count, total);
+      at = __shfl_sync(0xffffffffu, at, 0) + end - n;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        for (; fresh[q]; fresh[q] &= fresh[q] - 1u) {
+          const int64_t k = (w0 + q) * 32 + __ffs(fresh[q]) - 1;
+          Bf.need_list[at++] = isB ? (uint32_t)(in.bblk0 + k * in.bn + bi) | 0x80000000u
+                                   : (uint32_t)(in.ablk0 + (int64_t)bi * bk + k);
+        }
+    }
+  }
+}
+
 // Work queues of `per_cta` consecutive units per CTA (kUnitWarps warps per
 // unit).  The first slots come from the totals of all units (or of the groups
 // of units): a few KB from L2 per CTA, instead of a scan kernel of its own
 // between count and fill.  Count and fill together, without the memset, prep and
 // finalize launches they replace: 30 -> 11 us at 32 blocks per side, 48 -> 17 at
 // 64 (10% of the triples survive), 169 -> 26 at 128 (half of them survive: one
-// atomic per word of needed blocks instead of two per triple).
+// atomic per word of needed blocks instead of two per triple).  Then bound by
+// instruction fetches and round trips: what needs only the arguments is done while the
+// count kernel runs, the list of needed blocks is made beside the scan, short lists
+// are written by a lane per tile.  Inside the product's chain the kernel takes 4.7 us at
+// 32 blocks per side (7.1 before), 5.5 for 4 x 18 x 100 blocks (11.4), 12 at 128 with
+// split flags (21).
 __global__ void __launch_bounds__(kFillThreads)
     fill_kernel(InstRef R, PlanBuffers Bf, int per_cta, int prepped) {
-  pdl_wait();
-  pdl_trigger();
   constexpr int kMaxPer = 32;
-  __shared__ int s_red[kFillWarps][2 * kPartInts];
+  __shared__ __align__(16) int s_red[kFillWarps][2 * kPartInts];
   __shared__ int s_base[kPartInts];          // buckets 1 .. 11: first slots of the CTA's units
   __shared__ int s_nonempty;                 // non-empty tiles of all units
   __shared__ int s_part[kMaxPer][kPartInts];
   __shared__ UnitSums s_u[kStatWarps];
+  __shared__ double s_below[kFillWarps][32 * kBinsPerLane];
   __shared__ int s_m[kMaxPer];               // split flag binade of instance ii0 + z
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int U = Bf.count_ctas;
   const int u0 = blockIdx.x * per_cta, u1 = min(U, u0 + per_cta);
+  const int sub = warp / kUnitWarps, wu = warp % kUnitWarps;
+  // what needs only the arguments and the instance table, while the count kernel runs
+  const int ii0 = u0 < U ? inst_of_unit(R, u0) : 0;
+  const int first = R.at(ii0).count0;   // of u0's instance
+  FillLane f = fill_lane(R, min(u0 + sub, U - 1));
+  asm volatile("" ::"r"(f.ii), "r"(f.nch), "r"(f.i), "r"(f.j), "l"(f.g), "l"(f.mask), "r"(first),
+               "l"(Bf.cnt), "l"(Bf.surv_mask), "l"(Bf.part), "l"(Bf.group), "l"(Bf.order),
+               "l"(Bf.tile_beg), "l"(Bf.k_idx), "l"(Bf.need_bits), "l"(Bf.need_list), "l"(Bf.bdev));
+  pdl_wait();
+  pdl_trigger();
   if (u0 >= U) {   // no split modes: one more CTA per instance forms its statistics
     instance_stats(R.at(blockIdx.x - (U + per_cta - 1) / per_cta), Bf, prepped != 0);
     return;
   }
-  const int ii0 = inst_of_unit(R, u0);
-  const int first = R.at(ii0).count0;   // of u0's instance
-  const int sub = warp / kUnitWarps, wu = warp % kUnitWarps;
   // the first unit of this warp: its counts and first words, on their way while
   // the totals are added up
   int count_next = 0;
   uint32_t word_next[4] = {0u, 0u, 0u, 0u};
-  if (u0 + sub < u1) {
-    const Inst& in = R.at(inst_of_unit(R, u0 + sub));
-    const Unit u = unit_at(in, u0 + sub - in.count0);
-    const int nch = (in.bk + 31) >> 5;
-    const int c = lane / u.rows, r = lane - c * u.rows;
-    if (c < u.cols) {
-      const int64_t t = (int64_t)(u.r0 + r) * in.bn + u.j0 + c;
-      count_next = __ldcg(Bf.cnt + in.tile0 + t);
+  if (u0 + sub < u1 && f.act) {
+    count_next = __ldcg(Bf.cnt + f.g);
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < nch) word_next[q] = __ldcg(Bf.surv_mask + in.mask0 + t * nch + q);
-    }
+    for (int q = 0; q < 4; ++q)
+      if (q < f.nch) word_next[q] = __ldcg(Bf.surv_mask + f.mask + q);
   }
   const int ii1 = R.any_split ? inst_of_unit(R, u1 - 1) : ii0;
   // split modes: the flag binade of every instance with units here, one warp per
@@ -1126,82 +1244,76 @@ __global__ void __launch_bounds__(kFillThreads)
       UnitSums u = unit_sums(in, Bf, 0);
       for (int v = 1; v < kStatWarps && 32 * v < units_of(in); ++v)
         merge_sums(u, unit_sums(in, Bf, v));
-      const int m = write_stats(in, Bf, u, true, in.count0 >= u0);
+      if (in.split) flag_prefix(in, s_below[warp]);
+      const int m = write_stats(in, Bf, u, true, in.count0 >= u0, s_below[warp]);
       if (lane == 0) s_m[z] = m;
     }
   }
-  const int scan_warps = lone ? kFillWarps - kStatWarps : kFillWarps;
+  // the roles up to the scan's result: the first warps add up the totals (warp 0
+  // finishes them), the last kStatWarps form a lone instance's statistics, and the
+  // kNeedWarps before the last list the blocks that the CTA's units need, which
+  // depends on neither: they only arrive at the barrier before the scan, and wait for
+  // its result on a barrier of their own
+  constexpr int kNeedWarps = kFillWarps / kUnitWarps, kNeed0 = kFillWarps - 1 - kNeedWarps;
+  const bool needs = warp >= kNeed0 && warp < kNeed0 + kNeedWarps;
+  const int scan_warps = lone ? kFillWarps - kStatWarps : kNeed0;
   const int scan_threads = scan_warps * 32;
-  if (warp >= scan_warps) {
-    stat_part(R.at(ii0), Bf, s_u, warp - scan_warps);
-  } else {
-    // per thread: totals of the buckets over all units and over those before
-    // u0; survivors of u0's instance before u0
-    int tot[kPartInts], bef[kPartInts];
+  if (lone && warp >= scan_warps) stat_part(R.at(ii0), Bf, s_u, warp - scan_warps);
+  if (warp < scan_warps) {
+    // four threads per unit, a quarter of its slots each, eight units' loads at a time:
+    // the buckets' totals over all units and over those before u0; survivors of u0's
+    // instance before u0.  (A thread per unit with all slots in registers is
+    // straight-line code of 24 warp reductions: its instruction fetches alone took 1 us.)
+    static_assert(kPartInts == 16 && kPartS == 0, "slots by quarters");
+    const int quarter = tid & 3, step = scan_threads / 4, gs = Bf.group_shift;
+    const int n = (U + (1 << gs) - 1) >> gs, ub = u0 >> gs, lb = first >> gs;
+    const int4* units = reinterpret_cast<const int4*>(Bf.part) + quarter;
+    const int4* src = gs ? reinterpret_cast<const int4*>(Bf.group) + quarter : units;
+    int4 tot = make_int4(0, 0, 0, 0), bef = tot;
+    for (int q0 = tid >> 2; q0 < n; q0 += 8 * step) {
+      int4 x[8];
 #pragma unroll
-    for (int q = 0; q < kPartInts; ++q) tot[q] = bef[q] = 0;
-    auto add = [&](int (&dst)[kPartInts], const int* p, int sign) {
-      const int4* v = reinterpret_cast<const int4*>(p);
+      for (int z = 0; z < 8; ++z)
+        x[z] = q0 + z * step < n ? __ldcg(src + (int64_t)(q0 + z * step) * 4) : make_int4(0, 0, 0, 0);
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int4 x = __ldcg(v + q);
-        dst[4 * q] += sign * x.x;
-        dst[4 * q + 1] += sign * x.y;
-        dst[4 * q + 2] += sign * x.z;
-        dst[4 * q + 3] += sign * x.w;
+      for (int z = 0; z < 8; ++z) {
+        const int q = q0 + z * step;
+        add4(tot, x[z]);
+        if (quarter == 0 && q < lb) x[z].x = 0;
+        if (q < ub) add4(bef, x[z]);
       }
-    };
-    if (Bf.group_shift == 0) {
-      for (int q = tid; q < U; q += scan_threads) {
-        int x[kPartInts];
-#pragma unroll
-        for (int z = 0; z < kPartInts; ++z) x[z] = 0;
-        add(x, Bf.part + (int64_t)q * kPartInts, 1);
-        const bool before = q < u0;
-        if (q >= first && before) bef[kPartS] += x[kPartS];
-#pragma unroll
-        for (int z = 1; z < kOrderKeys; ++z) {
-          tot[z] += x[z];
-          if (before) bef[z] += x[z];
-        }
-      }
-    } else {
-      const int gs = Bf.group_shift, ng = (U + (1 << gs) - 1) >> gs;
-      const int gu = u0 >> gs, gf = first >> gs;
-      for (int q = tid; q < ng; q += scan_threads) {
-        int x[kPartInts];
-#pragma unroll
-        for (int z = 0; z < kPartInts; ++z) x[z] = 0;
-        add(x, Bf.group + (int64_t)q * kPartInts, 1);
-        if (q < gu) bef[kPartS] += x[kPartS];
-        if (q < gf) bef[kPartS] -= x[kPartS];
-#pragma unroll
-        for (int z = 1; z < kOrderKeys; ++z) {
-          tot[z] += x[z];
-          if (q < gu) bef[z] += x[z];
-        }
-      }
-      for (int q = (gu << gs) + tid; q < u0; q += scan_threads)
-        add(bef, Bf.part + (int64_t)q * kPartInts, 1);
-      for (int q = (gf << gs) + tid; q < first; q += scan_threads)
-        bef[kPartS] -= __ldcg(Bf.part + (int64_t)q * kPartInts + kPartS);
+    }
+    if (gs) {
+      for (int q = (ub << gs) + (tid >> 2); q < u0; q += step) add4(bef, __ldcg(units + (int64_t)q * 4));
+      if (quarter == 0)
+        for (int q = (lb << gs) + (tid >> 2); q < first; q += step) bef.x -= __ldcg(units + (int64_t)q * 4).x;
     }
 #pragma unroll
-    for (int q = 0; q < kOrderKeys; ++q) {
-      const int a = __reduce_add_sync(0xffffffffu, tot[q]);
-      const int b = __reduce_add_sync(0xffffffffu, bef[q]);
-      if (lane == 0) {
-        s_red[warp][q] = a;
-        s_red[warp][kPartInts + q] = b;
-      }
+    for (int off = 4; off < 32; off <<= 1) {
+      add4(tot, shfl_xor4(tot, off));
+      add4(bef, shfl_xor4(bef, off));
+    }
+    if (lane < 4) {
+      reinterpret_cast<int4*>(s_red[warp])[lane] = tot;
+      reinterpret_cast<int4*>(s_red[warp])[4 + lane] = bef;
     }
     for (int x = tid; x < (u1 - u0) * kPartInts; x += scan_threads)
       s_part[x / kPartInts][x % kPartInts] = __ldcg(Bf.part + (int64_t)u0 * kPartInts + x);
   }
-  __syncthreads();
+  if (needs) {
+    asm volatile("bar.arrive 1, %0;" ::"n"(kFillThreads) : "memory");
+    for (int un = u0 + warp - kNeed0; un < u1; un += kNeedWarps) need_blocks(R, Bf, fill_lane(R, un));
+  } else if (lone && warp == scan_warps) {   // beside the last warp, which waits for it
+    asm volatile("bar.arrive 1, %0;" ::"n"(kFillThreads) : "memory");
+    flag_prefix(R.at(ii0), s_below[0]);
+    asm volatile("bar.arrive 4, 64;" ::: "memory");
+  } else {
+    asm volatile("bar.sync 1, %0;" ::"n"(kFillThreads) : "memory");
+  }
   if (warp == kFillWarps - 1 && lone) {
     const Inst& in = R.at(ii0);   // the CTA of its first unit also writes its statistics
-    const int m = write_stats(in, Bf, merged(s_u), true, in.count0 >= u0);
+    asm volatile("bar.sync 4, 64;" ::: "memory");
+    const int m = write_stats(in, Bf, merged(s_u), true, in.count0 >= u0, s_below[0]);
     if (lane == 0) s_m[0] = m;
   }
   if (warp == 0) {
@@ -1209,16 +1321,17 @@ __global__ void __launch_bounds__(kFillThreads)
     int a = 0, b = 0;
     if (lane < kOrderKeys)
       for (int w = 0; w < scan_warps; ++w) {
-        a += s_red[w][lane];
+        if (lane != kPartS) a += s_red[w][lane];
         b += s_red[w][kPartInts + lane];
       }
-    int below = 0;   // non-empty tiles in the buckets above this lane's
-    const int all = __reduce_add_sync(0xffffffffu, a);
+    int upto = a;   // non-empty tiles in the buckets up to this lane's
 #pragma unroll
-    for (int q = 1; q < kOrderKeys; ++q) {
-      const int x = __shfl_sync(0xffffffffu, a, q);
-      if (q > lane) below += x;
+    for (int off = 1; off < 16; off <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, upto, off);
+      if (lane >= off) upto += y;
     }
+    const int all = __shfl_sync(0xffffffffu, upto, 15);
+    const int below = all - upto;   // in those above it
     const int ne_before = __reduce_add_sync(0xffffffffu, lane >= 1 ? b : 0);
     if (lane < kOrderKeys) s_base[lane] = lane == kPartS ? b : below + b;
     if (lane == kPartNe) s_base[lane] = ne_before;
@@ -1227,19 +1340,23 @@ __global__ void __launch_bounds__(kFillThreads)
       if (blockIdx.x == 0) Bf.bdev->nonempty = all;
     }
   }
-  __syncthreads();
+  constexpr int kOthers = kFillThreads - 32 * kNeedWarps, kLate = 64 + 32 * kNeedWarps;
+  if (needs) {
+    asm volatile("bar.sync 3, %0;" ::"n"(kLate) : "memory");
+  } else {
+    if (warp == 0 || warp == kFillWarps - 1) asm volatile("bar.arrive 3, %0;" ::"n"(kLate) : "memory");
+    asm volatile("bar.sync 2, %0;" ::"n"(kOthers) : "memory");
+  }
   const int nonempty = s_nonempty;
   for (int un = u0 + sub; un < u1; un += kFillWarps / kUnitWarps) {
-    const int ii = inst_of_unit(R, un);
+    const bool first_round = un == u0 + sub;
+    if (!first_round) f = fill_lane(R, un);
+    const int ii = f.ii, nch = f.nch, r = f.r, i = f.i, j = f.j;
     const Inst& in = R.at(ii);
     const int bk = in.bk, bn = in.bn;
-    const Unit u = unit_at(in, un - in.count0);
-    const int nch = (bk + 31) >> 5;
-    const int c = lane / u.rows, r = lane - c * u.rows;
-    const bool act = c < u.cols;
-    const int i = u.r0 + r, j = u.j0 + c;
-    const int64_t t = (int64_t)i * bn + j, g = in.tile0 + t;
-    const bool first_round = un == u0 + sub;
+    const Unit u = f.u;
+    const bool act = f.act;
+    const int64_t g = f.g;
     const int count = first_round ? count_next : (act ? Bf.cnt[g] : 0);
     // lane q: the unit's first slot in bucket q, lane 0: survivors before it in
     // its instance, lane kPartNe: non-empty tiles before it
@@ -1271,8 +1388,11 @@ __global__ void __launch_bounds__(kFillThreads)
         Bf.order[nonempty + (pos - (ne0 + __popc(ne_mask & lower)))] = (int)g;
       }
     }
-    // expand the bitmask words, tile by tile (the unit's warps take turns)
-    const uint32_t* mrow = Bf.surv_mask + in.mask0 + t * nch;
+    // expand the bitmask words.  Up to 16 entries per tile on average: a lane per tile
+    // (a warp per tile spends 900 cycles on each, however few its entries are); more: a
+    // warp per tile, whose stores are coalesced
+    const bool few = __shfl_sync(0xffffffffu, incl, 31) <= 16 * 32;
+    const uint32_t* mrow = Bf.surv_mask + f.mask;
     const int split = in.split;
     const int m = split ? s_m[ii - ii0] : 0;
     const double inv = split && ne_mask ? in.pd->inv_ab : 0.0;
@@ -1283,79 +1403,64 @@ __global__ void __launch_bounds__(kFillThreads)
       for (int q = 0; q < 4; ++q)
         word[q] = first_round && w0 == 0 ? word_next[q]
                                          : (count > 0 && w0 + q < nch ? __ldg(mrow + w0 + q) : 0u);
-      unsigned todo = ne_mask;
-      int turn = 0;
-      while (todo) {
-        const int src = __ffs(todo) - 1;
-        todo &= todo - 1u;
-        if ((turn++ & (kUnitWarps - 1)) != wu) continue;
-        int at = __shfl_sync(0xffffffffu, cursor, src);
-        const int si = __shfl_sync(0xffffffffu, i, src), sj = __shfl_sync(0xffffffffu, j, src);
+      if (few) {   // a lane per tile, a warp per word, four entries at a time
+        uint32_t bits = 0u;
+        int at = cursor;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const uint32_t bits = __shfl_sync(0xffffffffu, word[q], src);
-          if (bits == 0u) continue;   // uniform over the warp
-          if ((bits >> lane) & 1u) {
-            const int k = (w0 + q) * 32 + lane;
-            uint16_t v = (uint16_t)k;
-            if (split && rel_bin(__dmul_rn(in.nA[(int64_t)si * bk + k], in.nB[(int64_t)k * bn + sj]),
-                                 inv) >= m)
-              v |= kSplitFlag;
-            Bf.k_idx[at + __popc(bits & lower)] = v;
+          if (q == wu) bits = word[q];
+          if (q < wu) at += __popc(word[q]);
+        }
+        const int k0 = (w0 + wu) * 32;
+        while (bits) {
+          int k[4], v[4];
+#pragma unroll
+          for (int z = 0; z < 4; ++z) {
+            v[z] = k[z] = bits ? k0 + __ffs(bits) - 1 : -1;
+            bits &= bits - 1u;
           }
-          at += __popc(bits);
+          if (split) {
+            double pa[4], pb[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+              pa[z] = k[z] >= 0 ? in.nA[(int64_t)i * bk + k[z]] : 0.0;
+              pb[z] = k[z] >= 0 ? in.nB[(int64_t)k[z] * bn + j] : 0.0;
+            }
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+              if (k[z] >= 0 && rel_bin(__dmul_rn(pa[z], pb[z]), inv) >= m) v[z] |= kSplitFlag;
+          }
+#pragma unroll
+          for (int z = 0; z < 4; ++z)
+            if (k[z] >= 0) Bf.k_idx[at++] = (uint16_t)v[z];
+        }
+      } else {
+        unsigned todo = ne_mask;
+        int turn = 0;
+        while (todo) {
+          const int src = __ffs(todo) - 1;
+          todo &= todo - 1u;
+          if ((turn++ & (kUnitWarps - 1)) != wu) continue;
+          int at = __shfl_sync(0xffffffffu, cursor, src);
+          const int si = __shfl_sync(0xffffffffu, i, src), sj = __shfl_sync(0xffffffffu, j, src);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t bits = __shfl_sync(0xffffffffu, word[q], src);
+            if (bits == 0u) continue;   // uniform over the warp
+            if ((bits >> lane) & 1u) {
+              const int k = (w0 + q) * 32 + lane;
+              uint16_t v = (uint16_t)k;
+              if (split && rel_bin(__dmul_rn(in.nA[(int64_t)si * bk + k], in.nB[(int64_t)k * bn + sj]),
+                                   inv) >= m)
+                v |= kSplitFlag;
+              Bf.k_idx[at + __popc(bits & lower)] = v;
+            }
+            at += __popc(bits);
+          }
         }
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) cursor += __popc(word[q]);
-      if (in.quant && wu == kUnitWarps - 1) {
-        // the blocks of A and B that the unit's triples use: lane x < rows holds row x
-        // of A, the next cols lanes the columns of B, 32 k per word; the four words'
-        // round trips go out together
-        uint32_t mine[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          mine[q] = 0u;
-          if (!__any_sync(0xffffffffu, word[q] != 0u)) continue;
-          for (int x = 0; x < u.rows + u.cols; ++x) {
-            const bool in_set = x < u.rows ? r == x : c == x - u.rows;
-            const uint32_t o = __reduce_or_sync(0xffffffffu, in_set ? word[q] : 0u);
-            if (lane == x) mine[q] = o;
-          }
-        }
-        const bool isB = lane >= u.rows;
-        const int bi = isB ? u.j0 + lane - u.rows : u.r0 + lane;   // column of B / row of A
-        uint32_t* w = Bf.need_bits + (isB ? Bf.need_words_a + in.needb0 : in.needa0) +
-                      (int64_t)bi * nch + w0;
-        uint32_t fresh[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)   // a plain read first: a bit once set stays set
-          fresh[q] = mine[q] ? mine[q] & ~__ldcg(w + q) : 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (fresh[q]) fresh[q] = mine[q] & ~atomicOr(w + q, mine[q]);
-        int n = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) n += __popc(fresh[q]);
-        int end = n;
-        for (int off = 1; off < 32; off <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, end, off);
-          if (lane >= off) end += y;
-        }
-        const int total = __shfl_sync(0xffffffffu, end, 31);
-        if (total > 0) {
-          int at = 0;
-          if (lane == 0) at = atomicAdd(&Bf.bdev->need_count, total);
-          at = __shfl_sync(0xffffffffu, at, 0) + end - n;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            for (; fresh[q]; fresh[q] &= fresh[q] - 1u) {
-              const int64_t k = (w0 + q) * 32 + __ffs(fresh[q]) - 1;
-              Bf.need_list[at++] = isB ? (uint32_t)(in.bblk0 + k * bn + bi) | 0x80000000u
-                                       : (uint32_t)(in.ablk0 + (int64_t)bi * bk + k);
-            }
-        }
-      }
     }
   }
 }
