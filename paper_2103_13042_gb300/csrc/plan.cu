@@ -339,24 +339,24 @@ __global__ void __launch_bounds__(kPrepThreads)
   }
 }
 
-// ||A||_F (lane 0) and ||B||_F (lane 1) from `count` partial sums at `first`, by one
+// ||A||_F^2 (lane 0) and ||B||_F^2 (lane 1) from `count` partial sums at `first`, by one
 // warp in a fixed order (every caller gets the same bits): the even lanes add up
-// A's, the odd ones B's, one square root serves both (FP64 is scarce here).
-__device__ __forceinline__ double sum_norms(const PlanBuffers& Bf, int first, int count) {
+// A's, the odd ones B's, so that one square root serves both (FP64 is scarce here).
+__device__ __forceinline__ double sum_norms2(const PlanBuffers& Bf, int first, int count) {
   const int lane = threadIdx.x & 31;
   const double* p = ((lane & 1) ? Bf.part_b : Bf.part_a) + first;
   double x = 0.0;
 #pragma unroll 4
   for (int i = lane >> 1; i < count; i += 16) x += __ldcg(p + i);
   for (int off = 16; off > 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-  return sqrt(x);
+  return x;
 }
 
 // After prep: 1 / (||A|| ||B||) for a CTA of the instance (one warp calls it);
 // `publish`: also write the norms to the instance's statistics.
 __device__ __forceinline__ double instance_norms(const Inst& in, const PlanBuffers& Bf,
                                                  bool publish) {
-  const double x = sum_norms(Bf, in.prep0, prep_parts(in));
+  const double x = sqrt(sum_norms2(Bf, in.prep0, prep_parts(in)));
   const double na = __shfl_sync(0xffffffffu, x, 0), nb = __shfl_sync(0xffffffffu, x, 1);
   const double ab = na * nb, inv = ab > 0.0 ? 1.0 / ab : 0.0;
   if (publish && (threadIdx.x & 31) == 0) {
@@ -423,7 +423,8 @@ struct UnitSums {
 // One warp's part v of an instance's sums: its lane l takes the units 32 v + l,
 // 32 v + l + 32 kStatWarps, ... (four units' loads at a time).  The kStatWarps parts
 // are merged in order (merge_sums), whoever forms them, so that a single call and
-// a batch give the same bits.
+// a batch give the same bits.  WHAT: 1 the counts and b1, 2 b2, 3 all.
+template <int WHAT>
 __device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers& Bf, int v) {
   const int units = units_of(in);
   constexpr int nt = 32 * kStatWarps;
@@ -438,8 +439,10 @@ __device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers&
       s4[z] = 0;
       hi[z] = bb[z] = make_int4(0, 0, 0, 0);
       if (q0 + z * nt < units) {
-        s4[z] = __ldcg(Bf.part + q * kPartInts + kPartS);
-        hi[z] = __ldcg(reinterpret_cast<const int4*>(Bf.part + q * kPartInts + kPartNe));
+        if (WHAT & 1) {
+          s4[z] = __ldcg(Bf.part + q * kPartInts + kPartS);
+          hi[z] = __ldcg(reinterpret_cast<const int4*>(Bf.part + q * kPartInts + kPartNe));
+        }
         bb[z] = __ldcg(reinterpret_cast<const int4*>(Bf.part_bound + 2 * q));
       }
     }
@@ -448,15 +451,17 @@ __device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers&
       r.S += s4[z];
       r.ne += hi[z].x;
       r.km = max(r.km, hi[z].y);
-      ext_add(r.b1, __int_as_float(bb[z].x), bb[z].y);
-      ext_add(r.b2, __int_as_float(bb[z].z), bb[z].w);
+      if (WHAT & 1) ext_add(r.b1, __int_as_float(bb[z].x), bb[z].y);
+      if (WHAT & 2) ext_add(r.b2, __int_as_float(bb[z].z), bb[z].w);
     }
   }
-  r.S = __reduce_add_sync(0xffffffffu, r.S);
-  r.ne = __reduce_add_sync(0xffffffffu, r.ne);
-  r.km = __reduce_max_sync(0xffffffffu, r.km);
-  r.b1 = ext_warp_sum(r.b1);
-  r.b2 = ext_warp_sum(r.b2);
+  if (WHAT & 1) {
+    r.S = __reduce_add_sync(0xffffffffu, r.S);
+    r.ne = __reduce_add_sync(0xffffffffu, r.ne);
+    r.km = __reduce_max_sync(0xffffffffu, r.km);
+    r.b1 = ext_warp_sum(r.b1);
+  }
+  if (WHAT & 2) r.b2 = ext_warp_sum(r.b2);
   return r;
 }
 
@@ -468,18 +473,32 @@ __device__ __forceinline__ void merge_sums(UnitSums& u, const UnitSums& v) {
   ext_add(u.b2, v.b2.m, v.b2.e);
 }
 
-// The statistics of one instance from its sums, by one warp (one square root and
-// one division for all of them).  prepped: the count kernel left the norms in the
-// statistics; otherwise they come from the units' partial sums and are written
-// too.  Returns the split-flag binade (below: flag_prefix's sums); publish = false:
-// only that.
-__device__ __forceinline__ int write_stats(const Inst& in, const PlanBuffers& Bf, const UnitSums& u,
-                                           bool prepped, bool publish, const double* below) {
+// The statistics of one instance from the parts of its sums, by one warp: lane 2 merges
+// the parts of b2, the others those of b1; one square root and one division for all of
+// them.  norm2: the operands' squared norms, which are then written too; null: the count
+// kernel left the norms in the statistics.  Returns the split-flag binade (below:
+// flag_prefix's sums); publish = false: only that.
+__device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts, int nparts,
+                                           const double* norm2, bool publish, const double* below) {
   const int lane = threadIdx.x & 31;
+  const bool prepped = norm2 == nullptr;
   PlanDevice* pd = in.pd;
-  double x = prepped ? 0.0 : sum_norms(Bf, in.count0, units_of(in));
-  if (lane == 2) x = sqrt(ext_value(u.b2));
-  if (prepped && lane < 2) x = __ldcg(lane ? &pd->norm_b : &pd->norm_a);
+  double x = 0.0;
+  if (lane < 2) x = prepped ? __ldcg(lane ? &pd->norm_b : &pd->norm_a) : norm2[lane];
+  UnitSums u = parts[0];
+  // (parts formed for the binade only hold no b1)
+  const ExtSum none{0.0f, 0};
+  ExtSum bound = lane == 2 ? u.b2 : (publish ? u.b1 : none);
+#pragma unroll 1
+  for (int v = 1; v < nparts; ++v) {
+    const ExtSum y = lane == 2 ? parts[v].b2 : (publish ? parts[v].b1 : none);
+    ext_add(bound, y.m, y.e);
+    u.S += parts[v].S;
+    u.ne += parts[v].ne;
+    u.km = max(u.km, parts[v].km);
+  }
+  const double root = sqrt(lane == 2 ? ext_value(bound) : x);
+  if (lane == 2 || !prepped) x = root;
   const double na = __shfl_sync(0xffffffffu, x, 0), nb = __shfl_sync(0xffffffffu, x, 1);
   const double bound2 = __shfl_sync(0xffffffffu, x, 2);
   const double ab = na * nb;
@@ -503,7 +522,7 @@ __device__ __forceinline__ int write_stats(const Inst& in, const PlanBuffers& Bf
       pd->norm_b = nb;
       pd->inv_ab = ab > 0.0 ? quot : 0.0;
     }
-    pd->bound1 = ext_value(u.b1);
+    pd->bound1 = ext_value(bound);
     pd->bound2 = bound2;
     pd->valid_ratio = ratio;
     pd->flag_exp = m;
@@ -513,27 +532,41 @@ __device__ __forceinline__ int write_stats(const Inst& in, const PlanBuffers& Bf
 }
 
 // Part v of one instance's sums into shared memory, by one warp.
+template <int WHAT>
 __device__ __forceinline__ void stat_part(const Inst& in, const PlanBuffers& Bf, UnitSums* parts,
                                           int v) {
-  const UnitSums u = unit_sums(in, Bf, v);
-  if ((threadIdx.x & 31) == 0) parts[v] = u;
+  const UnitSums u = unit_sums<WHAT>(in, Bf, v);
+  if ((threadIdx.x & 31) != 0) return;
+  if (WHAT & 1) {
+    parts[v].S = u.S;
+    parts[v].ne = u.ne;
+    parts[v].km = u.km;
+    parts[v].b1 = u.b1;
+  }
+  if (WHAT & 2) parts[v].b2 = u.b2;
 }
 
-__device__ __forceinline__ UnitSums merged(const UnitSums* parts) {
-  UnitSums u = parts[0];
-  for (int v = 1; v < kStatWarps; ++v) merge_sums(u, parts[v]);
-  return u;
-}
-
-// The statistics of one instance by a CTA of kStatWarps warps or more.
+// The statistics of one instance by a CTA of kStatWarps warps, or twice as many: then
+// the second half forms b2.  The norms (not prepped) are added up beside.
 __device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped) {
   __shared__ UnitSums s_u[kStatWarps];
-  __shared__ double s_below[32 * kBinsPerLane];
-  if (threadIdx.x / 32 < kStatWarps) stat_part(in, Bf, s_u, threadIdx.x / 32);
-  if (threadIdx.x < 32 && in.split) flag_prefix(in, s_below);
+  __shared__ double s_below[32 * kBinsPerLane], s_norm2[2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (!prepped && warp == kStatWarps - 1) {
+    const double x = sum_norms2(Bf, in.count0, units_of(in));
+    if (lane < 2) s_norm2[lane] = x;
+  }
+  if (blockDim.x < 2 * 32 * kStatWarps)
+    stat_part<3>(in, Bf, s_u, warp);
+  else if (warp < kStatWarps)
+    stat_part<1>(in, Bf, s_u, warp);
+  else if (warp < 2 * kStatWarps)
+    stat_part<2>(in, Bf, s_u, warp - kStatWarps);
+  if (warp == 0 && in.split) flag_prefix(in, s_below);
   __syncthreads();
-  if (threadIdx.x < 32) (void)write_stats(in, Bf, merged(s_u), prepped, true, s_below);
+  if (warp == 0) (void)write_stats(in, s_u, kStatWarps, prepped ? nullptr : s_norm2, true, s_below);
 }
+
 
 // Screens of one staged row or column: whole words of 32 k (the tail holds
 // zero norms) and two more, so that the rows start 16 bytes apart modulo the
@@ -1203,7 +1236,7 @@ __global__ void __launch_bounds__(kFillThreads)
   __shared__ int s_base[kPartInts];          // buckets 1 .. 11: first slots of the CTA's units
   __shared__ int s_nonempty;                 // non-empty tiles of all units
   __shared__ int s_part[kMaxPer][kPartInts];
-  __shared__ UnitSums s_u[kStatWarps];
+  __shared__ UnitSums s_u[kStatWarps], s_w[kFillWarps];
   __shared__ double s_below[kFillWarps][32 * kBinsPerLane];
   __shared__ int s_m[kMaxPer];               // split flag binade of instance ii0 + z
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1241,11 +1274,13 @@ __global__ void __launch_bounds__(kFillThreads)
   if (R.any_split && !lone) {
     for (int z = warp; z <= ii1 - ii0; z += kFillWarps) {
       const Inst& in = R.at(ii0 + z);
-      UnitSums u = unit_sums(in, Bf, 0);
+      UnitSums u = unit_sums<3>(in, Bf, 0);
       for (int v = 1; v < kStatWarps && 32 * v < units_of(in); ++v)
-        merge_sums(u, unit_sums(in, Bf, v));
+        merge_sums(u, unit_sums<3>(in, Bf, v));
       if (in.split) flag_prefix(in, s_below[warp]);
-      const int m = write_stats(in, Bf, u, true, in.count0 >= u0, s_below[warp]);
+      if (lane == 0) s_w[warp] = u;
+      __syncwarp();
+      const int m = write_stats(in, s_w + warp, 1, nullptr, in.count0 >= u0, s_below[warp]);
       if (lane == 0) s_m[z] = m;
     }
   }
@@ -1258,7 +1293,11 @@ __global__ void __launch_bounds__(kFillThreads)
   const bool needs = warp >= kNeed0 && warp < kNeed0 + kNeedWarps;
   const int scan_warps = lone ? kFillWarps - kStatWarps : kNeed0;
   const int scan_threads = scan_warps * 32;
-  if (lone && warp >= scan_warps) stat_part(R.at(ii0), Bf, s_u, warp - scan_warps);
+  if (lone && warp >= scan_warps) {   // the counts and b1: for the CTA that writes them
+    const Inst& in = R.at(ii0);
+    if (in.count0 >= u0) stat_part<3>(in, Bf, s_u, warp - scan_warps);
+    else stat_part<2>(in, Bf, s_u, warp - scan_warps);
+  }
   if (warp < scan_warps) {
     // four threads per unit, a quarter of its slots each, eight units' loads at a time:
     // the buckets' totals over all units and over those before u0; survivors of u0's
@@ -1313,7 +1352,7 @@ __global__ void __launch_bounds__(kFillThreads)
   if (warp == kFillWarps - 1 && lone) {
     const Inst& in = R.at(ii0);   // the CTA of its first unit also writes its statistics
     asm volatile("bar.sync 4, 64;" ::: "memory");
-    const int m = write_stats(in, Bf, merged(s_u), true, in.count0 >= u0, s_below[0]);
+    const int m = write_stats(in, s_u, kStatWarps, nullptr, in.count0 >= u0, s_below[0]);
     if (lane == 0) s_m[0] = m;
   }
   if (warp == 0) {
