@@ -236,11 +236,31 @@ __device__ __forceinline__ ExtSum ext_warp_sum_fast(ExtSum s) {
   return r;
 }
 
+// ext_add without branches (the same bits): for short sums on a critical path, whose
+// lanes would take every side of them.
+__device__ __forceinline__ void ext_add_flat(ExtSum& s, float q, int E) {
+  const int ea = s.e + fexp(s.m), eb = E + fexp(q);
+  const bool any = q > 0.0f, none = s.m == 0.0f;
+  const bool take = any && (none || eb > ea + 40);
+  const bool both = any && !none && eb <= ea + 40 && eb >= ea - 40;
+  float m = __fmaf_rn(q, pow2f(min(max(E - s.e, -84), 84)), s.m);
+  int e = s.e;
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {   // renormalise (m < 2^83)
+    const bool big = m >= 1099511627776.0f;
+    m = big ? m * pow2f(-40) : m;
+    e += big ? 40 : 0;
+  }
+  s.m = take ? q : (both ? m : s.m);
+  s.e = take ? E : (both ? e : s.e);
+}
+
 __device__ __forceinline__ ExtSum ext_warp_sum(ExtSum s) {
+#pragma unroll 1
   for (int off = 16; off > 0; off >>= 1) {
     const float m = __shfl_xor_sync(0xffffffffu, s.m, off);
     const int e = __shfl_xor_sync(0xffffffffu, s.e, off);
-    ext_add(s, m, e);
+    ext_add_flat(s, m, e);
   }
   return s;
 }
@@ -451,8 +471,8 @@ __device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers&
       r.S += s4[z];
       r.ne += hi[z].x;
       r.km = max(r.km, hi[z].y);
-      if (WHAT & 1) ext_add(r.b1, __int_as_float(bb[z].x), bb[z].y);
-      if (WHAT & 2) ext_add(r.b2, __int_as_float(bb[z].z), bb[z].w);
+      if (WHAT & 1) ext_add_flat(r.b1, __int_as_float(bb[z].x), bb[z].y);
+      if (WHAT & 2) ext_add_flat(r.b2, __int_as_float(bb[z].z), bb[z].w);
     }
   }
   if (WHAT & 1) {
@@ -469,8 +489,8 @@ __device__ __forceinline__ void merge_sums(UnitSums& u, const UnitSums& v) {
   u.S += v.S;
   u.ne += v.ne;
   u.km = max(u.km, v.km);
-  ext_add(u.b1, v.b1.m, v.b1.e);
-  ext_add(u.b2, v.b2.m, v.b2.e);
+  ext_add_flat(u.b1, v.b1.m, v.b1.e);
+  ext_add_flat(u.b2, v.b2.m, v.b2.e);
 }
 
 // The statistics of one instance from the parts of its sums, by one warp: lane 2 merges
@@ -479,7 +499,8 @@ __device__ __forceinline__ void merge_sums(UnitSums& u, const UnitSums& v) {
 // kernel left the norms in the statistics.  Returns the split-flag binade (below:
 // flag_prefix's sums); publish = false: only that.
 __device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts, int nparts,
-                                           const double* norm2, bool publish, const double* below) {
+                                           const double* norm2, bool full, bool publish,
+                                           const double* below) {
   const int lane = threadIdx.x & 31;
   const bool prepped = norm2 == nullptr;
   PlanDevice* pd = in.pd;
@@ -488,11 +509,11 @@ __device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts
   UnitSums u = parts[0];
   // (parts formed for the binade only hold no b1)
   const ExtSum none{0.0f, 0};
-  ExtSum bound = lane == 2 ? u.b2 : (publish ? u.b1 : none);
+  ExtSum bound = lane == 2 ? u.b2 : (full ? u.b1 : none);
 #pragma unroll 1
   for (int v = 1; v < nparts; ++v) {
-    const ExtSum y = lane == 2 ? parts[v].b2 : (publish ? parts[v].b1 : none);
-    ext_add(bound, y.m, y.e);
+    const ExtSum y = lane == 2 ? parts[v].b2 : (full ? parts[v].b1 : none);
+    ext_add_flat(bound, y.m, y.e);
     u.S += parts[v].S;
     u.ne += parts[v].ne;
     u.km = max(u.km, parts[v].km);
@@ -503,7 +524,7 @@ __device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts
   const double bound2 = __shfl_sync(0xffffffffu, x, 2);
   const double ab = na * nb;
   const int m = in.split ? flag_pick(in, ab, bound2, below) : kFlagBinMin - 1;
-  if (!publish) return m;
+  if (!full) return m;
   const double cube = (double)in.bm * (double)in.bk * (double)in.bn;
   const double quot = (lane == 0 ? 1.0 : (double)u.S) / (lane == 0 ? ab : cube);
   const double ratio = __shfl_sync(0xffffffffu, quot, 1);
@@ -513,7 +534,7 @@ __device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts
       if (kFlagBinMin + b >= m) f += (long long)__ldcg(&pd->bin_cnt[b]);
     for (int off = 16; off > 0; off >>= 1) f += __shfl_xor_sync(0xffffffffu, f, off);
   }
-  if (lane == 0) {
+  if (lane == 0 && publish) {
     pd->survivors = u.S;
     pd->max_tile = u.km;
     pd->nonempty = u.ne;
@@ -548,7 +569,8 @@ __device__ __forceinline__ void stat_part(const Inst& in, const PlanBuffers& Bf,
 
 // The statistics of one instance by a CTA of kStatWarps warps, or twice as many: then
 // the second half forms b2.  The norms (not prepped) are added up beside.
-__device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped) {
+__device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped,
+                                            bool publish) {
   __shared__ UnitSums s_u[kStatWarps];
   __shared__ double s_below[32 * kBinsPerLane], s_norm2[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -564,7 +586,7 @@ __device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& B
     stat_part<2>(in, Bf, s_u, warp - kStatWarps);
   if (warp == 0 && in.split) flag_prefix(in, s_below);
   __syncthreads();
-  if (warp == 0) (void)write_stats(in, s_u, kStatWarps, prepped ? nullptr : s_norm2, true, s_below);
+  if (warp == 0) (void)write_stats(in, s_u, kStatWarps, prepped ? nullptr : s_norm2, true, publish, s_below);
 }
 
 
@@ -813,7 +835,7 @@ __global__ void __launch_bounds__(kCountThreads)
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  instance_stats(in, Bf, true);
+  instance_stats(in, Bf, true, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -1250,12 +1272,22 @@ __global__ void __launch_bounds__(kFillThreads)
   asm volatile("" ::"r"(f.ii), "r"(f.nch), "r"(f.i), "r"(f.j), "l"(f.g), "l"(f.mask), "r"(first),
                "l"(Bf.cnt), "l"(Bf.surv_mask), "l"(Bf.part), "l"(Bf.group), "l"(Bf.order),
                "l"(Bf.tile_beg), "l"(Bf.k_idx), "l"(Bf.need_bits), "l"(Bf.need_list), "l"(Bf.bdev));
-  pdl_wait();
-  pdl_trigger();
   if (u0 >= U) {   // no split modes: one more CTA per instance forms its statistics
-    instance_stats(R.at(blockIdx.x - (U + per_cta - 1) / per_cta), Bf, prepped != 0);
+    // twice: the first pass, while the count kernel still runs, only fetches the
+    // instructions (its sums are of whatever is there, and are not published)
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      if (pass == 1) {
+        pdl_wait();
+        pdl_trigger();
+      }
+      instance_stats(R.at(blockIdx.x - (U + per_cta - 1) / per_cta), Bf, prepped != 0, pass == 1);
+      __syncthreads();
+    }
     return;
   }
+  pdl_wait();
+  pdl_trigger();
   // the first unit of this warp: its counts and first words, on their way while
   // the totals are added up
   int count_next = 0;
@@ -1280,7 +1312,7 @@ __global__ void __launch_bounds__(kFillThreads)
       if (in.split) flag_prefix(in, s_below[warp]);
       if (lane == 0) s_w[warp] = u;
       __syncwarp();
-      const int m = write_stats(in, s_w + warp, 1, nullptr, in.count0 >= u0, s_below[warp]);
+      const int m = write_stats(in, s_w + warp, 1, nullptr, in.count0 >= u0, true, s_below[warp]);
       if (lane == 0) s_m[z] = m;
     }
   }
@@ -1352,7 +1384,7 @@ __global__ void __launch_bounds__(kFillThreads)
   if (warp == kFillWarps - 1 && lone) {
     const Inst& in = R.at(ii0);   // the CTA of its first unit also writes its statistics
     asm volatile("bar.sync 4, 64;" ::: "memory");
-    const int m = write_stats(in, s_u, kStatWarps, nullptr, in.count0 >= u0, s_below[0]);
+    const int m = write_stats(in, s_u, kStatWarps, nullptr, in.count0 >= u0, true, s_below[0]);
     if (lane == 0) s_m[0] = m;
   }
   if (warp == 0) {
