@@ -35,10 +35,12 @@ int32_t* device_status_word();
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch: a kernel of the plan -> rounding -> multiply
 // chain is launched while its predecessor in the stream still runs (its CTAs
-// are placed and set up early); it calls pdl_wait() before anything else, which
-// returns once the predecessor grid has completed and its writes are visible.
-// Every kernel so launched waits unconditionally at its top, so completion
-// stays transitive along the chain.  pdl_trigger() lets the successor launch.
+// are placed and set up early); it calls pdl_wait(), which returns once the
+// predecessor grid has completed and its writes are visible, before it reads what
+// that grid writes and before it writes anything.  A kernel calls pdl_trigger(), which
+// lets the successor launch, only after its own wait, so completion stays transitive
+// along the chain: what was complete before the predecessor's wait (the arguments'
+// tables, for a multiply also the plan) may be read before the own one.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {

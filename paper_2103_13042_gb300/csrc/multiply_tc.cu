@@ -198,8 +198,10 @@ __global__ void __launch_bounds__(TcCfg<FMT, LEAF, SPLITMODE>::kThreads, 1)
   fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   // the set-up above (barriers, tensor memory) overlaps the previous kernel's
-  // tail; everything below reads what it wrote
-  pdl_wait();
+  // tail; everything below reads what it wrote.  The previous kernel is the rounding,
+  // placed once the plan was complete: the scheduler reads its first tiles' queues
+  // before it waits, which it does for the blocks' scales.
+  if (warp != 2) pdl_wait();
   const int ne = p.Bf.bdev->nonempty;
 
   if (warp == 2) {
@@ -284,6 +286,7 @@ __global__ void __launch_bounds__(TcCfg<FMT, LEAF, SPLITMODE>::kThreads, 1)
         const int i = (int)(lt / bnu), j = (int)(lt % bnu);
         const int ga = (int)(a0u + (int64_t)i * bku + k), gb = (int)(b0u + (int64_t)k * bnu + j);
         int32_t sexp = 0;
+        pdl_wait();
         if (act) sexp = p.img.ea[ga] + p.img.eb[gb];
         const bool split = SPLITMODE == 2 || (SPLITMODE == 1 && (ent & 0x8000u));
         const int32_t key = sexp * 2 + (split ? 1 : 0);
