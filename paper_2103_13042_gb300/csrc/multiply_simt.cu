@@ -10,15 +10,18 @@
 // entries of the tile (32 x 32 at leaf 32), a thread 8 rows x 8 (4) columns: rows
 // ty + 4 u, columns 4 tx .. 4 tx + 3 and 32 further on, so that the distinct
 // addresses of every shared-memory read fall into different banks.
-// The surviving k are streamed in slices of 16 of the inner dimension through a
-// three-stage ring filled by asynchronous copies (16 bytes where rows are
+// The surviving k are streamed in slices of the inner dimension through a ring of
+// stages filled by asynchronous copies (16 bytes where rows are
 // aligned, else 4; entries outside the matrix are filled with zeros), A as rows,
 // B as rows: neither is transposed.  The products accumulate in FP32 FMA over the
 // surviving k in increasing order, two columns per instruction (packed
 // fma.rn.f32x2: the same FP32 rate, half the issue slots).  Bound by the FP32 pipe
-// on dense skip sets: 45, 48 and 41 TFLOP/s at leaf 32, 64 and 128 (n = 4096,
+// on dense skip sets: 48, 49 and 44 TFLOP/s at leaf 32, 64 and 128 (n = 4096,
 // 30% of the triples; 256 threads per tile with transposed A slices: 19, 30 and
-// 29), 41 at leaf 64 with unaligned rows (26).
+// 29), 42 at leaf 64 with unaligned rows (26).  Slices of 32 in two stages instead of
+// 16 in three give 45 -> 48 and 42 -> 44 at leaf 32 and 128; at leaf 64 49 -> 52, but
+// lists of 2 to 3 blocks become 6% slower (the first slice is all that a tile has on its
+// way at its start), so it keeps 16.
 #include <algorithm>
 
 #include "tc_common.cuh"
@@ -26,10 +29,6 @@
 namespace spamm {
 namespace {
 
-constexpr int kSlice = 16;
-constexpr int kStages = 3;
-constexpr int kLdA = kSlice + 4;   // floats per staged row of A: 16-byte rows, four rows apart in
-                                   // different banks
 // Outputs up to this size: the multiply writes the empty tiles itself (a second
 // kernel on a side stream costs more than their stores)
 constexpr int64_t kOwnZeroBytes = (int64_t)64 << 20;
@@ -38,12 +37,15 @@ template <int LEAF>
 struct SimtTile {
   static constexpr int kWarps = LEAF == 128 ? 8 : (LEAF == 64 ? 2 : 1);
   static constexpr int kThreads = 32 * kWarps;
+  // slices of the inner dimension, stages of the ring
+  static constexpr int kSlice = LEAF == 64 ? 16 : 32, kStages = LEAF == 64 ? 3 : 2;
+  static constexpr int kLdA = kSlice + 4;   // floats per staged row of A: 16-byte rows, four
+                                            // rows apart in different banks
   static constexpr int TN = LEAF == 32 ? 4 : 8;                      // columns per thread
   static constexpr int kWarpCols = 8 * TN;                           // 64, 32 at leaf 32
   static constexpr int kStageFloats = LEAF * kLdA + kSlice * LEAF;   // A rows, then B rows
   static constexpr size_t kSmem = (size_t)kStages * kStageFloats * sizeof(float);
-  static constexpr int kPieces = LEAF * kSlice / 4 / kThreads;       // 16-byte pieces per thread
-    // groups per CTA, one CTA per SM: 168 registers per thread at leaf 32 and 64 (8 and 16
+  // groups per CTA, one CTA per SM: 168 registers per thread at leaf 32 and 64 (8 and 16
   // groups at 128 registers spill: 37 and 42 TFLOP/s against 48 and 45)
   static constexpr int kGroups = LEAF == 128 ? 1 : (LEAF == 64 ? 6 : 12);
   static constexpr int kCtaThreads = kGroups * kThreads;
@@ -140,6 +142,7 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
     simt_kernel(InstRef R, PlanBuffers Bf, int dynamic, int zeros) {
   using T = SimtTile<LEAF>;
   constexpr int TN = T::TN, kHalves = TN / 4;
+  constexpr int kSlice = T::kSlice, kStages = T::kStages, kLdA = T::kLdA;
   extern __shared__ __align__(16) float smem_all[];
   __shared__ int s_taken;               // tiles of this SM handed to its groups
   __shared__ int s_next[T::kGroups];
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
             const float f = e == 0 ? a[u].x : a[u].y;
             const uint64_t aa = pair(f, f);
 #pragma unroll
-            for (int v = 0; v < TN / 2; ++v) acc[u][v] = fma2(aa, b[v], acc[u][v]);
+            for (int v = 0; v < TN / 2; ++v) acc[u][v] = fma2(b[v], aa, acc[u][v]);
           }
         }
       }
