@@ -596,27 +596,49 @@ __device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& B
 __host__ __device__ __forceinline__ int staged_len(int bk) { return ((bk + 31) & ~31) + 2; }
 
 // A unit's screens into shared memory (rows of A, then columns of B, their
-// exponents relative to eT), by kCountThreads threads.
+// exponents relative to eT), by kCountThreads threads.  Units of four columns: a warp
+// takes two rows of A and a quarter of B's (k, column) pairs of 32 k (whole 32-byte
+// sectors), four times 32 k at a time: twelve loads in flight, one round trip up to 128
+// blocks (rows and columns in turn took three).
 __device__ __forceinline__ void stage_unit(const Inst& in, const Unit& u, Screen* sa, Screen* sb,
                                            int eT) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bk = in.bk, bn = in.bn, len = staged_len(bk), kpad = len - 2;
   const double* __restrict__ nA = in.nA;
   const double* __restrict__ nB = in.nB;
-  for (int x = warp; x < u.rows; x += kCountWarps) {
-    const double* src = nA + (int64_t)(u.r0 + x) * bk;
-#pragma unroll 8
-    for (int k = lane; k < kpad; k += 32) sa[x * len + k] = test_screen(k < bk ? src[k] : 0.0);
-  }
-  if (u.cols == 4) {   // lanes over (k, column): whole 32-byte sectors
-#pragma unroll 8
-    for (int x = tid; x < 4 * kpad; x += kCountThreads) {
-      const int k = x >> 2, c = x & 3;
-      Screen b = test_screen(k < bk ? nB[(int64_t)k * bn + u.j0 + c] : 0.0);
-      b.e -= eT;
-      sb[c * len + k] = b;
+  if (u.cols == 4) {
+    static_assert(kBandRows <= 2 * kCountWarps && kCountThreads == 128, "two rows, one pair");
+    const int x1 = warp + kCountWarps, kb = tid >> 2, c = tid & 3;
+    const bool has0 = warp < u.rows, has1 = x1 < u.rows;
+    const double* a0 = nA + (int64_t)(u.r0 + warp) * bk;
+    const double* a1 = a0 + (int64_t)kCountWarps * bk;
+    const double* b0 = nB + u.j0 + c;
+    for (int w0 = 0; w0 < kpad; w0 += 128) {
+      double v[3][4];
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int k = w0 + 32 * z + lane, k2 = w0 + 32 * z + kb;
+        v[0][z] = has0 && k < bk ? a0[k] : 0.0;
+        v[1][z] = has1 && k < bk ? a1[k] : 0.0;
+        v[2][z] = k2 < bk ? b0[(int64_t)k2 * bn] : 0.0;
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        const int k = w0 + 32 * z + lane, k2 = w0 + 32 * z + kb;
+        if (w0 + 32 * z >= kpad) break;
+        if (has0) sa[warp * len + k] = test_screen(v[0][z]);
+        if (has1) sa[x1 * len + k] = test_screen(v[1][z]);
+        Screen b = test_screen(v[2][z]);
+        b.e -= eT;
+        sb[c * len + k2] = b;
+      }
     }
   } else {
+    for (int x = warp; x < u.rows; x += kCountWarps) {
+      const double* src = nA + (int64_t)(u.r0 + x) * bk;
+#pragma unroll 8
+      for (int k = lane; k < kpad; k += 32) sa[x * len + k] = test_screen(k < bk ? src[k] : 0.0);
+    }
     for (int k = tid; k < kpad; k += kCountThreads)
 #pragma unroll 4
       for (int c = 0; c < u.cols; ++c) {
@@ -636,8 +658,6 @@ __device__ __forceinline__ void stage_unit(const Inst& in, const Unit& u, Screen
 template <bool SPLIT, bool BAND>
 __global__ void __launch_bounds__(kCountThreads)
     count_kernel(InstRef R, PlanBuffers Bf, int prepped, int stats) {
-  pdl_wait();
-  pdl_trigger();
   extern __shared__ __align__(16) Screen s_scr[];   // [rows][len] of A, then [cols][len] of B
   __shared__ double s_bin_sum[SPLIT ? kFlagBins : 1];
   __shared__ int s_bin_cnt[SPLIT ? kFlagBins : 1];
@@ -655,6 +675,10 @@ __global__ void __launch_bounds__(kCountThreads)
   const double* __restrict__ nA = in.nA;
   const double* __restrict__ nB = in.nB;
   const TestTau T = test_tau(in.T);
+  asm volatile("" ::"r"(u.r0), "r"(u.rows), "r"(u.j0), "r"(u.cols), "r"(bk), "l"(nA), "l"(nB),
+               "f"(T.lo), "l"(Bf.part), "l"(Bf.cnt), "l"(Bf.surv_mask), "l"(Bf.need_bits));
+  pdl_wait();   // the above needs only the arguments and the instance table
+  pdl_trigger();
   if (!prepped) {   // the accumulators of the fill kernel
     const int64_t gs = (int64_t)gridDim.x * kCountThreads;
     if (in.quant)
