@@ -459,7 +459,9 @@ spamm_status_t spamm_tau_for_valid_ratio(spamm_plan_t plan, const double* normA,
  * spamm_mlp_train: `steps` Adam steps (numbers t0 + 1 ...); step s uses the
  *   samples idx[s * batch .. (s + 1) * batch) (device int32) of X / y_true;
  *   loss_hist (device [steps], may be NULL) receives each step's loss.  One
- *   CTA runs the whole loop with the weights on chip.
+ *   cluster of 16 CTAs (8 where 16 cannot be placed) runs the whole loop with
+ *   the weights on chip.  If one of its bounded waits runs out, all weights and
+ *   losses become NaN, m and v are left as they were, and spamm_last_device_status reports SPAMM_ERR_TIMEOUT.
  * All are asynchronous unless stated.
  * ------------------------------------------------------------------------- */
 spamm_status_t spamm_norm_histogram(spamm_plan_t plan, const double* normA, const double* normB,
@@ -540,20 +542,23 @@ spamm_status_t spamm_peak_rates(double* tflops, void* stream);
  * Status helpers.
  * spamm_status_string: static description of a status code.
  * spamm_last_device_status: reads and clears the library's device status word
- *   for the current device, and the static one of spamm_multiply_fp32_noalloc
- *   once that entry point has run in the current context (0 = clean, else a
- *   spamm_status_t; the library's word first when both are set).  Blocks.
+ *   for the current device, the static one of spamm_multiply_fp32_noalloc
+ *   once that entry point has run in the current context, and that of
+ *   spamm_mlp_train once it has run on the device (0 = clean, else a
+ *   spamm_status_t; the first one set, in this order).  Blocks.
  * ------------------------------------------------------------------------- */
 const char* spamm_status_string(spamm_status_t status);
 spamm_status_t spamm_last_device_status(void* stream, int32_t* code);
 
 /* spamm_selftest_bounded_wait: runs the bounded wait routines of the
  *   tensor-core multiply (one thread) and of the norm map (a whole warp) on an
- *   mbarrier phase that nothing completes, with the given limit (1 us .. 1 s).
+ *   mbarrier phase that nothing completes, and training steps whose exchange
+ *   between the CTAs is withheld, with the given limit (1 us .. 1 s).
  *   Each wait gives up, raises its abort flag and latches SPAMM_ERR_TIMEOUT in
- *   the device status word (read it with spamm_last_device_status); returns
- *   SPAMM_OK when all of that happened for both, *elapsed_ns (may be NULL) =
- *   the shorter of the two waits.  Blocks.  No part of the GPU is left waiting. */
+ *   the device status word (read it with spamm_last_device_status; the training
+ *   loop's word is checked and cleared here, and its results must all be NaN);
+ *   returns SPAMM_OK when all of that happened, *elapsed_ns (may be NULL) =
+ *   the shortest of the waits.  Blocks.  No part of the GPU is left waiting. */
 spamm_status_t spamm_selftest_bounded_wait(int64_t limit_ns, int64_t* elapsed_ns, void* stream);
 
 #ifdef __cplusplus

@@ -924,25 +924,38 @@ spamm_status_t spamm_selftest_bounded_wait(int64_t limit_ns, int64_t* elapsed_ns
   int32_t* status = device_status_word();
   if (!status) return SPAMM_ERR_NO_MEMORY;
   const cudaStream_t s = (cudaStream_t)stream;
+  const int results = mlp_wait_selftest_results();
+  const size_t bytes = 8 * sizeof(long long) + mlp_wait_selftest_floats() * sizeof(float);
   long long* out = nullptr;
-  if (cudaMalloc(&out, 6 * sizeof(long long)) != cudaSuccess) {
+  if (cudaMalloc(&out, bytes) != cudaSuccess) {
     (void)cudaGetLastError();
     return SPAMM_ERR_NO_MEMORY;
   }
-  long long h[6] = {0, 0, 0, 0, 0, 0};
-  // the multiply's wait (one thread) and the norm map's warp-wide wait
+  float* net = reinterpret_cast<float*>(out + 8);
+  long long h[7] = {0, 0, 0, 0, 0, 0, 0};
+  int32_t latched = 0;
+  std::vector<float> w(results, 0.0f);
+  // the multiply's wait (one thread), the norm map's warp-wide wait, the training loop's
   cudaError_t err = launch_wait_selftest(status, (uint64_t)limit_ns, out, s);
   if (err == cudaSuccess) err = launch_normmap_wait_selftest(status, (uint64_t)limit_ns, out + 3, s);
+  if (err == cudaSuccess) err = launch_mlp_wait_selftest(net, (uint64_t)limit_ns, out + 6, s);
   if (err == cudaSuccess) err = cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, s);
+  if (err == cudaSuccess)
+    err = cudaMemcpyAsync(w.data(), net, results * sizeof(float), cudaMemcpyDeviceToHost, s);
+  if (err == cudaSuccess) err = mlp_take_status(s, &latched);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   cudaFree(out);
   if (err != cudaSuccess) {
     (void)cudaGetLastError();
     return SPAMM_ERR_CUDA;
   }
-  if (elapsed_ns) *elapsed_ns = h[2] < h[5] ? h[2] : h[5];
-  // both waits must have given up and raised their abort flags
-  return (h[0] == 1 && h[1] == 1 && h[3] == 1 && h[4] == 1) ? SPAMM_OK : SPAMM_ERR_DEVICE_FAULT;
+  if (elapsed_ns) *elapsed_ns = std::min(h[2], std::min(h[5], h[6]));
+  bool all_nan = true;
+  for (float x : w) all_nan = all_nan && x != x;
+  // every wait must have given up, with its abort flag raised or its status latched
+  return (h[0] == 1 && h[1] == 1 && h[3] == 1 && h[4] == 1 && latched == SPAMM_ERR_TIMEOUT && all_nan)
+             ? SPAMM_OK
+             : SPAMM_ERR_DEVICE_FAULT;
 }
 
 spamm_status_t spamm_last_device_status(void* stream, int32_t* code) {
@@ -950,12 +963,14 @@ spamm_status_t spamm_last_device_status(void* stream, int32_t* code) {
   int32_t* w = device_status_word();
   if (!w) return SPAMM_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
-  int32_t other = 0;
+  int32_t other = 0, train = 0;
   SPAMM_CUDA_TRY(cudaMemcpyAsync(code, w, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   SPAMM_CUDA_TRY(cudaMemsetAsync(w, 0, sizeof(int32_t), s));
   SPAMM_CUDA_TRY(noalloc_take_status(s, &other));   // the no-allocation entry point's word
+  SPAMM_CUDA_TRY(mlp_take_status(s, &train));       // the training loop's word
   SPAMM_CUDA_TRY(cudaStreamSynchronize(s));
   if (*code == 0) *code = other;
+  if (*code == 0) *code = train;
   return SPAMM_OK;
 }
 

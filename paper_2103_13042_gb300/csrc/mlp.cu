@@ -19,7 +19,9 @@
 // memory, completion counted on its mbarrier), sums the sixteen parts of its own
 // share in a fixed order, updates those weights (Adam, the moments in registers)
 // and sends them to every CTA.  A 256-sample step is 13 MFLOP: on one SM that
-// alone is 25 us.  Waits are bounded as in the multiply.
+// alone is 25 us.  Waits are bounded as in the multiply: one that runs out ends the
+// training of every CTA, leaves NaN in all weights and latches SPAMM_ERR_TIMEOUT.
+#include <atomic>
 #include <cmath>
 
 #include <cooperative_groups.h>
@@ -124,8 +126,12 @@ struct Net {
   float y[2][kChunk], g3[kChunk], loss[kThreads / 32], gb3[kThreads / 32], half[4 * kH];
   Params recv;                // this CTA's share of every CTA's partial gradient, by rank
   uint64_t bar[2];            // all shares / all weights have arrived
-  int abort_flag, gave_up;    // a wait ran out
+  int abort_flag;             // a wait of some CTA of the cluster ran out
 };
+
+// Status word of the training loop: static, so that a call needs no allocation (it may be
+// captured); spamm_last_device_status reads and clears it with the library's own.
+static __device__ int32_t g_train_status;
 
 // Place of parameter p (the flat order of the weights) in Params, in floats.
 __device__ __forceinline__ int place(int p) {
@@ -398,20 +404,25 @@ __device__ __forceinline__ void load_weights(Net& n, const float* __restrict__ W
 }
 
 // One cluster: `steps` Adam steps; step s uses the samples idx[s * batch .. (s + 1) *
-// batch).  A wait that runs out leaves NaN weights (nothing is allocated for a status:
-// the call may be captured).
+// batch).  A thread whose wait runs out latches SPAMM_ERR_TIMEOUT in g_train_status and
+// raises the abort flag of its CTA and of the others; from then on it neither sends nor
+// arrives, and its waits return after a few polls, so that the remaining steps end quickly
+// (leaving the loop in its middle, or reading the flag before every send, costs 8 to 12 us
+// in 64 steps).  With the flag up, all weights and losses end as NaN, and m and v keep what they held.  WITHHOLD (self-test):
+// nothing is sent, so the first wait runs out after limit_ns; elapsed receives the longest
+// time a thread of the cluster waited.
 // 64 steps of 256 samples: 515 us, 8 us a step.  Of a step's 15.7 thousand cycles each
 // layer takes 1.6 to 2.0 (shared memory and latency), the outer products 2.3 (shared
 // memory), Adam 1.2, the two exchanges 5 (35 KB each way per CTA at the ~20 bytes per
 // clock of the cluster's network).  Before: one CTA, W2 read with 32-way bank conflicts,
 // 15.1 ms; the cluster with a thread per unit and four samples, and the exchange by
 // remote loads and stores, 746 us.
-template <int CL>
+template <int CL, bool WITHHOLD>
 __global__ void __launch_bounds__(kThreads, 1)
     train_kernel(float* __restrict__ Wg, float* __restrict__ mg, float* __restrict__ vg, int t0,
                  const float* __restrict__ X, const float* __restrict__ Y,
                  const int* __restrict__ idx, int steps, int batch, float lr, float q,
-                 float* __restrict__ loss_hist) {
+                 float* __restrict__ loss_hist, uint64_t limit_ns, long long* elapsed) {
   extern __shared__ __align__(16) unsigned char smem[];
   Net& n = *reinterpret_cast<Net*>(smem);
   auto cl = cooperative_groups::this_cluster();
@@ -420,11 +431,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr uint32_t kBytes = kSlice * 16;
   const int g = rank * kSlice + t;           // this thread's group
   const bool mine = t < kSlice;
-  const int to = (t & 31) ? CL : t >> 5;     // a copy per warp: their issue is serial within one
+  // a copy per warp: their issue is serial within one (CL: none)
+  int to = (t & 31) ? CL : t >> 5;
   if (t == 0) {
     tc::mbar_init(&n.bar[0], 1);
     tc::mbar_init(&n.bar[1], 1);
-    n.abort_flag = n.gave_up = 0;
+    n.abort_flag = 0;
     tc::fence_mbarrier_init();
   }
   load_weights(n, Wg);
@@ -446,6 +458,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   fetch(n, 0, X, Y, sample_row(idx, rank * kChunk, batch));
   cl.sync();   // every CTA's barriers are initialised
   uint32_t phase = 0;
+  auto wait = [&](uint64_t* bar) {
+    if (wait_ab(bar, phase, &n.abort_flag, &g_train_status, WITHHOLD ? limit_ns : kWaitLimitNs)) return;
+    if (to < CL) *cl.map_shared_rank(&n.abort_flag, to) = 1;
+    to = CL;
+  };
   for (int s = 0; s < steps; ++s, phase ^= 1u) {
     const int* now = idx + (int64_t)s * batch;
     const int row = s + 1 < steps ? sample_row(now + batch, rank * kChunk, batch) : -1;
@@ -454,14 +471,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     // send every CTA its share; a share's place in the receiver is free: it sent the
     // weights this step started from after it had summed the previous shares
-    if (t == 0) tc::mbar_arrive_expect_tx(&n.bar[0], CL * kBytes);
-    if (to < CL)
+    if (t == 0 && to < CL) tc::mbar_arrive_expect_tx(&n.bar[0], CL * kBytes);
+    if (!WITHHOLD && to < CL)
       tc::bulk_s2peer(tc::peer_addr(reinterpret_cast<float4*>(&n.recv) + rank * kSlice, to),
                       reinterpret_cast<float4*>(&n.part) + to * kSlice, kBytes,
                       tc::peer_addr(&n.bar[0], to));
     const int step = t0 + s + 1;
     const float c1 = 1.0f - powf(0.9f, (float)step), c2 = 1.0f - powf(0.999f, (float)step);
-    (void)wait_ab(&n.bar[0], phase, &n.abort_flag, &n.gave_up);
+    const uint64_t since = WITHHOLD ? tc::globaltimer_ns() : 0;
+    wait(&n.bar[0]);
+    if (WITHHOLD) atomicMax(elapsed, (long long)(tc::globaltimer_ns() - since));
     if (mine) {
       const float4* r4 = reinterpret_cast<const float4*>(&n.recv) + t;
       float4 d = r4[0];
@@ -488,14 +507,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     // send the new weights to the others (which have all finished this step's
     // gradient: their shares are here)
-    if (t == 0) tc::mbar_arrive_expect_tx(&n.bar[1], (CL - 1) * kBytes);
+    if (t == 0 && to < CL) tc::mbar_arrive_expect_tx(&n.bar[1], (CL - 1) * kBytes);
     if (to < CL && to != rank)
       tc::bulk_s2peer(tc::peer_addr(reinterpret_cast<float4*>(&n.w) + rank * kSlice, to),
                       reinterpret_cast<float4*>(&n.w) + rank * kSlice, kBytes,
                       tc::peer_addr(&n.bar[1], to));
-    (void)wait_ab(&n.bar[1], phase, &n.abort_flag, &n.gave_up);
+    wait(&n.bar[1]);
   }
   cl.sync();   // no CTA leaves while another sends to it
+  if (*const_cast<volatile int*>(&n.abort_flag)) {   // the same in every CTA
+    asm volatile("cp.async.wait_all;" ::: "memory");   // the next samples' copies
+    // copies sent before the barrier may still be on their way (35 KB in all, microseconds)
+    const uint64_t since = tc::globaltimer_ns(), drain = min(limit_ns, kDrainLimitNs);
+    while (tc::globaltimer_ns() - since < drain) __nanosleep(1000);
+    for (int p = t; p < kParams; p += kThreads)
+      if (place(p) / 4 / kSlice == rank) Wg[p] = NAN;
+    if (loss_hist && rank == 0)
+      for (int s = t; s < steps; s += kThreads) loss_hist[s] = NAN;
+    cl.sync();
+    return;
+  }
   // weights and moments back, each CTA its own groups
   for (int pass = 0; pass < 2; ++pass) {
     __syncthreads();
@@ -505,7 +536,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int at = place(p);
       if (at / 4 / kSlice != rank) continue;
       (pass ? vg : mg)[p] = reinterpret_cast<float*>(&n.part)[at];
-      if (!pass) Wg[p] = n.gave_up ? NAN : reinterpret_cast<float*>(&n.w)[at];
+      if (!pass) Wg[p] = reinterpret_cast<float*>(&n.w)[at];
     }
   }
 }
@@ -634,6 +665,10 @@ cudaError_t launch_cluster(void (*k16)(KArgs...), void (*k8)(KArgs...), cudaStre
 
 }  // namespace mlp
 
+namespace {
+std::atomic<bool> g_train_ran[64];   // per device: the status word may hold something
+}
+
 int mlp_param_count() { return mlp::kParams; }
 
 cudaError_t launch_mlp_forward(const float* W, const float* X, int count, float* Y,
@@ -661,8 +696,52 @@ cudaError_t launch_mlp_train(float* W, float* m, float* v, int t0, const float* 
                              const int* idx, int steps, int batch, float lr, float q,
                              float* loss_hist, cudaStream_t s) {
   if (steps <= 0) return cudaSuccess;
-  return mlp::launch_cluster(mlp::train_kernel<16>, mlp::train_kernel<8>, s, W, m, v, t0, X, Y, idx,
-                             steps, batch, lr, q, loss_hist);
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < 64) g_train_ran[dev].store(true, std::memory_order_relaxed);
+  return mlp::launch_cluster(mlp::train_kernel<16, false>, mlp::train_kernel<8, false>, s, W, m, v, t0,
+                             X, Y, idx, steps, batch, lr, q, loss_hist, kWaitLimitNs,
+                             (long long*)nullptr);
+}
+
+cudaError_t mlp_take_status(cudaStream_t s, int32_t* code) {
+  *code = 0;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || !g_train_ran[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+  void* w = nullptr;
+  e = cudaGetSymbolAddress(&w, mlp::g_train_status);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(code, w, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, sizeof(int32_t), s);
+  return e;
+}
+
+namespace {
+constexpr int kSelftestSteps = 64;
+}
+
+int mlp_wait_selftest_results() { return mlp::kParams + kSelftestSteps; }
+int mlp_wait_selftest_floats() {
+  return 3 * mlp::kParams + mlp::kIn + 1 + 2 * kSelftestSteps;
+}
+
+cudaError_t launch_mlp_wait_selftest(float* buf, uint64_t limit_ns, long long* elapsed,
+                                     cudaStream_t s) {
+  // steps of one sample each: W, losses, m, v, the sample's features and target, the steps'
+  // indexes (all zero)
+  cudaError_t e = cudaMemsetAsync(buf, 0, mlp_wait_selftest_floats() * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(elapsed, 0, sizeof(long long), s);
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < 64) g_train_ran[dev].store(true, std::memory_order_relaxed);
+  float *W = buf, *loss = W + mlp::kParams, *m = loss + kSelftestSteps, *v = m + mlp::kParams;
+  float *X = v + mlp::kParams, *Y = X + mlp::kIn;
+  return mlp::launch_cluster(mlp::train_kernel<16, true>, mlp::train_kernel<8, true>, s, W, m, v, 0, X, Y,
+                             reinterpret_cast<const int*>(Y + 1), kSelftestSteps, 1, 1e-3f, 0.5f,
+                             loss, limit_ns, elapsed);
 }
 
 cudaError_t launch_tau_from_hist(const InstRef& ref, const float* W, float* feats, double* tau,

@@ -307,6 +307,15 @@ cudaError_t launch_mlp_adam(float* W, const float* grad, float* m, float* v, int
 cudaError_t launch_mlp_train(float* W, float* m, float* v, int t0, const float* X, const float* Y,
                              const int* idx, int steps, int batch, float lr, float q,
                              float* loss_hist, cudaStream_t s);
+// The status word of the training loop's bounded waits, read into *code and cleared
+// (nothing is touched before the first training call on the device).
+cudaError_t mlp_take_status(cudaStream_t s, int32_t* code);
+// Self-test of those waits: training steps whose exchange is withheld; weights and losses,
+// the first mlp_wait_selftest_results() floats of buf, end as NaN.
+int mlp_wait_selftest_results();
+int mlp_wait_selftest_floats();
+cudaError_t launch_mlp_wait_selftest(float* buf, uint64_t limit_ns, long long* elapsed,
+                                     cudaStream_t s);
 // tau[i] (and the 65 features, when feats is non-null) of every instance
 // from pd[i].hist, pd[i].norm_a/b and Inst::target_rel.
 cudaError_t launch_tau_from_hist(const InstRef& ref, const float* W, float* feats, double* tau,
