@@ -2,7 +2,8 @@
 // kernel; the baseline the tensor-core modes are measured against).
 //
 // One persistent CTA per SM holds several independent groups of warps; a group
-// multiplies one tile at a time: 1 warp at leaf 32, 2 at 64, 8 at 128.  The
+// multiplies one tile at a time: 1 warp at leaf 32, 2 at 64, 8 at 128, and 4 at leaf 32
+// and 64 where there are few tiles (kWideTiles).  The
 // non-empty tiles of all instances (most survivors first) are dealt over the SMs
 // with a fixed stride; inside an SM its groups take them from a shared-memory
 // counter, so a group that met short tiles takes more of them (a fixed deal to
@@ -33,21 +34,41 @@ namespace {
 // kernel on a side stream costs more than their stores)
 constexpr int64_t kOwnZeroBytes = (int64_t)64 << 20;
 
-template <int LEAF>
+// Up to this many non-empty tiles per SM, four warps share a tile, in three groups with a
+// longer ring: with one or two warps per tile the other schedulers of an SM would idle
+// through its list.  One tile per SM, lists of 256 blocks at leaf 32: 325 -> 221 us (256
+// threads per tile, one group: 298), of 128 at leaf 64: 451 -> 310 (417); 32 tiles of 1024
+// blocks at leaf 32: 954 -> 532 (848), 8 of 256 at leaf 64: 895 -> 614 (822).  Two per SM
+// 254 -> 200 and 499 -> 470; three 263 -> 287 at leaf 32, and at leaf 64 757 -> 629 with
+// equal lists, but the selection of tau (uneven ones) 800 -> 812: hence the limit.  The
+// sums are in the same order in both forms.
+constexpr int kWideTiles = 2;
+
+// How a CTA is cut into groups of warps, a group's tile into warps and a warp's part
+// into threads: thread (ty, tx) of a warp has the rows ty + kTy u (u < TM) and the columns
+// 4 tx .. 4 tx + 3 and 4 kTx further on.
+template <int LEAF_, bool WIDE>
 struct SimtTile {
-  static constexpr int kWarps = LEAF == 128 ? 8 : (LEAF == 64 ? 2 : 1);
+  static_assert(!WIDE || LEAF_ < 128, "leaf 128: one form");
+  static constexpr int LEAF = LEAF_;
+  static constexpr int kWarps = WIDE ? 4 : (LEAF == 128 ? 8 : (LEAF == 64 ? 2 : 1));
   static constexpr int kThreads = 32 * kWarps;
-  // slices of the inner dimension, stages of the ring
-  static constexpr int kSlice = LEAF == 64 ? 16 : 32, kStages = LEAF == 64 ? 3 : 2;
-  static constexpr int kLdA = kSlice + 4;   // floats per staged row of A: 16-byte rows, four
-                                            // rows apart in different banks
-  static constexpr int TN = LEAF == 32 ? 4 : 8;                      // columns per thread
-  static constexpr int kWarpCols = 8 * TN;                           // 64, 32 at leaf 32
-  static constexpr int kStageFloats = LEAF * kLdA + kSlice * LEAF;   // A rows, then B rows
-  static constexpr size_t kSmem = (size_t)kStages * kStageFloats * sizeof(float);
   // groups per CTA, one CTA per SM: 168 registers per thread at leaf 32 and 64 (8 and 16
   // groups at 128 registers spill: 37 and 42 TFLOP/s against 48 and 45)
-  static constexpr int kGroups = LEAF == 128 ? 1 : (LEAF == 64 ? 6 : 12);
+  static constexpr int kGroups = WIDE ? 3 : (LEAF == 128 ? 1 : (LEAF == 64 ? 6 : 12));
+  // slices of the inner dimension, stages of the ring
+  static constexpr int kSlice = LEAF == 64 ? 16 : 32;
+  static constexpr int kStages = (LEAF == 64 ? 3 : 2) * (WIDE ? 12 / (kGroups * (LEAF == 64 ? 2 : 1)) : 1);
+  static constexpr int kLdA = kSlice + 4;   // floats per staged row of A: 16-byte rows, kTy
+                                            // rows in different banks
+  static constexpr bool kSmall = WIDE && LEAF == 32;   // 2 x 4 entries per thread
+  static constexpr int kTy = kSmall ? 8 : 4, kTx = 32 / kTy;
+  static constexpr int TM = kSmall ? 2 : 8;                          // rows per thread
+  static constexpr int TN = LEAF == 32 || WIDE ? 4 : 8;              // columns per thread
+  static constexpr int kWarpRows = kTy * TM, kWarpCols = kTx * TN;
+  static_assert(kWarps * kWarpRows * kWarpCols == LEAF * LEAF, "the warps cover the tile");
+  static constexpr int kStageFloats = LEAF * kLdA + kSlice * LEAF;   // A rows, then B rows
+  static constexpr size_t kSmem = (size_t)kStages * kStageFloats * sizeof(float);
   static constexpr int kCtaThreads = kGroups * kThreads;
   static constexpr size_t kCtaSmem = kGroups * kSmem;
   static_assert(kCtaSmem <= 227 * 1024 && kCtaThreads <= 1024 && kGroups <= 15, "CTA shape");
@@ -106,18 +127,18 @@ __device__ __forceinline__ void unpair(uint64_t d, float& x, float& y) {
 }
 
 // The barrier of one group (hardware barrier 1 + group).
-template <int LEAF>
+template <class T>
 __device__ __forceinline__ void tile_sync(int group) {
-  if constexpr (SimtTile<LEAF>::kWarps == 1)
+  if constexpr (T::kWarps == 1)
     __syncwarp();
   else
-    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(SimtTile<LEAF>::kThreads) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(T::kThreads) : "memory");
 }
 
 // An empty tile of an instance with beta = 0: zeros, and the tile's norm.
-template <int LEAF>
+template <class T>
 __device__ __forceinline__ void zero_tile(const Inst& in, int64_t t, int tid) {
-  constexpr int kThreads = SimtTile<LEAF>::kThreads;
+  constexpr int LEAF = T::LEAF, kThreads = T::kThreads;
   const int i = (int)(t / in.bn), j = (int)(t - (int64_t)i * in.bn);
   const int64_t r0 = (int64_t)i * LEAF, c0 = (int64_t)j * LEAF;
   const int rows = (int)min((int64_t)LEAF, in.m - r0), cols = (int)min((int64_t)LEAF, in.n - c0);
@@ -136,39 +157,37 @@ __device__ __forceinline__ void zero_tile(const Inst& in, int64_t t, int tid) {
   if (in.nC && tid == 0) in.nC[t] = 0.0;
 }
 
-// zeros: also write the tiles without survivors (every instance has beta = 0).
-template <int LEAF>
-__global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
-    simt_kernel(InstRef R, PlanBuffers Bf, int dynamic, int zeros) {
-  using T = SimtTile<LEAF>;
-  constexpr int TN = T::TN, kHalves = TN / 4;
-  constexpr int kSlice = T::kSlice, kStages = T::kStages, kLdA = T::kLdA;
+// The groups of one CTA multiply their tiles; zeros: they also write the tiles without
+// survivors (every instance has beta = 0).
+template <class T>
+__device__ __forceinline__ void multiply_tiles(const InstRef& R, const PlanBuffers& Bf, int64_t ne,
+                                               int dynamic, int zeros, int* s_taken, int* s_next,
+                                               SumSq* s_norm, const int thread) {
   extern __shared__ __align__(16) float smem_all[];
-  __shared__ int s_taken;               // tiles of this SM handed to its groups
-  __shared__ int s_next[T::kGroups];
-  __shared__ SumSq s_norm[T::kGroups][T::kWarps];
-  const int group = threadIdx.x / T::kThreads, tid = threadIdx.x % T::kThreads;
+  constexpr int LEAF = T::LEAF, TM = T::TM, TN = T::TN, kHalves = TN / 4;
+  constexpr int kSlice = T::kSlice, kStages = T::kStages, kLdA = T::kLdA, kTy = T::kTy, kTx = T::kTx;
+  const int group = thread / T::kThreads, tid = thread % T::kThreads;
   const int warp = tid >> 5, lane = tid & 31;
-  const int tx = lane & 7, ty = lane >> 3;
+  const int tx = lane % kTx, ty = lane / kTx;
   constexpr int kWarpsAcross = LEAF / T::kWarpCols;
-  const int wr = warp / kWarpsAcross * 32, wc = warp % kWarpsAcross * T::kWarpCols;
+  const int wr = warp / kWarpsAcross * T::kWarpRows, wc = warp % kWarpsAcross * T::kWarpCols;
   float* smem = smem_all + (size_t)group * kStages * T::kStageFloats;
-  if (threadIdx.x == 0) s_taken = 0;
-  __syncthreads();
-  pdl_wait();
-  const int64_t ne = Bf.bdev->nonempty, all = zeros ? Bf.tiles : ne;
+  const int all = (int)(zeros ? Bf.tiles : ne);
 
-  for (;;) {
-    if (tid == 0)   // dynamic: from the table's counter (it hands out non-empty tiles only)
-      s_next[group] = dynamic ? atomicAdd(&Bf.bdev->mul_ticket, 1) : atomicAdd(&s_taken, 1);
-    tile_sync<LEAF>(group);   // also: the previous tile's readers are done with the ring
+  for (bool first = true;; first = false) {
+    // dynamic: from the table's counter (it hands out non-empty tiles only); else a group's
+    // first tile is its own, so that few tiles fall on warps of different schedulers
+    if (tid == 0)
+      s_next[group] = dynamic ? atomicAdd(&Bf.bdev->mul_ticket, 1)
+                              : (first ? group : T::kGroups + atomicAdd(s_taken, 1));
+    tile_sync<T>(group);   // also: the previous tile's readers are done with the ring
     const int64_t w = dynamic ? s_next[group] : blockIdx.x + (int64_t)s_next[group] * gridDim.x;
     if (w >= (dynamic ? ne : all)) break;
     const int g = Bf.order[w];
     const Inst& in = R.at(inst_of(R, Bf, g));
     if (w >= ne) {
-      zero_tile<LEAF>(in, g - in.tile0, tid);
-      tile_sync<LEAF>(group);   // s_next is rewritten next
+      zero_tile<T>(in, g - in.tile0, tid);
+      tile_sync<T>(group);   // s_next is rewritten next
       continue;
     }
     const int beg = Bf.tile_beg[g], cnt = Bf.cnt[g];
@@ -184,9 +203,9 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
     const int i = (int)(t / bn), j = (int)(t % bn);
     const int64_t r0 = (int64_t)i * LEAF, c0 = (int64_t)j * LEAF;
 
-    uint64_t acc[8][TN / 2];
+    uint64_t acc[TM][TN / 2];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < TM; ++u)
 #pragma unroll
       for (int v = 0; v < TN / 2; ++v) acc[u][v] = 0ull;
 
@@ -243,27 +262,27 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
     for (int q = 0; q < kStages - 1; ++q) fetch(q);
     for (int q = 0; q < nslices; ++q) {
       asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
-      tile_sync<LEAF>(group);   // slice q is here; slice q - 1 has been read
+      tile_sync<T>(group);   // slice q is here; slice q - 1 has been read
       fetch(q + kStages - 1);
       const float* sa = smem + (q % kStages) * T::kStageFloats + (wr + ty) * kLdA;
       const float* sb = smem + (q % kStages) * T::kStageFloats + LEAF * kLdA + wc + tx * 4;
 #pragma unroll
       for (int s2 = 0; s2 < kSlice; s2 += 2) {
-        float2 a[8];
+        float2 a[TM];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] = *reinterpret_cast<const float2*>(sa + 4 * u * kLdA + s2);
+        for (int u = 0; u < TM; ++u) a[u] = *reinterpret_cast<const float2*>(sa + kTy * u * kLdA + s2);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           uint64_t b[TN / 2];
 #pragma unroll
           for (int h = 0; h < kHalves; ++h) {
             const ulonglong2 x =
-                *reinterpret_cast<const ulonglong2*>(sb + (s2 + e) * LEAF + 32 * h);
+                *reinterpret_cast<const ulonglong2*>(sb + (s2 + e) * LEAF + 4 * kTx * h);
             b[2 * h] = x.x;
             b[2 * h + 1] = x.y;
           }
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
+          for (int u = 0; u < TM; ++u) {
             const float f = e == 0 ? a[u].x : a[u].y;
             const uint64_t aa = pair(f, f);
 #pragma unroll
@@ -278,15 +297,15 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
     const float alpha = in.alpha, beta = in.beta;
     SumSq ss = sumsq_empty();
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int64_t r = r0 + wr + ty + 4 * u;
+    for (int u = 0; u < TM; ++u) {
+      const int64_t r = r0 + wr + ty + kTy * u;
       const bool row_in = r < m;
       float x[TN];
 #pragma unroll
       for (int v = 0; v < TN / 2; ++v) unpair(acc[u][v], x[2 * v], x[2 * v + 1]);
 #pragma unroll
       for (int h = 0; h < kHalves; ++h) {
-        const int64_t c = c0 + wc + 32 * h + tx * 4;
+        const int64_t c = c0 + wc + 4 * kTx * h + tx * 4;
         float* p = C + r * ldc + c;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -306,7 +325,7 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
       if (in.nC) {   // C's norm map for a chained product: the row's stored values
 #pragma unroll
         for (int q = 0; q < TN; ++q)
-          if (!(row_in && c0 + wc + 32 * (q / 4) + tx * 4 + q % 4 < n)) x[q] = 0.0f;
+          if (!(row_in && c0 + wc + 4 * kTx * (q / 4) + tx * 4 + q % 4 < n)) x[q] = 0.0f;
         sumsq_group<TN>(ss, x);
       }
     }
@@ -318,12 +337,12 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
         const int e = __shfl_xor_sync(0xffffffffu, ss.e, off);
         sumsq_merge_any(ss, h, l, e);
       }
-      if (lane == 0) s_norm[group][warp] = ss;
-      tile_sync<LEAF>(group);
+      if (lane == 0) s_norm[group * T::kWarps + warp] = ss;
+      tile_sync<T>(group);
       if (tid == 0) {
-        SumSq tot = s_norm[group][0];
+        SumSq tot = s_norm[group * T::kWarps];
         for (int w2 = 1; w2 < T::kWarps; ++w2) {
-          const SumSq o = s_norm[group][w2];
+          const SumSq o = s_norm[group * T::kWarps + w2];
           sumsq_merge_any(tot, o.hi, o.lo, o.e);
         }
         in.nC[t] = sumsq_sqrt(tot);
@@ -335,14 +354,51 @@ __global__ void __launch_bounds__(SimtTile<LEAF>::kCtaThreads, 1)
   for (int64_t w = ne + blockIdx.x * T::kGroups + group; w < all; w += (int64_t)gridDim.x * T::kGroups) {
     const int g = Bf.order[w];
     const Inst& in = R.at(inst_of(R, Bf, g));
-    zero_tile<LEAF>(in, g - in.tile0, tid);
+    zero_tile<T>(in, g - in.tile0, tid);
   }
+}
+
+// Few tiles.  A function of its own: with both forms in the kernel's body the other one
+// fetches its first instructions from further on, 1 to 3 us.
+template <int LEAF>
+__device__ __noinline__ void multiply_wide(const InstRef& R, const PlanBuffers& Bf, int dynamic,
+                                           int zeros) {
+  using T = SimtTile<LEAF, true>;
+  static_assert(T::kCtaThreads == SimtTile<LEAF, false>::kCtaThreads &&
+                    T::kCtaSmem == SimtTile<LEAF, false>::kCtaSmem,
+                "one launch serves both forms");
+  __shared__ int s_taken, s_next[T::kGroups];
+  __shared__ SumSq s_norm[T::kGroups * T::kWarps];
+  if (threadIdx.x == 0) s_taken = 0;
+  __syncthreads();
+  multiply_tiles<T>(R, Bf, Bf.bdev->nonempty, dynamic, zeros, &s_taken, s_next, s_norm, threadIdx.x);
+}
+
+template <int LEAF>
+__global__ void __launch_bounds__(SimtTile<LEAF, false>::kCtaThreads, 1)
+    simt_kernel(InstRef R, PlanBuffers Bf, int dynamic, int zeros) {
+  using T = SimtTile<LEAF, false>;
+  __shared__ int s_taken;               // tiles of this SM handed out after its groups' first
+  __shared__ int s_next[T::kGroups];
+  __shared__ SumSq s_norm[T::kGroups * T::kWarps];
+  const int thread = threadIdx.x;
+  if (thread == 0) s_taken = 0;
+  __syncthreads();
+  pdl_wait();
+  const int ne = Bf.bdev->nonempty;
+  if constexpr (LEAF < 128) {
+    if (ne <= kWideTiles * (int)gridDim.x) {
+      multiply_wide<LEAF>(R, Bf, dynamic, zeros);
+      return;
+    }
+  }
+  multiply_tiles<T>(R, Bf, ne, dynamic, zeros, &s_taken, s_next, s_norm, thread);
 }
 
 template <int LEAF>
 cudaError_t launch(const InstRef& ref, const PlanBuffers& b, int schedule, bool zeros,
                    cudaStream_t s) {
-  using T = SimtTile<LEAF>;
+  using T = SimtTile<LEAF, false>;
   static int sms[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
