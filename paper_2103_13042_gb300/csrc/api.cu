@@ -161,7 +161,10 @@ bool own_zeros(const Engine& e, const InstRef& ref) {
   return e.precision == SPAMM_FP32 && simt_writes_zeros(ref, e.buf, e.leaf);
 }
 
-// The multiply of the non-empty tiles (operand rounding first in tensor modes).
+// The multiply of the non-empty tiles (operand rounding first in tensor modes).  The order
+// of the launches matters: the tensor-core multiply's scheduler reads the plan and takes
+// tiles from mul_ticket before its own wait.  Plan and cleared counter must therefore be
+// complete before the wait of the kernel right before it in the stream, which is the rounding.
 cudaError_t multiply_nonempty(Engine& e, const InstRef& ref, int32_t* status, cudaStream_t s,
                               cudaEvent_t after_round) {
   cudaError_t err = cudaSuccess;

@@ -40,7 +40,8 @@ int32_t* device_status_word();
 // that grid writes and before it writes anything.  A kernel calls pdl_trigger(), which
 // lets the successor launch, only after its own wait, so completion stays transitive
 // along the chain: what was complete before the predecessor's wait (the arguments'
-// tables, for a multiply also the plan) may be read before the own one.
+// tables, for a tensor-core multiply also the plan and its cleared tile counter, which
+// it may then take from) may be used before the own one.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {

@@ -200,7 +200,10 @@ __global__ void __launch_bounds__(TcCfg<FMT, LEAF, SPLITMODE>::kThreads, 1)
   // the set-up above (barriers, tensor memory) overlaps the previous kernel's
   // tail; everything below reads what it wrote.  The previous kernel is the rounding,
   // placed once the plan was complete: the scheduler reads its first tiles' queues
-  // before it waits, which it does for the blocks' scales.
+  // before it waits, which it does for the blocks' scales.  In the dynamic order it also
+  // takes them from the counter, which was cleared before the rounding was launched (tiles
+  // dealt in advance, or a wait before the first one: 1 to 3 us more, as the SMs that are
+  // free first no longer start first).
   if (warp != 2) pdl_wait();
   const int ne = p.Bf.bdev->nonempty;
 
