@@ -386,12 +386,14 @@ __global__ void __launch_bounds__(kPrepThreads)
 // ||A||_F^2 (lane 0) and ||B||_F^2 (lane 1) from `count` partial sums at `first`, by one
 // warp in a fixed order (every caller gets the same bits): the even lanes add up
 // A's, the odd ones B's, so that one square root serves both (FP64 is scarce here).
-__device__ __forceinline__ double sum_norms2(const PlanBuffers& Bf, int first, int count) {
+// live = false: no load (instance_stats).
+__device__ __forceinline__ double sum_norms2(const PlanBuffers& Bf, int first, int count,
+                                             bool live = true) {
   const int lane = threadIdx.x & 31;
   const double* p = ((lane & 1) ? Bf.part_b : Bf.part_a) + first;
   double x = 0.0;
 #pragma unroll 4
-  for (int i = lane >> 1; i < count; i += 16) x += __ldcg(p + i);
+  for (int i = lane >> 1; i < count; i += 16) x += live ? __ldcg(p + i) : 0.0;
   for (int off = 16; off > 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
   return x;
 }
@@ -467,9 +469,11 @@ struct UnitSums {
 // One warp's part v of an instance's sums: its lane l takes the units 32 v + l,
 // 32 v + l + 32 kStatWarps, ... (four units' loads at a time).  The kStatWarps parts
 // are merged in order (merge_sums), whoever forms them, so that a single call and
-// a batch give the same bits.  WHAT: 1 the counts and b1, 2 b2, 3 all.
+// a batch give the same bits.  WHAT: 1 the counts and b1, 2 b2, 3 all.  live = false: no
+// load (instance_stats).
 template <int WHAT>
-__device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers& Bf, int v) {
+__device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers& Bf, int v,
+                                              bool live = true) {
   const int units = units_of(in);
   constexpr int nt = 32 * kStatWarps;
   UnitSums r{0, 0, 0, {0.0f, 0}, {0.0f, 0}};
@@ -482,7 +486,7 @@ __device__ __forceinline__ UnitSums unit_sums(const Inst& in, const PlanBuffers&
       const int64_t q = in.count0 + q0 + z * nt;
       s4[z] = 0;
       hi[z] = bb[z] = make_int4(0, 0, 0, 0);
-      if (q0 + z * nt < units) {
+      if (live && q0 + z * nt < units) {
         if (WHAT & 1) {
           s4[z] = __ldcg(Bf.part + q * kPartInts + kPartS);
           hi[z] = __ldcg(reinterpret_cast<const int4*>(Bf.part + q * kPartInts + kPartNe));
@@ -529,7 +533,7 @@ __device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts
   const bool prepped = norm2 == nullptr;
   PlanDevice* pd = in.pd;
   double x = 0.0;
-  if (lane < 2) x = prepped ? __ldcg(lane ? &pd->norm_b : &pd->norm_a) : norm2[lane];
+  if (lane < 2 && publish) x = prepped ? __ldcg(lane ? &pd->norm_b : &pd->norm_a) : norm2[lane];
   UnitSums u = parts[0];
   // (parts formed for the binade only hold no b1)
   const ExtSum none{0.0f, 0};
@@ -579,8 +583,8 @@ __device__ __forceinline__ int write_stats(const Inst& in, const UnitSums* parts
 // Part v of one instance's sums into shared memory, by one warp.
 template <int WHAT>
 __device__ __forceinline__ void stat_part(const Inst& in, const PlanBuffers& Bf, UnitSums* parts,
-                                          int v) {
-  const UnitSums u = unit_sums<WHAT>(in, Bf, v);
+                                          int v, bool live = true) {
+  const UnitSums u = unit_sums<WHAT>(in, Bf, v, live);
   if ((threadIdx.x & 31) != 0) return;
   if (WHAT & 1) {
     parts[v].S = u.S;
@@ -592,22 +596,23 @@ __device__ __forceinline__ void stat_part(const Inst& in, const PlanBuffers& Bf,
 }
 
 // The statistics of one instance by a CTA of kStatWarps warps, or twice as many: then
-// the second half forms b2.  The norms (not prepped) are added up beside.
+// the second half forms b2.  The norms (not prepped) are added up beside.  publish = false:
+// the same instructions without a load from the plan's buffers or a store to them.
 __device__ __noinline__ void instance_stats(const Inst& in, const PlanBuffers& Bf, bool prepped,
                                             bool publish) {
   __shared__ UnitSums s_u[kStatWarps];
   __shared__ double s_below[32 * kBinsPerLane], s_norm2[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (!prepped && warp == kStatWarps - 1) {
-    const double x = sum_norms2(Bf, in.count0, units_of(in));
+    const double x = sum_norms2(Bf, in.count0, units_of(in), publish);
     if (lane < 2) s_norm2[lane] = x;
   }
   if (blockDim.x < 2 * 32 * kStatWarps)
-    stat_part<3>(in, Bf, s_u, warp);
+    stat_part<3>(in, Bf, s_u, warp, publish);
   else if (warp < kStatWarps)
-    stat_part<1>(in, Bf, s_u, warp);
+    stat_part<1>(in, Bf, s_u, warp, publish);
   else if (warp < 2 * kStatWarps)
-    stat_part<2>(in, Bf, s_u, warp - kStatWarps);
+    stat_part<2>(in, Bf, s_u, warp - kStatWarps, publish);
   if (warp == 0 && in.split) flag_prefix(in, s_below);
   __syncthreads();
   if (warp == 0) (void)write_stats(in, s_u, kStatWarps, prepped ? nullptr : s_norm2, true, publish, s_below);
@@ -1322,7 +1327,7 @@ __global__ void __launch_bounds__(kFillThreads)
                "l"(Bf.tile_beg), "l"(Bf.k_idx), "l"(Bf.need_bits), "l"(Bf.need_list), "l"(Bf.bdev));
   if (u0 >= U) {   // no split modes: one more CTA per instance forms its statistics
     // twice: the first pass, while the count kernel still runs, only fetches the
-    // instructions (its sums are of whatever is there, and are not published)
+    // instructions (it loads nothing that kernel writes)
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
       if (pass == 1) {
