@@ -158,7 +158,7 @@ namespace {
 
 // The multiply writes the empty tiles too: no zero-fill on the side stream.
 bool own_zeros(const Engine& e, const InstRef& ref) {
-  return e.precision == SPAMM_FP32 && simt_writes_zeros(ref, e.buf, e.leaf);
+  return e.precision == SPAMM_FP32 && simt_writes_zeros(ref, e.buf, e.leaf, true);
 }
 
 // The multiply of the non-empty tiles (operand rounding first in tensor modes).  The order

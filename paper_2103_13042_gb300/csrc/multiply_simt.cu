@@ -30,9 +30,18 @@
 namespace spamm {
 namespace {
 
-// Outputs up to this size: the multiply writes the empty tiles itself (a second
-// kernel on a side stream costs more than their stores)
-constexpr int64_t kOwnZeroBytes = (int64_t)64 << 20;
+// Outputs up to this size: the multiply writes the empty tiles itself.  A second kernel
+// beside it (on a side stream) costs two events and a launch, but its stores overlap the
+// multiply's latency.  Product on exponential decay (nearly all tiles empty), second
+// kernel -> own stores: at 4 MB 21.0 -> 19.4, 27.1 -> 23.9 and 53.8 -> 50.7 us at leaf 32, 64
+// and 128; at 31 MB 33.0 -> 30.0, 33.2 -> 28.6, 55.8 -> 57.7; at 64 MB 45.7 -> 45.2, 41.3 ->
+// 34.8, 57.8 -> 64.6; at 127 MB 63.3 -> 87.6, 58.5 -> 56.9, 77.7 -> 95.9 (16 MB, leaf 128:
+// 53.8 -> 52.1).  Leaf 128 has the fewest warps to store with.  Against a second kernel
+// behind the multiply, in the same stream, own stores win at leaf 128 too (product without
+// allocation, 64 MB: 123 -> 117 us).
+constexpr int64_t own_zero_bytes(int leaf, bool beside) {
+  return (int64_t)(leaf == 128 && beside ? 24 : 64) << 20;
+}
 
 // Up to this many non-empty tiles per SM, four warps share a tile, in three groups with a
 // longer ring: with one or two warps per tile the other schedulers of an SM would idle
@@ -419,8 +428,8 @@ cudaError_t launch(const InstRef& ref, const PlanBuffers& b, int schedule, bool 
 
 }  // namespace
 
-bool simt_writes_zeros(const InstRef& ref, const PlanBuffers& b, int leaf) {
-  return !ref.any_scaled && b.tiles * leaf * leaf * (int64_t)sizeof(float) <= kOwnZeroBytes;
+bool simt_writes_zeros(const InstRef& ref, const PlanBuffers& b, int leaf, bool beside) {
+  return !ref.any_scaled && b.tiles * leaf * leaf * (int64_t)sizeof(float) <= own_zero_bytes(leaf, beside);
 }
 
 cudaError_t launch_multiply_simt(const InstRef& ref, const PlanBuffers& b, int leaf,

@@ -188,7 +188,7 @@ extern "C" spamm_status_t spamm_multiply_fp32_noalloc(const float* A, const floa
   cudaError_t e = launch_normmap(A, n, leaf, nA, addr.status, s);
   if (e == cudaSuccess) e = launch_normmap(B, n, leaf, nB, addr.status, s);
   if (e == cudaSuccess) e = run_plan(ref, buf, s);
-  const bool own = simt_writes_zeros(ref, buf, leaf);
+  const bool own = simt_writes_zeros(ref, buf, leaf, false);
   if (e == cudaSuccess) e = launch_multiply_simt(ref, buf, leaf, kScheduleStatic, own, s);
   if (e == cudaSuccess && !own) e = launch_zero_empty_tiles(ref, buf, leaf, s);
   if (e != cudaSuccess) {

@@ -285,8 +285,8 @@ cudaError_t launch_normmap_jobs(const NormJob* dev_jobs, int n_vec, int units_ve
 cudaError_t launch_multiply_simt(const InstRef& ref, const PlanBuffers& b, int leaf,
                                  int schedule, bool zeros, cudaStream_t s);
 // Every instance has beta = 0 and the outputs are small: no kernel of their own
-// for the empty tiles.
-bool simt_writes_zeros(const InstRef& ref, const PlanBuffers& b, int leaf);
+// for the empty tiles (which would run beside the multiply, or after it).
+bool simt_writes_zeros(const InstRef& ref, const PlanBuffers& b, int leaf, bool beside);
 
 // Per-tile partial sums of squares of the tensor-core epilogue (output norm
 // maps): one per epilogue warp of a tile, merged by launch_norm_out_finish.
