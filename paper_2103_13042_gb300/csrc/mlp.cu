@@ -88,7 +88,7 @@ __device__ __forceinline__ void adam_update(float& w, float g, float& m, float& 
   const bool m0 = m == 0.0f, v0 = v == 0.0f;
   const float mhat = (m0 ? 1.0f : m) / c1, root = sqrtf((v0 ? 1.0f : v) / c2);
   const float step = lr * mhat / ((v0 ? 0.0f : root) + 1e-8f);
-  w -= m0 ? 0.0f : step;
+  w -= m0 ? 0.0f * lr : step;   // (an infinite rate gives NaN, as in the formula)
 }
 
 __global__ void adam_kernel(float* __restrict__ W, const float* __restrict__ grad,
