@@ -681,7 +681,7 @@ __device__ __forceinline__ void stage_unit(const Inst& in, const Unit& u, Screen
 // One CTA per unit.  A lane owns a tile, so nothing is reduced across lanes per
 // tile and a word of the survivor mask is built in a register; about 25
 // instructions per triple and lane, bound by issue and by the latency of staging
-// (eight loads in flight per thread).  The previous form (a warp per tile, lanes
+// (twelve loads in flight per thread).  The previous form (a warp per tile, lanes
 // over k: ballots and some 150 instructions of reductions per tile) took 69 us at
 // bk = 256 (1.7e7 triples), this one 40; for 256 uneven split instances 148 -> 55.
 template <bool SPLIT, bool BAND>
@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(kCountThreads)
 // a tile's bound at a point is the sum of the gaps below it), and its last CTA
 // takes the four decisions and lays out the next points.  No host round trip in
 // between: 36 counting half-plans with a synchronisation each took 1.0 ms at 64
-// blocks per side, this takes 0.2.
+// blocks per side, this takes 0.11 (nine passes of about 12 us each).
 // ---------------------------------------------------------------------------
 
 // Grid point x as a threshold.
@@ -1026,7 +1026,7 @@ __global__ void __launch_bounds__(kCountThreads) cert_pass_kernel(InstRef R, Pla
   __syncthreads();
   // the tiles' sums up to every point (a lane per tile), then the points' sums of
   // squares, eight threads each, in the order of a warp's butterfly (both by one warp,
-  // a point after the other, took 11 of a pass's 24 us)
+  // a point after the other, took 11 of the 24 us that a pass then lasted)
   if (warp == 0) {
     int emax = kSkipNone;
 #pragma unroll
