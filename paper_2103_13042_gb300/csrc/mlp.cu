@@ -142,13 +142,6 @@ __device__ __forceinline__ int place(int p) {
   return kB1 + kH + p - kOffB2;   // b2, w3, b3 follow each other
 }
 
-__device__ __forceinline__ void copy4(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-
 // Row of this warp's sample of the chunk at c0: -1 past `count`.
 __device__ __forceinline__ int sample_row(const int* __restrict__ idx, int c0, int count) {
   const int s = c0 + (int)(threadIdx.x >> 5);
@@ -163,10 +156,10 @@ __device__ __forceinline__ void fetch(Net& n, int buf, const float* __restrict__
   float* dst = n.x[buf] + s * kLd;
   if (row >= 0) {
     const float* src = Xg + (int64_t)row * kIn;
-    copy4(dst + lane, src + lane);
-    copy4(dst + lane + 32, src + lane + 32);
-    if (lane == 0) copy4(dst + 64, src + 64);
-    if (lane == 1) copy4(&n.y[buf][s], Yg + row);
+    tc::copy4(dst + lane, src + lane);
+    tc::copy4(dst + lane + 32, src + lane + 32);
+    if (lane == 0) tc::copy4(dst + 64, src + 64);
+    if (lane == 1) tc::copy4(&n.y[buf][s], Yg + row);
   } else {
     dst[lane] = 0.0f;
     dst[lane + 32] = 0.0f;

@@ -83,18 +83,6 @@ struct SimtTile {
   static_assert(kCtaSmem <= 227 * 1024 && kCtaThreads <= 1024 && kGroups <= 15, "CTA shape");
 };
 
-// Copies 16 (4) bytes, `bytes` of them from src and the rest zeros.
-__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
-               "r"(bytes)
-               : "memory");
-}
-
 // Stages rows [r, r + ROWS) x columns [c, c + COLS) of a rows x cols matrix with
 // leading dimension ld as ROWS rows of LD floats.
 template <int ROWS, int COLS, int LD, int THREADS>
@@ -108,14 +96,14 @@ __device__ __forceinline__ void stage(float* dst, const float* __restrict__ M, i
       const int p = tid + l * THREADS, pr = p / kPerRow, pc = p % kPerRow * 4;
       const int64_t left = r + pr < rows ? cols - (c + pc) : 0;
       const int bytes = left >= 4 ? 16 : (left > 0 ? (int)left * 4 : 0);
-      copy16(dst + pr * LD + pc, bytes ? M + (r + pr) * ld + c + pc : M, bytes);
+      tc::copy16(dst + pr * LD + pc, bytes ? M + (r + pr) * ld + c + pc : M, bytes);
     }
   } else {
 #pragma unroll 4
     for (int l = 0; l < ROWS * COLS / THREADS; ++l) {
       const int p = tid + l * THREADS, pr = p / COLS, pc = p % COLS;
       const bool in = r + pr < rows && c + pc < cols;
-      copy4(dst + pr * LD + pc, in ? M + (r + pr) * ld + c + pc : M, in ? 4 : 0);
+      tc::copy4(dst + pr * LD + pc, in ? M + (r + pr) * ld + c + pc : M, in ? 4 : 0);
     }
   }
 }
@@ -240,24 +228,24 @@ __device__ __forceinline__ void multiply_tiles(const InstRef& R, const PlanBuffe
             constexpr int kStep = kThr / kPc;
 #pragma unroll
             for (int l = 0; l < LEAF / kStep; ++l, src += kStep * lda)
-              copy16(s + (pa + l * kStep) * kLdA + ca, src, 16);
+              tc::copy16(s + (pa + l * kStep) * kLdA + ca, src, 16);
           } else {
             constexpr int kStep = kThr / kSlice;
 #pragma unroll 8
             for (int l = 0; l < LEAF / kStep; ++l, src += kStep * lda)
-              copy4(s + (pa + l * kStep) * kLdA + ca, src, 4);
+              tc::copy4(s + (pa + l * kStep) * kLdA + ca, src, 4);
           }
           src = base_b + k0 * ldb;
           if (vec_b) {
             constexpr int kStep = kThr / kPl;
 #pragma unroll
             for (int l = 0; l < kSlice / kStep; ++l, src += kStep * ldb)
-              copy16(sb + (pb + l * kStep) * LEAF + cb, src, 16);
+              tc::copy16(sb + (pb + l * kStep) * LEAF + cb, src, 16);
           } else {
             constexpr int kStep = kThr / LEAF;
 #pragma unroll 8
             for (int l = 0; l < kSlice / kStep; ++l, src += kStep * ldb)
-              copy4(sb + (pb + l * kStep) * LEAF + cb, src, 4);
+              tc::copy4(sb + (pb + l * kStep) * LEAF + cb, src, 4);
           }
         } else {
           stage<LEAF, kSlice, kLdA, kThr>(s, A, m, kd, lda, r0, k0, vec_a);

@@ -1,14 +1,15 @@
-// Operand rounding for the tensor-core multiply (spec mixed precision on
-// top of the paper's FP16 tensor-core kernel, Section 3.3 / Algorithm 3).
+// Operand rounding for the tensor-core multiply (mixed precision on top of the
+// paper's FP16 tensor-core kernel, Section 3.3 / Algorithm 3).
 //
 // For every leaf block that some surviving triple uses (the plan's list of
 // needed blocks) a CTA finds e = frexp exponent of its largest magnitude,
 // scales by 2^-e (exact), rounds to nearest-even in the operand format (hi)
-// and, in split modes, rounds the exact residual scaled by 2^s_lo (lo).  The result is written directly as the K-major, 128-byte
-// swizzled image the MMA reads: chunk c of a block holds K elements
-// [c*kc, (c+1)*kc) (kc = 128 bytes / element size) for every row, 128 bytes
-// per row, 16-byte pieces XOR-swizzled by (row mod 8).  A blocks keep their
-// rows; B blocks are transposed (image row n = column n of the block).
+// and, in split modes, rounds the exact residual scaled by 2^s_lo (lo).  The
+// result is written directly as the K-major, 128-byte swizzled image the MMA
+// reads: chunk c of a block holds K elements [c*kc, (c+1)*kc) (kc = 128 bytes /
+// element size) for every row, 128 bytes per row, 16-byte pieces XOR-swizzled by
+// (row mod 8).  A blocks keep their rows; B blocks are transposed (image row n =
+// column n of the block).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -17,7 +18,6 @@
 
 namespace spamm {
 namespace {
-
 
 // Round to nearest even, keeping 10 explicit significand bits (TF32), on the
 // IEEE bit pattern; NaN/Inf pass through unchanged.
@@ -28,23 +28,73 @@ __device__ __forceinline__ float round_tf32(float x) {
   return __uint_as_float(u & 0xffffe000u);
 }
 
+// A block's exponent from its largest magnitude.  BF16 and TF32 have FP32's exponent
+// range: the scaling only has to keep products and sums inside it, so e is rounded up to a
+// multiple of 32 (scaled maximum in [2^-33, 1)).  The roundings are those of the exact
+// exponent for every entry above 2^-94 of the block's maximum (hi parts) and above 2^-80
+// (lo parts of the split modes), and the blocks of a tile mostly share one exponent sum:
+// the multiply's runs (one accumulator pass per change of the sum) stay long.  FP16 keeps
+// the exact exponent: its range is the constraint.
 template <uint32_t FMT>
-__device__ __forceinline__ float round_op(float x) {
-  if constexpr (FMT == tc::kFmtBF16) return __bfloat162float(__float2bfloat16_rn(x));
-  else if constexpr (FMT == tc::kFmtF16) return __half2float(__float2half_rn(x));
-  else return round_tf32(x);
+__device__ __forceinline__ int block_exponent(float mx) {
+  int ex = 0;
+  if (mx > 0.0f && mx <= 3.402823466e38f) frexpf(mx, &ex);
+  return FMT == tc::kFmtF16 ? ex : ((ex + 31) >> 5) << 5;
 }
 
+// Two entries rounded to nearest even and packed (the first in the low half).
 template <uint32_t FMT>
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
+__device__ __forceinline__ uint32_t pack_pair(float a, float b) {
   if constexpr (FMT == tc::kFmtBF16) {
-    const uint32_t lo = __bfloat16_as_ushort(__float2bfloat16_rn(a));
-    const uint32_t hi = __bfloat16_as_ushort(__float2bfloat16_rn(b));
-    return lo | (hi << 16);
+    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+    return (uint32_t)__bfloat16_as_ushort(p.x) | ((uint32_t)__bfloat16_as_ushort(p.y) << 16);
   } else {
-    const uint32_t lo = __half_as_ushort(__float2half_rn(a));
-    const uint32_t hi = __half_as_ushort(__float2half_rn(b));
-    return lo | (hi << 16);
+    const __half2 p = __floats2half2_rn(a, b);
+    return (uint32_t)__half_as_ushort(__low2half(p)) | ((uint32_t)__half_as_ushort(__high2half(p)) << 16);
+  }
+}
+
+// The two values back (exact).
+template <uint32_t FMT>
+__device__ __forceinline__ void unpack_pair(uint32_t w, float& a, float& b) {
+  if constexpr (FMT == tc::kFmtBF16) {
+    a = __uint_as_float(w << 16);
+    b = __uint_as_float(w & 0xffff0000u);
+  } else {
+    a = __half2float(__ushort_as_half((unsigned short)(w & 0xffffu)));
+    b = __half2float(__ushort_as_half((unsigned short)(w >> 16)));
+  }
+}
+
+// One 16-byte piece of an image: v scaled by 2^-ex, rounded (hi), and in split modes
+// the exact residual scaled by 2^lo shift, rounded (lo).
+template <uint32_t FMT, bool SPLIT>
+__device__ __forceinline__ void q_round(float* v, bool pow2_ok, float scale, int ex,
+                                        float lo_scale, uint4* ph, uint4* pl) {
+  constexpr int N = FMT == tc::kFmtTF32 ? 4 : 8;
+#pragma unroll
+  for (int z = 0; z < N; ++z) v[z] = pow2_ok ? __fmul_rn(v[z], scale) : ldexpf(v[z], -ex);
+  uint32_t w[4];
+#pragma unroll
+  for (int z = 0; z < 4; ++z) {
+    if constexpr (FMT == tc::kFmtTF32) w[z] = __float_as_uint(round_tf32(v[z]));
+    else w[z] = pack_pair<FMT>(v[2 * z], v[2 * z + 1]);
+  }
+  *ph = make_uint4(w[0], w[1], w[2], w[3]);
+  if constexpr (SPLIT) {
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      if constexpr (FMT == tc::kFmtTF32) {
+        w[z] = __float_as_uint(
+            round_tf32(__fmul_rn(__fsub_rn(v[z], __uint_as_float(w[z])), lo_scale)));
+      } else {
+        float h0, h1;
+        unpack_pair<FMT>(w[z], h0, h1);
+        w[z] = pack_pair<FMT>(__fmul_rn(__fsub_rn(v[2 * z], h0), lo_scale),
+                          __fmul_rn(__fsub_rn(v[2 * z + 1], h1), lo_scale));
+      }
+    }
+    *pl = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -164,17 +214,7 @@ __global__ void __launch_bounds__(kQ64Threads, (q64_ctas<FMT>()))
     mx = 0.0f;
 #pragma unroll
     for (int w = 0; w < kThreads / 32; ++w) mx = fmaxf(mx, s_max[w]);
-    int ex = 0;
-    if (mx > 0.0f && mx <= 3.402823466e38f) frexpf(mx, &ex);
-    // BF16 and TF32 have FP32's exponent range: the scaling only has to keep
-    // products and sums inside it, so e is rounded up to a multiple of 32
-    // (scaled maximum in [2^-33, 1)).  The roundings are those of the exact
-    // exponent for every entry above 2^-94 of the block's maximum (hi parts)
-    // and above 2^-80 (lo parts of the split modes), and
-    // the blocks of a tile mostly share one exponent sum: the multiply's runs
-    // (one accumulator pass per change of the sum) stay long.  FP16 keeps the
-    // exact exponent: its range is the constraint.
-    if constexpr (FMT != tc::kFmtF16) ex = ((ex + 31) >> 5) << 5;
+    const int ex = block_exponent<FMT>(mx);
     if (tid == 0) (isB ? img.eb : img.ea)[blk] = ex;
     // 2^-ex as a float when it is a normal number (the usual case), else ldexpf
     const bool pow2_ok = ex >= -126 && ex <= 126;
@@ -186,89 +226,13 @@ __global__ void __launch_bounds__(kQ64Threads, (q64_ctas<FMT>()))
     for (int r = 0; r < U; ++r) {
       const int u = tid + r * kThreads;
       const int row = u / PPR, k0 = (u % PPR) * PER16;
-      float hv[PER16], lv[PER16];
-#pragma unroll
-      for (int q = 0; q < PER16; ++q) {
-        const float sc = pow2_ok ? __fmul_rn(x[r][q], scale) : ldexpf(x[r][q], -ex);
-        const float h = round_op<FMT>(sc);
-        hv[q] = h;
-        if constexpr (SPLIT) lv[q] = round_op<FMT>(__fmul_rn(__fsub_rn(sc, h), lo_scale));
-      }
       uint4 ph, pl;
-      if constexpr (FMT == tc::kFmtTF32) {
-        ph = make_uint4(__float_as_uint(hv[0]), __float_as_uint(hv[1]), __float_as_uint(hv[2]),
-                        __float_as_uint(hv[3]));
-        if constexpr (SPLIT)
-          pl = make_uint4(__float_as_uint(lv[0]), __float_as_uint(lv[1]), __float_as_uint(lv[2]),
-                          __float_as_uint(lv[3]));
-      } else {
-        ph = make_uint4(pack2<FMT>(hv[0], hv[1]), pack2<FMT>(hv[2], hv[3]),
-                        pack2<FMT>(hv[4], hv[5]), pack2<FMT>(hv[6], hv[7]));
-        if constexpr (SPLIT)
-          pl = make_uint4(pack2<FMT>(lv[0], lv[1]), pack2<FMT>(lv[2], lv[3]),
-                          pack2<FMT>(lv[4], lv[5]), pack2<FMT>(lv[6], lv[7]));
-      }
+      q_round<FMT, SPLIT>(x[r], pow2_ok, scale, ex, lo_scale, &ph, &pl);
       const uint32_t off = (uint32_t)(k0 / KC) * (LEAF * 128) + tc::sw128_offset(row, (k0 % KC) / PER16);
       *reinterpret_cast<uint4*>(hi_img + off) = ph;
       if constexpr (SPLIT) *reinterpret_cast<uint4*>(lo_img + off) = pl;
     }
     __syncthreads();   // s_max and s_blk are rewritten for the next block
-  }
-}
-
-// Two entries rounded to nearest even and packed (the first in the low half).
-template <uint32_t FMT>
-__device__ __forceinline__ uint32_t pack_pair(float a, float b) {
-  if constexpr (FMT == tc::kFmtBF16) {
-    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
-    return (uint32_t)__bfloat16_as_ushort(p.x) | ((uint32_t)__bfloat16_as_ushort(p.y) << 16);
-  } else {
-    const __half2 p = __floats2half2_rn(a, b);
-    return (uint32_t)__half_as_ushort(__low2half(p)) | ((uint32_t)__half_as_ushort(__high2half(p)) << 16);
-  }
-}
-
-// The two values back (exact).
-template <uint32_t FMT>
-__device__ __forceinline__ void unpack_pair(uint32_t w, float& a, float& b) {
-  if constexpr (FMT == tc::kFmtBF16) {
-    a = __uint_as_float(w << 16);
-    b = __uint_as_float(w & 0xffff0000u);
-  } else {
-    a = __half2float(__ushort_as_half((unsigned short)(w & 0xffffu)));
-    b = __half2float(__ushort_as_half((unsigned short)(w >> 16)));
-  }
-}
-
-// One 16-byte piece of an image: v scaled by 2^-ex, rounded (hi), and in split modes
-// the exact residual scaled by 2^lo shift, rounded (lo).
-template <uint32_t FMT, bool SPLIT>
-__device__ __forceinline__ void q_round(float* v, bool pow2_ok, float scale, int ex,
-                                        float lo_scale, uint4* ph, uint4* pl) {
-  constexpr int N = FMT == tc::kFmtTF32 ? 4 : 8;
-#pragma unroll
-  for (int z = 0; z < N; ++z) v[z] = pow2_ok ? __fmul_rn(v[z], scale) : ldexpf(v[z], -ex);
-  uint32_t w[4];
-#pragma unroll
-  for (int z = 0; z < 4; ++z) {
-    if constexpr (FMT == tc::kFmtTF32) w[z] = __float_as_uint(round_tf32(v[z]));
-    else w[z] = pack_pair<FMT>(v[2 * z], v[2 * z + 1]);
-  }
-  *ph = make_uint4(w[0], w[1], w[2], w[3]);
-  if constexpr (SPLIT) {
-#pragma unroll
-    for (int z = 0; z < 4; ++z) {
-      if constexpr (FMT == tc::kFmtTF32) {
-        w[z] = __float_as_uint(
-            round_tf32(__fmul_rn(__fsub_rn(v[z], __uint_as_float(w[z])), lo_scale)));
-      } else {
-        float h0, h1;
-        unpack_pair<FMT>(w[z], h0, h1);
-        w[z] = pack_pair<FMT>(__fmul_rn(__fsub_rn(v[2 * z], h0), lo_scale),
-                          __fmul_rn(__fsub_rn(v[2 * z + 1], h1), lo_scale));
-      }
-    }
-    *pl = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -330,11 +294,6 @@ __device__ __forceinline__ QBlock q_block(const InstRef& R, uint32_t ent) {
   return q;
 }
 
-__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src),
-               "r"(bytes)
-               : "memory");
-}
 // Distance of row r of a block from the 16-byte boundary its staged row starts at.
 __device__ __forceinline__ int q_shift(const QBlock& q, int r) {
   return (int)(((uint32_t)(reinterpret_cast<uintptr_t>(q.src) >> 2) + (uint32_t)r * (uint32_t)q.ld) & 3u);
@@ -353,14 +312,14 @@ __device__ __forceinline__ void q_fetch(float* dst, const QBlock& q) {
 #pragma unroll
     for (int l = 0; l < LEAF / kStep; ++l, src += kStep * q.ld) {
       const int b = r0 + l * kStep < q.rows ? bytes : 0;
-      copy16(dst + (r0 + l * kStep) * LD + c, b ? src : q.src, b);
+      tc::copy16(dst + (r0 + l * kStep) * LD + c, b ? src : q.src, b);
     }
   } else {
     // piece c / 4 of a row, and one more per row for the entries the shift moves out
     auto piece = [&](int r, const float* at, float* to) {
       const float* p = reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(at) & ~(uintptr_t)15);
       const int64_t left = q.end - p;
-      if (r < q.rows && left > 0) copy16(to, p, left >= 4 ? 16 : (int)left * 4);
+      if (r < q.rows && left > 0) tc::copy16(to, p, left >= 4 ? 16 : (int)left * 4);
     };
 #pragma unroll
     for (int l = 0; l < LEAF / kStep; ++l, src += kStep * q.ld)
@@ -487,17 +446,7 @@ __global__ void __launch_bounds__(QCfg<FMT, LEAF, SPLIT>::kThreads, (QCfg<FMT, L
     mx = s_max[par][lane < C::kWarps ? lane : 0];
     mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
     par ^= 1u;
-    int ex = 0;
-    if (mx > 0.0f && mx <= 3.402823466e38f) frexpf(mx, &ex);
-    // BF16 and TF32 have FP32's exponent range: the scaling only has to keep
-    // products and sums inside it, so e is rounded up to a multiple of 32
-    // (scaled maximum in [2^-33, 1)).  The roundings are those of the exact
-    // exponent for every entry above 2^-94 of the block's maximum (hi parts)
-    // and above 2^-80 (lo parts of the split modes), and
-    // the blocks of a tile mostly share one exponent sum: the multiply's runs
-    // (one accumulator pass per change of the sum) stay long.  FP16 keeps the
-    // exact exponent: its range is the constraint.
-    if constexpr (FMT != tc::kFmtF16) ex = ((ex + 31) >> 5) << 5;
+    const int ex = block_exponent<FMT>(mx);
     if (tid == 0) (q.isB ? img.eb : img.ea)[q.blk] = ex;
     // 2^-ex as a float when it is a normal number (the usual case), else ldexpf
     const bool pow2_ok = ex >= -126 && ex <= 126;

@@ -101,6 +101,18 @@ __device__ __forceinline__ void bulk_wait_read0() {
 __device__ __forceinline__ void bulk_wait0() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
+// Asynchronous copies of 16 (4) bytes, `bytes` of them from src and the rest zeros (this
+// thread's groups: cp.async.commit_group, cp.async.wait_group).
+__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes = 16) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes = 4) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
 // The cluster address of this CTA's shared-memory object in CTA `rank`.
 __device__ __forceinline__ uint32_t peer_addr(const void* p, int rank) {
   uint32_t a;
