@@ -404,7 +404,7 @@ __device__ __forceinline__ void load_weights(Net& n, const float* __restrict__ W
 // in 64 steps).  With the flag up, all weights and losses end as NaN, and m and v keep what they held.  WITHHOLD (self-test):
 // nothing is sent, so the first wait runs out after limit_ns; elapsed receives the longest
 // time a thread of the cluster waited.
-// 64 steps of 256 samples: 518 us, 8 us a step.  Of a step's 16 thousand cycles (clock
+// 64 steps of 256 samples: 516 us, 8 us a step.  Of a step's 16 thousand cycles (clock
 // stamps in a copy of the kernel) each
 // layer takes 1.6 to 2.0 (shared memory and latency), the outer products 2.3 (shared
 // memory), Adam 1.2, the two exchanges 5 (35 KB each way per CTA at the ~20 bytes per
