@@ -45,12 +45,15 @@ constexpr int64_t own_zero_bytes(int leaf, bool beside) {
 
 // Up to this many non-empty tiles per SM, four warps share a tile, in three groups with a
 // longer ring: with one or two warps per tile the other schedulers of an SM would idle
-// through its list.  One tile per SM, lists of 256 blocks at leaf 32: 325 -> 221 us (256
-// threads per tile, one group: 298), of 128 at leaf 64: 451 -> 310 (417); 32 tiles of 1024
-// blocks at leaf 32: 954 -> 532 (848), 8 of 256 at leaf 64: 895 -> 614 (822).  Two per SM
-// 254 -> 200 and 499 -> 470; three 263 -> 287 at leaf 32, and at leaf 64 757 -> 629 with
-// equal lists, but the selection of tau (uneven ones) 800 -> 812: hence the limit.  The
-// sums are in the same order in both forms.
+// through its list.  One tile per SM, lists of 256 blocks at leaf 32: 325 -> 217 us (256
+// threads per tile, one group: 298), of 128 at leaf 64: 451 -> 301 (417); 32 tiles of 1024
+// blocks at leaf 32: 954 -> 523 (848), 8 of 256 at leaf 64: 895 -> 590 (822).  Two per SM
+// 254 -> 192 and 499 -> 496; three 263 -> 287 at leaf 32, and at leaf 64 757 -> 629 with
+// equal lists, but the selection of tau (uneven ones) 800 -> 812: hence the limit.  With
+// many empty tiles to write beside them the idle warps are not idle: only up to one tile per
+// SM then (two per SM, 23 empty ones each, short lists at leaf 32: product 31.1 -> 33.5 us; one
+// per SM at leaf 64, five empty ones: 39.2 -> 35.2).  The sums are in the same order in
+// both forms.
 constexpr int kWideTiles = 2;
 
 // How a CTA is cut into groups of warps, a group's tile into warps and a warp's part
@@ -132,10 +135,9 @@ __device__ __forceinline__ void tile_sync(int group) {
     asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(T::kThreads) : "memory");
 }
 
-// An empty tile of an instance with beta = 0: zeros, and the tile's norm.
-template <class T>
+// An empty tile of an instance with beta = 0: zeros, and the tile's norm; by kThreads threads.
+template <int LEAF, int kThreads>
 __device__ __forceinline__ void zero_tile(const Inst& in, int64_t t, int tid) {
-  constexpr int LEAF = T::LEAF, kThreads = T::kThreads;
   const int i = (int)(t / in.bn), j = (int)(t - (int64_t)i * in.bn);
   const int64_t r0 = (int64_t)i * LEAF, c0 = (int64_t)j * LEAF;
   const int rows = (int)min((int64_t)LEAF, in.m - r0), cols = (int)min((int64_t)LEAF, in.n - c0);
@@ -183,7 +185,7 @@ __device__ __forceinline__ void multiply_tiles(const InstRef& R, const PlanBuffe
     const int g = Bf.order[w];
     const Inst& in = R.at(inst_of(R, Bf, g));
     if (w >= ne) {
-      zero_tile<T>(in, g - in.tile0, tid);
+      zero_tile<LEAF, T::kThreads>(in, g - in.tile0, tid);
       tile_sync<T>(group);   // s_next is rewritten next
       continue;
     }
@@ -351,12 +353,13 @@ __device__ __forceinline__ void multiply_tiles(const InstRef& R, const PlanBuffe
   for (int64_t w = ne + blockIdx.x * T::kGroups + group; w < all; w += (int64_t)gridDim.x * T::kGroups) {
     const int g = Bf.order[w];
     const Inst& in = R.at(inst_of(R, Bf, g));
-    zero_tile<T>(in, g - in.tile0, tid);
+    zero_tile<LEAF, T::kThreads>(in, g - in.tile0, tid);
   }
 }
 
 // Few tiles.  A function of its own: with both forms in the kernel's body the other one
-// fetches its first instructions from further on, 1 to 3 us.
+// fetches its first instructions from further on, 1 to 3 us.  The empty tiles are taken by
+// single warps (by the groups of four 1 to 2 us more with a dozen of them per SM).
 template <int LEAF>
 __device__ __noinline__ void multiply_wide(const InstRef& R, const PlanBuffers& Bf, int dynamic,
                                            int zeros) {
@@ -364,11 +367,23 @@ __device__ __noinline__ void multiply_wide(const InstRef& R, const PlanBuffers& 
   static_assert(T::kCtaThreads == SimtTile<LEAF, false>::kCtaThreads &&
                     T::kCtaSmem == SimtTile<LEAF, false>::kCtaSmem,
                 "one launch serves both forms");
-  __shared__ int s_taken, s_next[T::kGroups];
+  __shared__ int s_taken, s_zeroed, s_next[T::kGroups];
   __shared__ SumSq s_norm[T::kGroups * T::kWarps];
-  if (threadIdx.x == 0) s_taken = 0;
+  if (threadIdx.x == 0) s_taken = s_zeroed = 0;
   __syncthreads();
-  multiply_tiles<T>(R, Bf, Bf.bdev->nonempty, dynamic, zeros, &s_taken, s_next, s_norm, threadIdx.x);
+  const int ne = Bf.bdev->nonempty, lane = threadIdx.x & 31;
+  multiply_tiles<T>(R, Bf, ne, dynamic, 0, &s_taken, s_next, s_norm, threadIdx.x);
+  if (!zeros) return;
+  for (;;) {
+    int z = 0;
+    if (lane == 0) z = atomicAdd(&s_zeroed, 1);
+    z = __shfl_sync(0xffffffffu, z, 0);
+    const int64_t w = ne + blockIdx.x + (int64_t)z * gridDim.x;
+    if (w >= Bf.tiles) return;
+    const int g = Bf.order[w];
+    const Inst& in = R.at(inst_of(R, Bf, g));
+    zero_tile<LEAF, 32>(in, g - in.tile0, lane);
+  }
 }
 
 template <int LEAF>
@@ -384,7 +399,8 @@ __global__ void __launch_bounds__(SimtTile<LEAF, false>::kCtaThreads, 1)
   pdl_wait();
   const int ne = Bf.bdev->nonempty;
   if constexpr (LEAF < 128) {
-    if (ne <= kWideTiles * (int)gridDim.x) {
+    const int64_t sms = gridDim.x, empty = zeros ? Bf.tiles - ne : 0;
+    if (ne <= sms || (ne <= kWideTiles * sms && empty <= kWideTiles * sms)) {
       multiply_wide<LEAF>(R, Bf, dynamic, zeros);
       return;
     }

@@ -49,3 +49,23 @@ def test_few_and_many_tiles_give_the_same_bits(rows, cols, k, alpha, beta, leaf,
     # the norms: sums of the same squares, merged in another order (FP64 grade)
     ok = (n_many - nC.repeat(copies, 1)).abs() <= 1e-12 * nC.repeat(copies, 1)
     assert bool(ok.all())
+
+
+@pytest.mark.parametrize("schedule", ["static", "dynamic"])
+@pytest.mark.parametrize("leaf", [32, 64])
+@pytest.mark.parametrize("cut", [0, 3])
+def test_few_tiles_among_many_empty_ones(cut, leaf, schedule):
+    """Three block rows of forty hold anything: 75 tiles of 1000, the others are written as zeros."""
+    m, n, k = 40 * leaf - cut, 25 * leaf - cut, 200
+    g = torch.Generator(device="cuda")
+    g.manual_seed(leaf + cut)
+    A = torch.zeros(m, k, device="cuda")
+    for i in (0, 17, 39):
+        A[i * leaf:(i + 1) * leaf] = torch.randn(A[i * leaf:(i + 1) * leaf].shape, generator=g, device="cuda")
+    B = torch.randn(k, n, generator=g, device="cuda")
+    C, nC = _product(A, B, torch.full((m, n), float("nan"), device="cuda"), leaf, schedule, 1.0, 0.0)
+    bound = k * 2.0 ** -24 * 1.01 * (A.double().abs() @ B.double().abs())     # one FMA chain per entry
+    assert bool(((C.double() - A.double() @ B.double()).abs() <= bound).all())
+    empty = torch.ones(40, dtype=torch.bool)
+    empty[[0, 17, 39]] = False
+    assert bool((nC[empty.cuda()] == 0.0).all()) and bool((nC[~empty.cuda()] > 0.0).all())
